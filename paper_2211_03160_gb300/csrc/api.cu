@@ -652,6 +652,30 @@ extern "C" int tlbm_create(tlbm_t* out, int nx, int ny, int nz, int lattice, dou
         t.g0c = qp * rest;
     }
 
+    {
+        // FP64 constants of the two-relaxation-time collision (KParams::td)
+        auto& t = kp.td;
+        t.hsp = 0.5 * (1.0 - kp.sp);
+        t.hsm = 0.5 * (1.0 - kp.sm);
+        t.osp = 1.0 - kp.sp;
+        t.sp = kp.sp;
+        t.k15 = -1.5 * kp.sp;
+        t.k6 = -6.0 * kp.shp;
+        t.b1 = 4.5 * kp.sp;
+        t.b2 = 18.0 * kp.shp;
+        t.a1 = 3.0 * kp.sm;
+        t.a2 = 6.0 * kp.shm;
+        t.hgb = 0.5 * kp.gbeta;
+        for (int a = 0; a < 3; ++a) t.hb[a] = 0.5 * kp.body[a];
+        const double wT = 0.5 * kp.omega;
+        t.hqp = 0.5 * (1.0 - kp.qp);
+        t.hqm = 0.5 * (1.0 - kp.qm);
+        t.oqp = 1.0 - kp.qp;
+        t.qpwT = kp.qp * wT;
+        t.hq = 0.5 * kp.qm;
+        t.g0c = kp.qp * (1.0 - (h->qg - 1) * wT);
+    }
+
     if ((long long)(h->qf + h->qg) * kp.L.plane + kp.L.P >= (1ll << 31)) {
         delete h;
         return fail(nullptr, TLBM_ERR_ARG, "cell too large: a population set must hold fewer than 2^31 elements");

@@ -95,6 +95,17 @@ struct KParams {
         float m3shp, r1, r3, c1, c2, omsp, w0s, was, wbs, f9a, f9b, f3a, f3b;
         float t1, t2, qpwT, hqm, omqp, g0c;
     } tf;
+    // FP64 constants of the two-relaxation-time collision (collide_trt_d): with
+    // h_a = body_a / 2 (+ gbeta T / 2 on the gravity axis),
+    //   hsp = (1 - sp)/2, hsm = (1 - sm)/2, osp = 1 - sp, sp, k15 = -1.5 sp,
+    //   k6 = -6 shp, b1 = 4.5 sp, b2 = 18 shp, a1 = 3 sm, a2 = 6 shm,
+    //   hgb = gbeta/2, hb = body/2; thermal, with wT = omega/2:
+    //   hqp = (1 - qp)/2, hqm = (1 - qm)/2, oqp = 1 - qp, qpwT = qp wT,
+    //   hq = qm/2, g0c = qp (1 - (Q_g - 1) wT)
+    struct {
+        double hsp, hsm, osp, sp, k15, k6, b1, b2, a1, a2, hgb, hb[3];
+        double hqp, hqm, oqp, qpwT, hq, g0c;
+    } td;
 #ifdef TLBM_DEBUG_BOUNDS
     // the population buffers of the handle and the violation counter
     const char* dbg_lo;
@@ -273,12 +284,6 @@ __device__ __forceinline__ uint32_t step_salt(uint32_t t) { return t * 0x9E3779B
 // parameter accessors in the compute precision
 template <class C> struct PV;
 template <> struct PV<double> {
-    __device__ static double sp(const KParams& p) { return p.sp; }
-    __device__ static double sm(const KParams& p) { return p.sm; }
-    __device__ static double shp(const KParams& p) { return p.shp; }
-    __device__ static double shm(const KParams& p) { return p.shm; }
-    __device__ static double qp(const KParams& p) { return p.qp; }
-    __device__ static double qm(const KParams& p) { return p.qm; }
     __device__ static double S(const KParams& p, int k) { return p.S[k]; }
     __device__ static double Sh(const KParams& p, int k) { return p.Sh[k]; }
     __device__ static double Q(const KParams& p, int k) { return p.Q[k]; }
@@ -335,9 +340,10 @@ __device__ __forceinline__ S enc_g(C g, C scale) {
     else return from_c<S>(g);
 }
 // the same as stored by a time step (stochastic rounding for 16-bit storage)
-template <class LF, class S, class C>
+template <class LF, class S, class C, bool RAW = false>
 __device__ __forceinline__ S enc_f_step(C d, int i, C scale, uint32_t salt) {
     if constexpr (Storage<S>::offset) return from_c_step<S>(d * scale, salt);
+    else if constexpr (RAW) return from_c_step<S>(d, salt);
     else return from_c_step<S>(weight<LF, C>(i) + d, salt);
 }
 template <class S, class C>
@@ -357,10 +363,6 @@ template <> struct ScaleOf<double> {
 };
 
 // ------------------------------------------------------------------ collision
-
-// 1/x, correctly rounded in both precisions
-__device__ __forceinline__ float recip(float x) { return __frcp_rn(x); }
-__device__ __forceinline__ double recip(double x) { return 1.0 / x; }
 
 // Macroscopic moments of one node from deviations (§2.2):
 // rho = 1 + sum d, T = sum g, F = rho (g beta T ghat + a), u = (sum e f + F/2)/rho.
@@ -483,88 +485,148 @@ template <> struct Lat<3> { using F = D3Q19; using G = D3Q7; };
 // and the rest population as d_0+ = (1 - sp) d_0 + w_0 K0.  The thermal pairs:
 //   g_i+ = t1 g_i + t2 g_ibar + qp wT T + (qm/2) e.u T  (and - for ibar),
 //   t1 = 1 - (qp + qm)/2, t2 = (qm - qp)/2, wT = omega/2;  g_0+ = (1 - qp) g_0 + qp (1 - (q-1) wT) T.
-// SCALED: the inputs and outputs are the stored values d_i * scale and
-// g_i * scale (offset storage); every term is linear in them except through the
+// In FP32 the inputs and outputs are the stored values d_i * scale and g_i *
+// scale (offset storage): every term is linear in them except through the
 // node's rho, u and T, which are formed unscaled.
-template <int DIM, class C, bool SCALED>
-__device__ __forceinline__ void collide_trt(C (&d)[Lat<DIM>::F::Q], C (&g)[Lat<DIM>::G::Q], const KParams& p) {
+
+// FP64: arithmetic that the compiler neither contracts nor reorders, so that a
+// node's result does not depend on the kernel or translation unit it is in.
+__device__ __forceinline__ double dadd(double a, double b) { return __dadd_rn(a, b); }
+__device__ __forceinline__ double dsub(double a, double b) { return __dsub_rn(a, b); }
+__device__ __forceinline__ double dmul(double a, double b) { return __dmul_rn(a, b); }
+__device__ __forceinline__ double dfma(double a, double b, double c) { return __fma_rn(a, b, c); }
+
+// 1/x from an FP32 estimate y (relative error below 2^-22) and the geometric
+// series 1/x = y / (1 - e), e = 1 - x y: y (1 + e + e^2) is off by e^3 < 2^-66,
+// so its error is that of the last rounding.  Three FP64 instructions.
+__device__ __forceinline__ double drcp(double x) {
+    float y0;
+    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(y0) : "f"((float)x));
+    const double y = (double)y0;
+    const double e = dfma(-x, y, 1.0);
+    return dfma(y, dfma(e, e, e), y);
+}
+
+// First population of a set that moves by +1 along axis a only.
+template <class L>
+__host__ __device__ constexpr int axis_pop(int a) {
+    for (int i = 1; i < L::Q; ++i)
+        if (L::e(i, a) == 1 && L::e(i, (a + 1) % 3) == 0 && L::e(i, (a + 2) % 3) == 0) return i;
+    return 0;
+}
+
+// The FP64 collision, on the stored f_i themselves (FP64 storage keeps f_i, not
+// the deviation).  GB300 runs FP64 at 1/64 of the FP32 rate, so this form is
+// written for the fewest FP64 instructions, each multiply-add one instruction:
+// with s = d_i + d_ibar, a = d_i - d_ibar = f_i - f_ibar and h = F / (2 rho),
+//   u = j / rho + h,   K0 = sp drho - rho (1.5 sp u^2 + 6 shp u.h),
+//   B = 4.5 sp u + 18 shp h,   A = 3 sm u + 6 shm h,
+//   S = (1 - sp)/2 s + w_i K0 + w_i rho (e.u)(e.B),   D = (1 - sm)/2 a + w_i rho e.A,
+//   f_i+ = w_i + (S + D),   f_ibar+ = w_i + (S - D).
+// Everything but the last addition is of the deviations' size, so a stored
+// value takes one rounding at its own ulp.  (Folding the weights into S as well
+// saves another 15 % of the instructions, but then the error of u against an
+// exact evaluation grows from 1.2e-15 to 4e-15 after 16 steps at 4097^2.)
+// 114 FP64 instructions per node in 2D and 216 in 3D, against 217 and 488 of the
+// uncontracted pairwise form (K0, Ks and Ka above evaluated term by term).  The
+// FP64 pipe bounds both (530 G instructions/s): 4097^2 6.63 -> 3.69 ms per step,
+// 193^3 6.29 -> 3.43 ms.
+template <int DIM>
+__device__ __forceinline__ void collide_trt_d(double (&f)[Lat<DIM>::F::Q], double (&g)[Lat<DIM>::G::Q],
+                                              const KParams& p) {
     using LF = typename Lat<DIM>::F;
     using LG = typename Lat<DIM>::G;
-    using P = PV<C>;
-    C drs = C(0), jx = C(0), jy = C(0), jz = C(0), Ts = C(0);
+    const auto& c = p.td;
+    // pairs: f[i] <- s, f[ibar] <- a (i the smaller index)
+    const double d0 = dsub(f[0], weight<LF, double>(0));
+    double drho = d0;
     static_for<LF::Q>([&](auto ii) {
-        constexpr int i = decltype(ii)::value;
-        drs += d[i];
-        if constexpr (LF::e(i, 0) == 1) jx += d[i];
-        if constexpr (LF::e(i, 0) == -1) jx -= d[i];
-        if constexpr (LF::e(i, 1) == 1) jy += d[i];
-        if constexpr (LF::e(i, 1) == -1) jy -= d[i];
-        if constexpr (LF::e(i, 2) == 1) jz += d[i];
-        if constexpr (LF::e(i, 2) == -1) jz -= d[i];
-    });
-    static_for<LG::Q>([&](auto ii) { Ts += g[decltype(ii)::value]; });
-    C sc = C(1), inv = C(1);
-    if constexpr (SCALED) {
-        sc = ScaleOf<C>::s(p);
-        inv = ScaleOf<C>::inv(p);
-    }
-    const C drho = SCALED ? drs * inv : drs;
-    const C T = SCALED ? Ts * inv : Ts;
-    const C rho = C(1) + drho;
-    const C buoy = P::gbeta(p) * T;
-    const C Fx = rho * P::body(p, 0);
-    const C Fy = rho * (DIM == 2 ? buoy + P::body(p, 1) : P::body(p, 1));
-    const C Fz = DIM == 3 ? rho * (buoy + P::body(p, 2)) : C(0);
-    const C ir = recip(rho);
-    const C hx = C(0.5) * Fx, hy = C(0.5) * Fy, hz = C(0.5) * Fz;
-    const C ux = (SCALED ? fma(jx, inv, hx) : jx + hx) * ir;
-    const C uy = (SCALED ? fma(jy, inv, hy) : jy + hy) * ir;
-    const C uz = DIM == 3 ? (SCALED ? fma(jz, inv, hz) : jz + hz) * ir : C(0);
-    const C sp = P::sp(p), sm = P::sm(p), shp = P::shp(p), shm = P::shm(p);
-    const C uu15 = C(1.5) * (ux * ux + uy * uy + uz * uz);
-    const C uF3 = C(3) * (ux * Fx + uy * Fy + uz * Fz);
-    const C K0 = sp * (drho - rho * uu15) - shp * uF3;
-    const C R1 = C(4.5) * sp * rho, R2 = C(9) * shp;
-    const C R3 = C(3) * sm * rho, R4 = C(3) * shm;
-    const C c1 = C(1) - C(0.5) * (sp + sm), c2 = C(0.5) * (sm - sp);
-    {
-        constexpr C w0 = weight<LF, C>(0);
-        d[0] = (C(1) - sp) * d[0] + (w0 * sc) * K0;
-    }
-    static_for<LF::Q>([&](auto ii) {
-        constexpr int i = decltype(ii)::value;
-        constexpr int o = LF::opp(i);
+        constexpr int i = decltype(ii)::value, o = LF::opp(i);
         if constexpr (i != 0 && i < o) {
-            constexpr int ex = LF::e(i, 0), ey = LF::e(i, 1), ez = LF::e(i, 2);
-            const C ws = weight<LF, C>(i) * sc;
-            C eu = C(0), eF = C(0);
-            if constexpr (ex != 0) { eu += C(ex) * ux; eF += C(ex) * Fx; }
-            if constexpr (ey != 0) { eu += C(ey) * uy; eF += C(ey) * Fy; }
-            if constexpr (ez != 0) { eu += C(ez) * uz; eF += C(ez) * Fz; }
-            const C Ks = ws * (K0 + eu * (R1 * eu + R2 * eF));
-            const C Ka = ws * (R3 * eu + R4 * eF);
-            const C di = d[i], dob = d[o];
-            d[i] = c1 * di + c2 * dob + (Ks + Ka);
-            d[o] = c1 * dob + c2 * di + (Ks - Ka);
+            const double a = dsub(f[i], f[o]), s = dadd(dsub(f[i], 2.0 * weight<LF, double>(i)), f[o]);
+            f[i] = s;
+            f[o] = a;
+            drho = dadd(drho, s);
         }
     });
-    // thermal
-    const C qp = P::qp(p), qm = P::qm(p);
-    const C wT = C(0.5) * P::omega(p);
-    const C t1 = C(1) - C(0.5) * (qp + qm), t2 = C(0.5) * (qm - qp);
-    const C Ks_T = qp * wT * Ts;        // scaled like g
-    const C ka_T = C(0.5) * qm * Ts;    // times e.u
-    g[0] = (C(1) - qp) * g[0] + qp * (C(1) - C(LG::Q - 1) * wT) * Ts;
+    double j[3] = {0.0, 0.0, 0.0};
+    static_for<DIM>([&](auto aa) {
+        constexpr int ax = decltype(aa)::value, i0 = axis_pop<LF>(ax);
+        static_assert(i0 < LF::opp(i0), "the axis pair starts with its positive direction");
+        j[ax] = f[LF::opp(i0)];
+        static_for<LF::Q>([&](auto ii) {
+            constexpr int i = decltype(ii)::value, o = LF::opp(i);
+            if constexpr (i != 0 && i < o && i != i0) {
+                if constexpr (LF::e(i, ax) == 1) j[ax] = dadd(j[ax], f[o]);
+                if constexpr (LF::e(i, ax) == -1) j[ax] = dsub(j[ax], f[o]);
+            }
+        });
+    });
+    double T = g[0];
     static_for<LG::Q>([&](auto ii) {
-        constexpr int i = decltype(ii)::value;
-        constexpr int o = LG::opp(i);
+        constexpr int i = decltype(ii)::value, o = LG::opp(i);
         if constexpr (i != 0 && i < o) {
-            constexpr int ex = LG::e(i, 0), ey = LG::e(i, 1), ez = LG::e(i, 2);
-            const C eu = ex != 0 ? C(ex) * ux : (ey != 0 ? C(ey) * uy : C(ez) * uz);
-            const C Ka = ka_T * eu;
-            const C gi = g[i], go = g[o];
-            g[i] = t1 * gi + t2 * go + (Ks_T + Ka);
-            g[o] = t1 * go + t2 * gi + (Ks_T - Ka);
+            const double s = dadd(g[i], g[o]), a = dsub(g[i], g[o]);
+            g[i] = s;
+            g[o] = a;
+            T = dadd(T, s);
+        }
+    });
+    const double rho = dadd(1.0, drho);
+    const double ir = drcp(rho);
+    double u[3], B[3], A[3], uu = 0.0, uh = 0.0;
+#pragma unroll
+    for (int ax = 0; ax < DIM; ++ax) {
+        const double h = ax == DIM - 1 ? dfma(c.hgb, T, c.hb[ax]) : c.hb[ax];
+        u[ax] = dfma(j[ax], ir, h);
+        uu = ax == 0 ? dmul(u[0], u[0]) : dfma(u[ax], u[ax], uu);
+        uh = ax == 0 ? dmul(u[0], h) : dfma(u[ax], h, uh);
+        B[ax] = dfma(c.b1, u[ax], dmul(c.b2, h));
+        A[ax] = dfma(c.a1, u[ax], dmul(c.a2, h));
+    }
+    const double K0 = dfma(rho, dfma(c.k6, uh, dmul(c.k15, uu)), dmul(c.sp, drho));
+    constexpr double w0 = weight<LF, double>(0), wa = weight<LF, double>(1), wb = weight<LF, double>(LF::Q - 1);
+    const double ra = dmul(wa, rho), rb = dmul(wb, rho), Ka = dmul(wa, K0), Kb = dmul(wb, K0);
+    f[0] = dadd(w0, dfma(c.osp, d0, dmul(w0, K0)));
+    static_for<LF::Q>([&](auto ii) {
+        constexpr int i = decltype(ii)::value, o = LF::opp(i);
+        if constexpr (i != 0 && i < o) {
+            constexpr int ex = LF::e(i, 0), ey = LF::e(i, 1), ez = LF::e(i, 2);
+            constexpr int sg = ex != 0 ? ex : (ey != 0 ? ey : ez);  // sign of the pair's leading component
+            constexpr bool cls_a = LF::w36(i) == LF::w36(1);
+            static_assert(cls_a || LF::w36(i) == LF::w36(LF::Q - 1), "two weight classes");
+            constexpr double w = cls_a ? wa : wb;
+            double eu, eB, eA;
+            if constexpr (cls_a) {
+                constexpr int ax = ex != 0 ? 0 : (ey != 0 ? 1 : 2);
+                eu = u[ax];
+                eB = B[ax];
+                eA = A[ax];
+            } else {
+                constexpr int p0 = ex != 0 ? 0 : 1, p1 = ez != 0 ? 2 : 1;
+                constexpr bool same = LF::e(i, p0) == LF::e(i, p1);
+                eu = same ? dadd(u[p0], u[p1]) : dsub(u[p0], u[p1]);
+                eB = same ? dadd(B[p0], B[p1]) : dsub(B[p0], B[p1]);
+                eA = same ? dadd(A[p0], A[p1]) : dsub(A[p0], A[p1]);
+            }
+            const double r = cls_a ? ra : rb;
+            const double S = dfma(r, dmul(eu, eB), dfma(c.hsp, f[i], cls_a ? Ka : Kb));
+            // eA carries the leading component's sign: taken out here
+            const double D = dfma(sg > 0 ? r : -r, eA, dmul(c.hsm, f[o]));
+            f[i] = dadd(w, dadd(S, D));
+            f[o] = dadd(w, dsub(S, D));
+        }
+    });
+    const double KT = dmul(c.qpwT, T), kT = dmul(c.hq, T);
+    g[0] = dfma(c.oqp, g[0], dmul(c.g0c, T));
+    static_for<LG::Q>([&](auto ii) {
+        constexpr int i = decltype(ii)::value, o = LG::opp(i);
+        if constexpr (i != 0 && i < o) {
+            constexpr int ax = LG::e(i, 0) != 0 ? 0 : (LG::e(i, 1) != 0 ? 1 : 2);
+            static_assert(LG::e(i, ax) == 1, "the pair starts with its positive direction");
+            const double S = dfma(c.hqp, g[i], KT), D = dfma(kT, u[ax], dmul(c.hqm, g[o]));
+            g[i] = dadd(S, D);
+            g[o] = dsub(S, D);
         }
     });
 }
@@ -604,7 +666,7 @@ __device__ __forceinline__ V vdot_unit(V x, V y, V z) {
     return r;
 }
 
-// The collision of collide_trt above in FP32, over V = float or float2.  Per
+// The pairwise form above in FP32, over V = float or float2.  Per
 // pair (i, ibar) the direction with a leading +1 component, e*, carries the
 // antisymmetric part: with sg = +1 if e_i = e*, -1 otherwise,
 //   d_i+ = c1 d_i + c2 d_ibar + Ks + sg Ka*,  d_ibar+ = c1 d_ibar + c2 d_i + Ks - sg Ka*,
@@ -719,7 +781,7 @@ __device__ __forceinline__ void collide_trt_v(V (&d)[Lat<DIM>::F::Q], V (&g)[Lat
 template <int DIM, bool TRT, class C, bool SCALED = false, bool HC = false>
 __device__ __forceinline__ void collide(C (&d)[Lat<DIM>::F::Q], C (&g)[Lat<DIM>::G::Q], const KParams& p) {
     if constexpr (TRT && std::is_same<C, float>::value) collide_trt_v<DIM, float, SCALED, HC>(d, g, p);
-    else if constexpr (TRT) collide_trt<DIM, C, SCALED>(d, g, p);
+    else if constexpr (TRT) collide_trt_d<DIM>(d, g, p);
     else if constexpr (DIM == 2) collide_2d<C>(d, g, p);
     else collide_3d<C>(d, g, p);
 }
@@ -913,7 +975,9 @@ constexpr int PULL = 0, AA_EVEN = 1, AA_ODD = 2;
 // the ghost slot the following AA_ODD half reads it from.  AA_ODD: into the slot
 // the next AA_EVEN half reads (the node's own slot of the opposite direction
 // for a wall, the image's own slot for a periodic face).
-template <class LS, bool THERMAL, int i, class S, class C, int MODE = PULL>
+// RAW: flow values are f_i as stored (FP64 with the two-relaxation-time
+// collision) rather than deviations.
+template <class LS, bool THERMAL, int i, class S, class C, int MODE, bool RAW>
 __device__ __forceinline__ void ghost_write(S* __restrict__ base, const KParams& p, int x, int y, int z, C val,
                                             C scale, uint32_t salt) {
     constexpr int ex = LS::e(i, 0), ey = LS::e(i, 1), ez = LS::e(i, 2);
@@ -945,7 +1009,7 @@ __device__ __forceinline__ void ghost_write(S* __restrict__ base, const KParams&
         constexpr int plane = MODE == AA_EVEN ? i : o;
         const long long s = MODE == AA_ODD ? L.slot(x, y, z) : L.slot(dx, dy, dz);
         if constexpr (THERMAL) *TLBM_DBG(p, (base + ((long long)plane * L.plane + s)), 0, 1) = enc_g_step<S, C>(out, scale, salt);
-        else *TLBM_DBG(p, (base + ((long long)plane * L.plane + s)), 0, 1) = enc_f_step<LS, S, C>(out, plane, scale, salt);
+        else *TLBM_DBG(p, (base + ((long long)plane * L.plane + s)), 0, 1) = enc_f_step<LS, S, C, RAW>(out, plane, scale, salt);
     } else {
         // periodic: the value reaches the image node w = wrap(x + e_i) as f_i;
         // written by PULL: slot (w - e_i) of plane i; by AA_EVEN: slot (w - e_i)
@@ -957,17 +1021,19 @@ __device__ __forceinline__ void ghost_write(S* __restrict__ base, const KParams&
         constexpr int plane = MODE == AA_EVEN ? o : i;
         const long long s = MODE == AA_ODD ? L.slot(wx, wy, wz) : L.slot(wx - ex, wy - ey, wz - ez);
         if constexpr (THERMAL) *TLBM_DBG(p, (base + ((long long)plane * L.plane + s)), 0, 1) = enc_g_step<S, C>(val, scale, salt);
-        else *TLBM_DBG(p, (base + ((long long)plane * L.plane + s)), 0, 1) = enc_f_step<LS, S, C>(val, plane, scale, salt);
+        else *TLBM_DBG(p, (base + ((long long)plane * L.plane + s)), 0, 1) = enc_f_step<LS, S, C, RAW>(val, plane, scale, salt);
     }
 }
 
 // ------------------------------------------------------------------ step kernel
 
 // decode a raw stored value (already converted to C) into the flow deviation;
-// with KS (keep scaled) offset storage stays in its scaled domain
+// with KS (keep stored; the two-relaxation-time collision) it stays as it is
+// stored: scaled deviations in offset storage, f_i itself in FP64
 template <class LF, class S, class C, bool KS>
 __device__ __forceinline__ C raw_to_dev_k(C raw, int i, C inv_scale) {
-    if constexpr (Storage<S>::offset) return KS ? raw : raw * inv_scale;
+    if constexpr (KS) return raw;
+    else if constexpr (Storage<S>::offset) return raw * inv_scale;
     else return raw - weight<LF, C>(i);
 }
 template <class S, class C, bool KS>
@@ -978,7 +1044,7 @@ __device__ __forceinline__ C raw_to_g_k(C raw, C inv_scale) {
 template <class LF, class S, class C, bool KS>
 __device__ __forceinline__ S enc_f_k(C d, int i, C scale, uint32_t salt) {
     if constexpr (Storage<S>::offset) return from_c_step<S>(KS ? d : d * scale, salt);
-    else return from_c_step<S>(weight<LF, C>(i) + d, salt);
+    else return from_c_step<S>(KS ? d : weight<LF, C>(i) + d, salt);
 }
 template <class S, class C, bool KS>
 __device__ __forceinline__ S enc_g_k(C g, C scale, uint32_t salt) {
@@ -1044,7 +1110,7 @@ __device__ __forceinline__ void pull_node_vec(const S* __restrict__ own, const K
 // Wall and periodic rules for the nodes of a thread at the edge of the cell.
 // Kept out of line: only edge threads call it, and its fully unrolled body
 // would otherwise crowd the instruction cache of the hot path.
-template <int DIM, class S, int VEC, class C, int MODE = PULL>
+template <int DIM, class S, int VEC, class C, int MODE, bool RAW>
 __device__ __noinline__ void edge_writes(S* __restrict__ dst, const KParams& p, int x0, int y, int z,
                                          const C* __restrict__ post, uint32_t salt) {
     using LF = typename Lat<DIM>::F;
@@ -1057,11 +1123,11 @@ __device__ __noinline__ void edge_writes(S* __restrict__ dst, const KParams& p, 
         if (x >= p.L.nx) break;
         static_for<QF>([&](auto ii) {
             constexpr int i = decltype(ii)::value;
-            ghost_write<LF, false, i, S, C, MODE>(dst, p, x, y, z, post[i * VEC + k], scale, salt);
+            ghost_write<LF, false, i, S, C, MODE, RAW>(dst, p, x, y, z, post[i * VEC + k], scale, salt);
         });
         static_for<QG>([&](auto ii) {
             constexpr int i = decltype(ii)::value;
-            ghost_write<LG, true, i, S, C, MODE>(gdst, p, x, y, z, post[(QF + i) * VEC + k], scale, salt);
+            ghost_write<LG, true, i, S, C, MODE, RAW>(gdst, p, x, y, z, post[(QF + i) * VEC + k], scale, salt);
         });
     }
 }
@@ -1073,7 +1139,7 @@ template <class LS, bool THERMAL, int SIDE, class S, int VEC, class C, bool KS, 
 __device__ __forceinline__ void x_face(S* __restrict__ base, const KParams& p, int x, int y, int z, int k,
                                        const C (&v)[LS::Q][VEC], uint32_t salt) {
     const C scale = ScaleOf<C>::s(p);
-    const C un = KS ? ScaleOf<C>::inv(p) : C(1);  // the wall rules take unscaled values
+    const C un = KS && Storage<S>::offset ? ScaleOf<C>::inv(p) : C(1);  // the wall rules take unscaled values
     static_for<LS::Q>([&](auto ii) {
         constexpr int i = decltype(ii)::value;
         if constexpr (LS::e(i, 0) == SIDE) {
@@ -1081,7 +1147,7 @@ __device__ __forceinline__ void x_face(S* __restrict__ base, const KParams& p, i
 #pragma unroll
             for (int kk = 1; kk < VEC; ++kk)
                 if (k == kk) val = v[i][kk];
-            ghost_write<LS, THERMAL, i, S, C, MODE>(base, p, x, y, z, KS ? val * un : val, scale, salt);
+            ghost_write<LS, THERMAL, i, S, C, MODE, KS && !Storage<S>::offset>(base, p, x, y, z, KS && Storage<S>::offset ? val * un : val, scale, salt);
         }
     });
 }
@@ -1102,15 +1168,15 @@ __device__ __forceinline__ void wall_writes(S* __restrict__ dst, const KParams& 
     const bool face_row = (y == 0) || (y == L.ny - 1) || (DIM == 3 && (z == 0 || z == L.nz - 1));
     if (face_row || ((xlo || xhi) && (p.periodic & 1))) {
         C post[(QF + QG) * VEC];
-        const C un = KS ? ScaleOf<C>::inv(p) : C(1);  // the wall rules take unscaled values
+        const C un = KS && Storage<S>::offset ? ScaleOf<C>::inv(p) : C(1);  // the wall rules take unscaled values
 #pragma unroll
         for (int k = 0; k < VEC; ++k) {
 #pragma unroll
-            for (int i = 0; i < QF; ++i) post[i * VEC + k] = KS ? f[i][k] * un : f[i][k];
+            for (int i = 0; i < QF; ++i) post[i * VEC + k] = KS && Storage<S>::offset ? f[i][k] * un : f[i][k];
 #pragma unroll
-            for (int i = 0; i < QG; ++i) post[(QF + i) * VEC + k] = KS ? g[i][k] * un : g[i][k];
+            for (int i = 0; i < QG; ++i) post[(QF + i) * VEC + k] = KS && Storage<S>::offset ? g[i][k] * un : g[i][k];
         }
-        edge_writes<DIM, S, VEC, C, MODE>(dst, p, x0, y, z, post, salt);
+        edge_writes<DIM, S, VEC, C, MODE, KS && !Storage<S>::offset>(dst, p, x0, y, z, post, salt);
         return;
     }
     S* __restrict__ gdst = dst + (long long)QF * L.plane;
@@ -1145,7 +1211,7 @@ __device__ __forceinline__ void step_block(const S* __restrict__ src, S* __restr
     const int x0ld = min(x0, p.xmax_load);
     const C scale = ScaleOf<C>::s(p);
     const long long row = L.row(y, z);
-    constexpr bool KS = TRT && Storage<S>::offset;  // TRT works on the stored, scaled values
+    constexpr bool KS = TRT;  // TRT works on the stored values
     const uint32_t tcount = step_count<S, CG>(src, 0);
     const uint32_t salt = step_salt(tcount);
     advance_count<S>(dst, 0, tcount, bx == 0 && by == 0 && bz == 0 && threadIdx.x == 0 && threadIdx.y == 0);
@@ -1265,7 +1331,7 @@ __device__ __forceinline__ void step_block_aa(S* buf, const KParams& p, int bx, 
     const C scale = ScaleOf<C>::s(p);
     const C inv_scale = ScaleOf<C>::inv(p);
     const long long row = L.row(y, z);
-    constexpr bool KS = TRT && Storage<S>::offset;
+    constexpr bool KS = TRT;
     // the step counter alternates between words 0 and 1 of the single buffer
     const uint32_t tcount = step_count<S>(buf, MODE == AA_ODD ? 1 : 0);
     const uint32_t salt = step_salt(tcount);
@@ -1485,7 +1551,7 @@ __device__ __forceinline__ void step_rows_block(const S* __restrict__ src, S* __
                                                 int bx, int by, int bz) {
     using C = typename Storage<S>::C;
     constexpr int QF = Lat<DIM>::F::Q, QG = Lat<DIM>::G::Q;
-    constexpr bool KS = TRT && Storage<S>::offset;
+    constexpr bool KS = TRT;
     const Layout& L = p.L;
     const int lane = threadIdx.x & 31;
     const int y0 = (by * blockDim.y + threadIdx.y) * ROWS;
