@@ -26,6 +26,7 @@ COMMON = ["-O3", "-std=c++17", "-lineinfo", "-Xcompiler", "-fPIC", "-Xcompiler",
 # translation unit -> extra flags
 UNITS = {
     "api.cu": [],
+    "diag.cu": [],
     "step_2d_f32.cu": [],
     "step_2d_f16.cu": [],
     "step_3d_f32.cu": [],

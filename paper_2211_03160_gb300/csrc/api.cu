@@ -12,6 +12,7 @@
 #include <new>
 
 #include "../../include/tlbm.h"
+#include "diag.h"
 #include "dispatch.h"
 #include "handle.h"
 
@@ -19,9 +20,8 @@ using namespace tlbm;
 
 namespace {
 
-constexpr int RED_BLOCKS = 1024;   // fixed reduction grid: the summation order never changes
-constexpr int RED_THREADS = 256;
-constexpr int RED_FIELDS = 6;      // sum u_h T, sum 1/2 rho u^2, sum rho, max u^2, bad, sum T
+constexpr int RED_ROWS = 1024;     // rows of reduction partials in the bound block's scratch
+static_assert(RED_ROWS >= RED_BLOCKS, "scratch of the reductions");
 constexpr long long STAGE_NODES = 1ll << 21;  // FP64 staging chunk for population transfers
 
 thread_local char g_create_error[256] = "";
@@ -251,105 +251,6 @@ __global__ void gather_kernel(const S* __restrict__ buf, double* __restrict__ st
     }
 }
 
-// rho, u, T of the current state into dense caller arrays.
-template <int DIM, class S, class O>
-__global__ void macros_kernel(const S* __restrict__ buf, const KParams p, O* rho, O* ux, O* uy, O* uz, O* T) {
-    using LF = typename Lat<DIM>::F;
-    using LG = typename Lat<DIM>::G;
-    const Layout& L = p.L;
-    const long long N = (long long)L.nx * L.ny * L.nz;
-    for (long long n = blockIdx.x * (long long)blockDim.x + threadIdx.x; n < N;
-         n += (long long)gridDim.x * blockDim.x) {
-        int x, y, z;
-        node_xyz(n, L, x, y, z);
-        double f[LF::Q], g[LG::Q], r, u[3], t;
-        pull_node<DIM, S, double>(buf, p, x, y, z, f, g);
-        node_macros<DIM, double>(f, g, p, r, u, t);
-        if (rho) rho[n] = (O)r;
-        if (ux) ux[n] = (O)u[0];
-        if (uy) uy[n] = (O)u[1];
-        if (uz) uz[n] = (O)u[2];
-        if (T) T[n] = (O)t;
-    }
-}
-
-// Deterministic FP64 reduction, pass 1: each block sums a fixed node subset in
-// a fixed order (per-thread serial loop over every (RED_BLOCKS * RED_THREADS)-th
-// node, then a fixed warp-shuffle tree and a fixed cross-warp order) and writes
-// its partials.  The node coordinates advance by the stride's (x, y, z) digits
-// with carries instead of a division per node.
-template <int DIM, class S>
-__global__ void __launch_bounds__(RED_THREADS) reduce_kernel(const S* __restrict__ buf, const KParams p,
-                                                            double* __restrict__ partials) {
-    const Layout& L = p.L;
-    const long long N = (long long)L.nx * L.ny * L.nz;
-    double acc[RED_FIELDS] = {0, 0, 0, 0, 0, 0};
-    const long long n0 = blockIdx.x * (long long)RED_THREADS + threadIdx.x;
-    if (n0 < N) {
-        constexpr long long STR = (long long)RED_BLOCKS * RED_THREADS;
-        int x, y, z;
-        node_xyz(n0, L, x, y, z);
-        int sx, sy, sz;
-        node_xyz(STR, L, sx, sy, sz);  // the stride in mixed radix (nx, ny, .)
-        while (z < L.nz) {
-            double t[5];
-            node_terms<DIM, S>(buf, p, x, y, z, t);
-            acc[0] += t[0];
-            acc[1] += t[1];
-            acc[2] += t[2];
-            acc[3] = fmax(acc[3], t[3]);
-            if (!isfinite(t[2]) || !isfinite(t[4]) || !isfinite(t[3])) acc[4] = 1.0;
-            acc[5] += t[4];
-            x += sx;
-            const int cx = x >= L.nx;
-            x -= cx * L.nx;
-            y += sy + cx;
-            const int cy = y >= L.ny;
-            y -= cy * L.ny;
-            z += sz + cy;
-        }
-    }
-#pragma unroll
-    for (int off = 16; off > 0; off >>= 1) {
-#pragma unroll
-        for (int k = 0; k < RED_FIELDS; ++k) {
-            const double o = __shfl_down_sync(0xffffffffu, acc[k], off);
-            acc[k] = (k == 3 || k == 4) ? fmax(acc[k], o) : acc[k] + o;
-        }
-    }
-    __shared__ double sm[RED_THREADS / 32][RED_FIELDS];
-    const int w = threadIdx.x >> 5;
-    if ((threadIdx.x & 31) == 0)
-        for (int k = 0; k < RED_FIELDS; ++k) sm[w][k] = acc[k];
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        double out[RED_FIELDS];
-        for (int k = 0; k < RED_FIELDS; ++k) out[k] = sm[0][k];
-        for (int j = 1; j < RED_THREADS / 32; ++j)
-            for (int k = 0; k < RED_FIELDS; ++k)
-                out[k] = (k == 3 || k == 4) ? fmax(out[k], sm[j][k]) : out[k] + sm[j][k];
-        for (int k = 0; k < RED_FIELDS; ++k) partials[(long long)blockIdx.x * RED_FIELDS + k] = out[k];
-    }
-}
-
-// Pass 2: one block combines the RED_BLOCKS partials in a fixed tree.
-__global__ void __launch_bounds__(RED_BLOCKS) reduce_final_kernel(const double* __restrict__ partials,
-                                                                 double* __restrict__ out) {
-    __shared__ double sm[RED_BLOCKS];
-    for (int k = 0; k < RED_FIELDS; ++k) {
-        sm[threadIdx.x] = partials[(long long)threadIdx.x * RED_FIELDS + k];
-        __syncthreads();
-        for (int s = RED_BLOCKS / 2; s > 0; s >>= 1) {
-            if ((int)threadIdx.x < s)
-                sm[threadIdx.x] = (k == 3 || k == 4) ? fmax(sm[threadIdx.x], sm[threadIdx.x + s])
-                                                     : sm[threadIdx.x] + sm[threadIdx.x + s];
-            __syncthreads();
-        }
-        if (threadIdx.x == 0) out[k] = sm[0];
-        __syncthreads();
-    }
-}
-
 template <int DIM, class S>
 struct DiagKernels {
     static cudaError_t init(void* buf, const KParams& p, uint64_t seed, double amp, cudaStream_t s) {
@@ -369,23 +270,6 @@ struct DiagKernels {
     static cudaError_t gather(const void* buf, double* st, int pop, long long n0, long long cnt, const Window& w,
                               const KParams& p, cudaStream_t s, bool dev = false) {
         gather_kernel<DIM, S><<<1024, 256, 0, s>>>((const S*)buf, st, pop, n0, cnt, w, p, dev);
-        return cudaGetLastError();
-    }
-    static cudaError_t macros(const void* buf, const KParams& p, void* r, void* ux, void* uy, void* uz, void* T,
-                              int dt, cudaStream_t s) {
-        if (dt == TLBM_OUT_F64)
-            macros_kernel<DIM, S, double><<<2048, 256, 0, s>>>((const S*)buf, p, (double*)r, (double*)ux,
-                                                               (double*)uy, (double*)uz, (double*)T);
-        else
-            macros_kernel<DIM, S, float><<<2048, 256, 0, s>>>((const S*)buf, p, (float*)r, (float*)ux,
-                                                              (float*)uy, (float*)uz, (float*)T);
-        return cudaGetLastError();
-    }
-    static cudaError_t reduce(const void* buf, const KParams& p, double* partials, double* out, cudaStream_t s) {
-        reduce_kernel<DIM, S><<<RED_BLOCKS, RED_THREADS, 0, s>>>((const S*)buf, p, partials);
-        cudaError_t e = cudaGetLastError();
-        if (e != cudaSuccess) return e;
-        reduce_final_kernel<<<1, RED_BLOCKS, 0, s>>>(partials, out);
         return cudaGetLastError();
     }
 };
@@ -689,7 +573,7 @@ extern "C" int tlbm_create(tlbm_t* out, int nx, int ny, int nz, int lattice, dou
         if (dim == 2 && precision == TLBM_FP32) h->by = 1;  // 57.4 vs 56.0 GLUPS with 32 x 4 at 8193^2
     }
     h->red_off = h->nbuf * h->popset_bytes;
-    h->res_off = h->red_off + align_up((size_t)RED_BLOCKS * RED_FIELDS * sizeof(double), 256);
+    h->res_off = h->red_off + align_up((size_t)RED_ROWS * RED_FIELDS * sizeof(double), 256);
     h->status_off = h->res_off + 128;
     h->stage_off = h->res_off + 256;
     const long long N = (long long)nx * ny * nz;
@@ -896,36 +780,89 @@ extern "C" int tlbm_macros(tlbm_t h, void* rho, void* ux, void* uy, void* uz, vo
     TLBM_CHECK_BOUND(h);
     if (out_dtype != TLBM_OUT_F64 && out_dtype != TLBM_OUT_F32) return fail(h, TLBM_ERR_ARG, "bad out_dtype");
     if (h->dim == 2) uz = nullptr;
-    cudaError_t e = with_types(h->dim, h->prec, [&](auto K) {
-        return decltype(K)::macros(h->buf[h->cur], h->kp, rho, ux, uy, uz, T, out_dtype, h->stream);
-    });
+    cudaError_t e = launch_macros(h->dim, h->prec, h->buf[h->cur], h->kp, rho, ux, uy, uz, T,
+                                  out_dtype == TLBM_OUT_F64, h->stream);
     if (e != cudaSuccess) return cuda_fail(h, e, "macros kernel");
     h->launches += 1;
     return TLBM_OK;
 }
 
+// the reduction's view of a handle's current state (parameters by value)
+static RedState red_state(tlbm_t h) {
+    return {h->buf[h->cur], nullptr, (double*)(h->mem + h->red_off), (const int*)(h->mem + h->status_off), 0, 0};
+}
+
 // runs the two-pass reduction and copies the six results to the host
 static int run_reduce(tlbm_t h, double* res) {
-    double* partials = (double*)(h->mem + h->red_off);
     double* out = (double*)(h->mem + h->res_off);
-    cudaError_t e = with_types(h->dim, h->prec, [&](auto K) {
-        return decltype(K)::reduce(h->buf[h->cur], h->kp, partials, out, h->stream);
-    });
+    RedStates st;
+    st.s[0] = red_state(h);
+    const KParams* kp = &h->kp;
+    cudaError_t e = launch_reduce(h->dim, h->prec, st, 1, &kp, out, h->stream);
     if (e != cudaSuccess) return cuda_fail(h, e, "reduction kernel");
     h->launches += 2;
-    e = cudaMemcpyAsync(res, out, RED_FIELDS * sizeof(double), cudaMemcpyDeviceToHost, h->stream);
-    if (e != cudaSuccess) return cuda_fail(h, e, "cudaMemcpyAsync");
-    int status = 0;
-    e = cudaMemcpyAsync(&status, h->mem + h->status_off, sizeof(int), cudaMemcpyDeviceToHost, h->stream);
+    double r[8];
+    e = cudaMemcpyAsync(r, out, sizeof(r), cudaMemcpyDeviceToHost, h->stream);
     if (e != cudaSuccess) return cuda_fail(h, e, "cudaMemcpyAsync");
     e = cudaStreamSynchronize(h->stream);
     if (e != cudaSuccess) return cuda_fail(h, e, "cudaStreamSynchronize");
-    if (status) return fail(h, TLBM_ERR_TIMEOUT, "a staged step gave up waiting for its copies");
+    memcpy(res, r, RED_FIELDS * sizeof(double));
+    if (r[6] != 0.0) return fail(h, TLBM_ERR_TIMEOUT, "a staged step gave up waiting for its copies");
     return TLBM_OK;
 }
 
 // the reduction found a non-finite value or |u| > 0.5 (|u|^2 > 0.25)
 static bool reduce_diverged(const double* r) { return r[4] != 0.0 || !(r[3] <= 0.25); }
+
+static double nusselt_of(tlbm_t h, const double* r) {
+    const double N = (double)h->nx * h->ny * h->nz;
+    const int ax = h->kp.heat_axis;
+    const double L = ax == 0 ? h->nx : (ax == 1 ? h->ny : h->nz);
+    return 1.0 + L * (r[0] / N) / (h->alpha * (h->prm.Th - h->prm.Tc));
+}
+
+// The reductions of n bound two-buffer handles of one lattice and storage whose
+// work is all on `stream`, RED_MANY at a time in two launches and one copy (a
+// reduction on its own costs about 20 us of launches, copy and wait whatever
+// its size).  d_kp[i]: handle i's parameters in device memory.  nu (may be
+// null) and diverged as tlbm_nusselt and tlbm_status give them.
+int tlbm::reduce_many(tlbm_t* hs, int n, const KParams* d_kp, cudaStream_t stream, double* nu, int* diverged,
+                      int* failed) {
+    for (int i0 = 0; i0 < n; i0 += RED_MANY) {
+        const int count = std::min(RED_MANY, n - i0);
+        RedStates st;
+        const KParams* kp[RED_MANY];
+        for (int i = 0; i < count; ++i) {
+            st.s[i] = red_state(hs[i0 + i]);
+            st.s[i].kp = d_kp + i0 + i;
+            kp[i] = &hs[i0 + i]->kp;
+        }
+        // results behind the first handle's partials
+        static_assert((RED_ROWS - RED_BLOCKS) * RED_FIELDS >= 8 * RED_MANY, "scratch of the results");
+        tlbm_t h = hs[i0];
+        double* out = (double*)(h->mem + h->red_off) + RED_BLOCKS * RED_FIELDS;
+        double r[8 * RED_MANY];
+        cudaError_t e = launch_reduce(h->dim, h->prec, st, count, kp, out, stream);
+        if (e == cudaSuccess) e = cudaMemcpyAsync(r, out, count * 8 * sizeof(double), cudaMemcpyDeviceToHost, stream);
+        if (e == cudaSuccess) e = cudaStreamSynchronize(stream);
+        *failed = i0;
+        if (e != cudaSuccess) return cuda_fail(h, e, "reduction");
+        h->launches += 2;
+        for (int i = 0; i < count; ++i) {
+            tlbm_t q = hs[i0 + i];
+            const double* v = r + 8 * i;
+            *failed = i0 + i;
+            q->err[0] = 0;
+            if (v[6] != 0.0) return fail(q, TLBM_ERR_TIMEOUT, "a staged step gave up waiting for its copies");
+            diverged[i0 + i] = reduce_diverged(v) ? 1 : 0;
+            if (nu) {
+                nu[i0 + i] = nusselt_of(q, v);
+                if (diverged[i0 + i]) fail(q, TLBM_ERR_DIVERGED, "the state has diverged (the value is written)");
+            }
+        }
+    }
+    return TLBM_OK;
+}
 
 extern "C" int tlbm_nusselt(tlbm_t h, double* nu) {
     TLBM_CHECK_HANDLE(h);
@@ -934,10 +871,7 @@ extern "C" int tlbm_nusselt(tlbm_t h, double* nu) {
     double r[RED_FIELDS];
     int rc = run_reduce(h, r);
     if (rc) return rc;
-    const double N = (double)h->nx * h->ny * h->nz;
-    const int ax = h->kp.heat_axis;
-    const double L = ax == 0 ? h->nx : (ax == 1 ? h->ny : h->nz);
-    *nu = 1.0 + L * (r[0] / N) / (h->alpha * (h->prm.Th - h->prm.Tc));
+    *nu = nusselt_of(h, r);
     if (reduce_diverged(r)) return fail(h, TLBM_ERR_DIVERGED, "the state has diverged (the value is written)");
     return TLBM_OK;
 }

@@ -909,21 +909,41 @@ extern "C" int tlbm_batch_instance(tlbm_batch_t b, int idx, tlbm_t* out) {
     return TLBM_OK;
 }
 
+// The instances' reductions into diverged[n] and, unless null, nu[n]: all
+// together where every instance still runs on the batch's stream and buffers
+// (a borrowed instance may have been given others), else one after the other.
+static int batch_reduce(tlbm_batch_t b, double* nu, int* diverged) {
+    bool together = b->mem != nullptr;
+    for (int i = 0; i < b->n; ++i)
+        together = together && b->inst[i]->stream == b->stream && b->inst[i]->mem == b->mem + b->off[i];
+    if (together) {
+        int at = 0;
+        const int rc = reduce_many(b->inst.data(), b->n, b->d_kp, b->stream, nu, diverged, &at);
+        return rc == TLBM_OK ? rc : bfail(b, rc, "instance %d: %s", at, tlbm_last_error(b->inst[at]));
+    }
+    for (int i = 0; i < b->n; ++i) {
+        int rc;
+        if (nu) {
+            rc = tlbm_nusselt(b->inst[i], &nu[i]);
+            diverged[i] = rc == TLBM_ERR_DIVERGED;
+            if (diverged[i]) rc = TLBM_OK;
+        } else {
+            rc = tlbm_status(b->inst[i], &diverged[i], nullptr);
+        }
+        if (rc != TLBM_OK) return bfail(b, rc, "instance %d: %s", i, tlbm_last_error(b->inst[i]));
+    }
+    return TLBM_OK;
+}
+
 extern "C" int tlbm_batch_nusselt(tlbm_batch_t b, double* nu) {
     if (!b) return bfail(nullptr, TLBM_ERR_ARG, "NULL batch");
     if (!nu) return bfail(b, TLBM_ERR_ARG, "nu is NULL");
-    int first_diverged = -1;
-    for (int i = 0; i < b->n; ++i) {
-        int rc = tlbm_nusselt(b->inst[i], &nu[i]);
-        if (rc == TLBM_ERR_DIVERGED) {
-            if (first_diverged < 0) first_diverged = i;
-        } else if (rc != TLBM_OK) {
-            return bfail(b, rc, "instance %d: %s", i, tlbm_last_error(b->inst[i]));
-        }
-    }
-    if (first_diverged >= 0)
-        return bfail(b, TLBM_ERR_DIVERGED, "instance %d (and maybe others) has diverged; every value is written",
-                      first_diverged);
+    std::vector<int> diverged(b->n, 0);
+    const int rc = batch_reduce(b, nu, diverged.data());
+    if (rc != TLBM_OK) return rc;
+    for (int i = 0; i < b->n; ++i)
+        if (diverged[i])
+            return bfail(b, TLBM_ERR_DIVERGED, "instance %d (and maybe others) has diverged; every value is written", i);
     return TLBM_OK;
 }
 
@@ -945,11 +965,7 @@ extern "C" int tlbm_batch_status(tlbm_batch_t b, int* diverged) {
         if (gs.status) return bfail(b, TLBM_ERR_TIMEOUT, "a persistent launch gave up waiting at a grid barrier");
         if (gs.staged_status) return bfail(b, TLBM_ERR_TIMEOUT, "a staged step gave up waiting for its copies");
     }
-    for (int i = 0; i < b->n; ++i) {
-        int rc = tlbm_status(b->inst[i], &diverged[i], nullptr);
-        if (rc != TLBM_OK) return bfail(b, rc, "instance %d: %s", i, tlbm_last_error(b->inst[i]));
-    }
-    return TLBM_OK;
+    return batch_reduce(b, nullptr, diverged);
 }
 
 extern "C" int tlbm_batch_macros(tlbm_batch_t b, int idx, void* rho, void* ux, void* uy, void* uz, void* T,

@@ -39,3 +39,10 @@ struct tlbm_s {
     int64_t launches;
     char err[256];
 };
+
+namespace tlbm {
+// The reductions of many handles at once (api.cu); the first handle that
+// failed in *failed.
+int reduce_many(tlbm_t* hs, int n, const KParams* d_kp, cudaStream_t stream, double* nu, int* diverged,
+                int* failed);
+}  // namespace tlbm

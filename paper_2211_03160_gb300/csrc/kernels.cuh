@@ -824,35 +824,6 @@ __device__ __forceinline__ void collide_vec(C (&f)[Lat<DIM>::F::Q][VEC], C (&g)[
     }
 }
 
-// Node macros from deviations (used by the diagnostic kernels).
-template <int DIM, class C>
-__device__ __forceinline__ void node_macros(const C (&d)[Lat<DIM>::F::Q], const C (&g)[Lat<DIM>::G::Q],
-                                            const KParams& p, C& rho, C (&u)[3], C& T) {
-    using LF = typename Lat<DIM>::F;
-    using LG = typename Lat<DIM>::G;
-    using P = PV<C>;
-    C drho = C(0), j[3] = {C(0), C(0), C(0)}, t = C(0);
-    static_for<LF::Q>([&](auto ii) {
-        constexpr int i = decltype(ii)::value;
-        drho += d[i];
-        if constexpr (LF::e(i, 0) == 1) j[0] += d[i];
-        if constexpr (LF::e(i, 0) == -1) j[0] -= d[i];
-        if constexpr (LF::e(i, 1) == 1) j[1] += d[i];
-        if constexpr (LF::e(i, 1) == -1) j[1] -= d[i];
-        if constexpr (LF::e(i, 2) == 1) j[2] += d[i];
-        if constexpr (LF::e(i, 2) == -1) j[2] -= d[i];
-    });
-    static_for<LG::Q>([&](auto ii) { t += g[decltype(ii)::value]; });
-    rho = C(1) + drho;
-    T = t;
-    C F[3] = {rho * P::body(p, 0), rho * P::body(p, 1), rho * P::body(p, 2)};
-    F[DIM - 1] += rho * P::gbeta(p) * t;
-    const C ir = C(1) / rho;
-    u[0] = (j[0] + C(0.5) * F[0]) * ir;
-    u[1] = (j[1] + C(0.5) * F[1]) * ir;
-    u[2] = DIM == 3 ? (j[2] + C(0.5) * F[2]) * ir : C(0);
-}
-
 // ------------------------------------------------------------------ vector IO
 
 // Loads of the populations: through the read-only path (ld.global.nc) when the
@@ -1070,17 +1041,6 @@ __device__ __forceinline__ void enc_vec(const C (&v)[VEC], int i, C scale, uint3
         for (int k = 0; k < VEC; ++k)
             out[k] = i >= 0 ? enc_f_k<LF, S, C, KS>(v[k], i, scale, salt) : enc_g_k<S, C, KS>(v[k], scale, salt);
     }
-}
-
-template <class LF, class S, class C>
-__device__ __forceinline__ C raw_to_dev(C raw, int i, C inv_scale) {
-    if constexpr (Storage<S>::offset) return raw * inv_scale;
-    else return raw - weight<LF, C>(i);
-}
-template <class S, class C>
-__device__ __forceinline__ C raw_to_g(C raw, C inv_scale) {
-    if constexpr (Storage<S>::offset) return raw * inv_scale;
-    else return raw;
 }
 
 // Pull the pre-collision populations of nodes x0 .. x0+VEC-1 whose own slot in
@@ -1617,46 +1577,6 @@ __device__ __forceinline__ long long pre_index(const KParams& p, int x, int y, i
     if (p.state == 1) return (long long)j * L.plane + L.slot(x, y, z);
     const int plane = p.state == 2 ? LS::opp(j) : j;
     return (long long)plane * L.plane + L.slot(x - ex, y - ey, z - ez);
-}
-
-// Canonical pre-collision populations of one node (scalar reads).
-template <int DIM, class S, class C>
-__device__ __forceinline__ void pull_node(const S* __restrict__ src, const KParams& p, int x, int y, int z,
-                                          C (&f)[Lat<DIM>::F::Q], C (&g)[Lat<DIM>::G::Q]) {
-    using LF = typename Lat<DIM>::F;
-    using LG = typename Lat<DIM>::G;
-    const Layout& L = p.L;
-    const C inv_scale = ScaleOf<C>::inv(p);
-    const S* __restrict__ gsrc = src + (long long)LF::Q * L.plane;
-    static_for<LF::Q>([&](auto ii) {
-        constexpr int i = decltype(ii)::value;
-        const C raw = to_c<C>(*TLBM_DBG(p, (src + pre_index<LF, i>(p, x, y, z)), 0, 1));
-        f[i] = raw_to_dev<LF, S, C>(raw, i, inv_scale);
-    });
-    static_for<LG::Q>([&](auto ii) {
-        constexpr int i = decltype(ii)::value;
-        const C raw = to_c<C>(*TLBM_DBG(p, (gsrc + pre_index<LG, i>(p, x, y, z)), 0, 1));
-        g[i] = raw_to_g<S, C>(raw, inv_scale);
-    });
-}
-
-// Per-node terms of the reductions (a6): u_h T, 1/2 rho |u|^2, rho, |u|^2, T,
-// formed in the storage's collision precision (FP64 storage: FP64; otherwise
-// FP32, the precision the state was computed in) and handed over in FP64 for
-// the FP64 sums.
-template <int DIM, class S>
-__device__ __forceinline__ void node_terms(const S* __restrict__ buf, const KParams& p, int x, int y, int z,
-                                           double (&t)[5]) {
-    using C = typename Storage<S>::C;
-    C f[Lat<DIM>::F::Q], g[Lat<DIM>::G::Q], r, u[3], T;
-    pull_node<DIM, S, C>(buf, p, x, y, z, f, g);
-    node_macros<DIM, C>(f, g, p, r, u, T);
-    const C u2 = u[0] * u[0] + u[1] * u[1] + u[2] * u[2];
-    t[0] = (double)(u[p.heat_axis] * T);
-    t[1] = (double)(C(0.5) * r * u2);
-    t[2] = (double)r;
-    t[3] = (double)u2;
-    t[4] = (double)T;
 }
 
 }  // namespace tlbm

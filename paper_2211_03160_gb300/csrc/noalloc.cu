@@ -18,8 +18,8 @@
 #include <mutex>
 
 #include "../../include/tlbm.h"
+#include "diag.cuh"
 #include "handle.h"
-#include "kernels.cuh"
 
 using namespace tlbm;
 
@@ -45,9 +45,7 @@ __device__ __align__(256) double g_noalloc_scratch[NA_SLOTS * NA_FIELDS + 8];
 // non-finite flag, sum T.
 template <int DIM, class S>
 __global__ void __launch_bounds__(NA_THREADS) noalloc_partials(const S* __restrict__ buf, const KParams p,
-                                                               double* __restrict__ scratch) {
-    using LF = typename Lat<DIM>::F;
-    using LG = typename Lat<DIM>::G;
+                                                               const DiagOff k, double* __restrict__ scratch) {
     const Layout& L = p.L;
     const long long N = (long long)L.nx * L.ny * L.nz;
     const long long n0 = (long long)blockIdx.x * NA_CHUNK;
@@ -58,12 +56,12 @@ __global__ void __launch_bounds__(NA_THREADS) noalloc_partials(const S* __restri
         const long long r = n / L.nx;
         const int y = (int)(r % L.ny);
         const int z = (int)(r / L.ny);
-        double t[5];
-        node_terms<DIM, S>(buf, p, x, y, z, t);
+        typename Storage<S>::C t[5];
+        node_terms<DIM, S>(buf + L.slot(x, y, z), p, k.off, t);
         acc[0] += t[0];
         acc[1] += t[1];
         acc[2] += t[2];
-        acc[3] = fmax(acc[3], t[3]);
+        acc[3] = fmax(acc[3], (double)t[3]);
         if (!isfinite(t[2]) || !isfinite(t[4]) || !isfinite(t[3])) acc[4] = 1.0;
         acc[5] += t[4];
     }
@@ -113,7 +111,7 @@ __global__ void __launch_bounds__(NA_FINAL_THREADS) noalloc_final(double* __rest
 
 template <int DIM, class S>
 cudaError_t launch_partials(const void* buf, const KParams& p, double* scratch, int slots, cudaStream_t s) {
-    noalloc_partials<DIM, S><<<slots, NA_THREADS, 0, s>>>((const S*)buf, p, scratch);
+    noalloc_partials<DIM, S><<<slots, NA_THREADS, 0, s>>>((const S*)buf, p, diag_offsets<DIM>(p), scratch);
     return cudaGetLastError();
 }
 

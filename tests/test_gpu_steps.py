@@ -32,3 +32,109 @@ def test_fp64_collision_with_a_force_on_every_axis(T, O, lattice, shape, pm, inp
     (fg, tg), (fo, to) = g.get_populations(), o.get_populations()
     assert np.abs(fg - fo).max() < 1e-14 and np.abs(tg - to).max() < 1e-14
     g.close()
+
+
+def _reference_fields(f, g, lattice, derived):
+    """rho, u, T in FP64 from populations f, g (the definitions of §2.2)."""
+    if lattice == D2:
+        E = [(0, 0), (1, 0), (0, 1), (-1, 0), (0, -1), (1, 1), (-1, 1), (-1, -1), (1, -1)]
+    else:
+        E = [(0, 0, 0), (1, 0, 0), (-1, 0, 0), (0, 1, 0), (0, -1, 0), (0, 0, 1), (0, 0, -1), (1, 1, 0), (-1, -1, 0),
+             (1, -1, 0), (-1, 1, 0), (1, 0, 1), (-1, 0, -1), (1, 0, -1), (-1, 0, 1), (0, 1, 1), (0, -1, -1),
+             (0, 1, -1), (0, -1, 1)]
+    rho, T = f.sum(0), g.sum(0)
+    dim = len(E[0])
+    j = [sum(e[a] * f[i] for i, e in enumerate(E) if e[a]) for a in range(dim)]
+    j[-1] = j[-1] + 0.5 * rho * derived["gbeta"] * T
+    return rho, [v / rho for v in j], T
+
+
+@pytest.mark.parametrize("prec", [0, 1, 2, 3])
+@pytest.mark.parametrize("lattice,shape", [(D2, (3, 3, 1)), (D2, (33, 5, 1)), (D2, (64, 40, 1)), (D3, (5, 4, 3)),
+                                           (D3, (65, 3, 4))])
+@pytest.mark.parametrize("inplace", [False, True])
+def test_fields_and_reductions_of_every_state_order(T, prec, lattice, shape, inplace):  # noqa: F811
+    """Fields (FP64 and FP32 arrays), Nusselt number, energy and mass against
+    their definitions, for every storage and state order (pull, natural,
+    swapped).  FP64 fields: a few roundings of 2^-53 of O(1) values.  FP32 fields:
+    the FP64 ones rounded, at most one unit apart where a rounding boundary
+    falls between the two evaluations.  Sums: FP64 storage to 1e-13 of the
+    terms' magnitudes, the others to the 2^-24 roundings of an FP32 term (about
+    20 of them)."""
+    import torch
+
+    nx, ny, nz = shape
+    qf, qg = (9, 5) if lattice == D2 else (19, 7)
+    full = (ny, nx) if lattice == D2 else (nz, ny, nx)
+    s = T.Sim(nx, ny, nz, lattice=lattice, Ra=1e5, Pr=0.71, Ma=0.1, precision=prec,
+              streaming=T.TLBM_STREAM_INPLACE if inplace else T.TLBM_STREAM_PULL)
+    w = np.array([16, 4, 4, 4, 4, 1, 1, 1, 1] if lattice == D2 else [12] + [2] * 6 + [1] * 12) / 36.0
+    f = w.reshape((qf,) + (1,) * len(full)) * (1 + 0.1 * inputs.uniform_array(3 + nx, (qf,) + full, -1, 1))
+    g = inputs.uniform_array(4 + nx, (qg,) + full, -0.1, 0.1)
+    s.set_populations(f, g)
+    d = s.derived()
+    for n in (0, 1, 1):
+        s.step(n)
+        fs, gs = s.get_populations()
+        rho, u, tt = _reference_fields(fs, gs, lattice, d)
+        m = {k: v.cpu().numpy() for k, v in s.macros().items()}
+        for name, ref in (("rho", rho), ("T", tt), ("ux", u[0]), ("uy", u[1])) + ((("uz", u[2]),) if lattice else ()):
+            assert np.abs(m[name] - ref).max() < 2e-14, (name, n)
+        m32 = {k: v.cpu().numpy() for k, v in s.macros(torch.float32).items()}
+        for name in m32:
+            r = m[name].astype(np.float32)
+            assert (np.abs(m32[name] - r) <= np.spacing(np.abs(r))).all(), (name, n)
+        uh = u[-1]
+        terms = {"nu": uh * tt, "e": 0.5 * rho * sum(v * v for v in u), "m": rho}
+        tol = {k: (1e-13 if prec == 0 else 20 * 2.0 ** -24) * np.abs(v).sum() for k, v in terms.items()}
+        L, alpha = full[0], d["alpha"]
+        nu = s.nusselt(allow_diverged=True)
+        e, mass = s.energy(allow_diverged=True)
+        assert abs((nu - 1) * alpha / L * rho.size - terms["nu"].sum()) <= tol["nu"]
+        assert abs(e - terms["e"].sum()) <= tol["e"] and abs(mass - rho.sum()) <= tol["m"]
+    s.close()
+
+
+@pytest.mark.parametrize("prec", [1, 3])
+def test_fields_outside_the_double_fp32_range(T, prec):  # noqa: F811
+    """FP32 fields of nodes whose density, momentum or temperature is too large,
+    zero, negative or not finite for the double-FP32 evaluation are those of FP64
+    arithmetic, cast."""
+    import torch
+
+    s = T.Sim(40, 6, Ra=1e5, Pr=0.71, Ma=0.1, precision=prec)
+    s.init(1, 0.0)
+    f, g = s.get_populations()
+    for k, v in enumerate((1e17, -1e20, np.inf, -np.inf, np.nan, -1.0, -40.0 / 9.0)):
+        f[1, 2, 5 * k] = v
+        g[2, 4, 5 * k] = v
+    s.set_populations(f, g)
+    m = s.macros()
+    m32 = s.macros(torch.float32)
+    for k in m:
+        a, b = m32[k].cpu().numpy(), m[k].float().cpu().numpy()
+        fin = np.isfinite(b)
+        assert np.array_equal(np.isnan(a), np.isnan(b)) and np.array_equal(np.isinf(a), np.isinf(b)), k
+        assert (np.abs(a[fin] - b[fin]) <= np.spacing(np.abs(b[fin]))).all(), k
+    s.close()
+
+
+@pytest.mark.parametrize("lattice,prec,n", [(D2, 1, 70), (D2, 2, 64), (D3, 0, 65), (D2, 0, 1)])
+def test_reductions_of_a_batch_equal_those_of_its_cells(T, lattice, prec, n):  # noqa: F811
+    """tlbm_batch_nusselt and tlbm_batch_status reduce up to 64 cells per launch:
+    bitwise the numbers of the cells reduced alone, also past the first 64, and
+    a diverged cell is named."""
+    size = lambda i: (17 + 3 * (i % 7), 12 + i % 5, 9 if lattice == D3 else 1)  # noqa: E731
+    b = T.Batch([size(i) + (1e5, 0.71, 0.1, i) for i in range(n)], lattice=lattice, precision=prec)
+    b.init(1e-2)
+    b.step(11)
+    nu = b.nusselt()
+    assert nu == [T.tlbm_nusselt(b.instance(i)) for i in range(n)] and b.status() == [False] * n
+    f, g = b.get_populations(n - 1)
+    f[1] = np.nan
+    T.tlbm_set_populations(b.instance(n - 1), f, g)
+    assert b.status() == [False] * (n - 1) + [True]
+    with pytest.raises(T.TlbmError) as ei:
+        b.nusselt()
+    assert ei.value.code == T.TLBM_ERR_DIVERGED and f"instance {n - 1} " in str(ei.value)
+    b.close()
