@@ -442,6 +442,7 @@ extern "C" int tlbm_create(tlbm_t* out, int nx, int ny, int nz, int lattice, dou
         kp.qpf = (float)kp.qp; kp.qmf = (float)kp.qm;
     }
     h->trt = kp.trt;
+    h->flat = precision == TLBM_FP64 && kp.trt;
     {
         // per-population pull / store offsets (elements, relative to a node's own
         // slot in plane 0): plane j, shifted back by the population's e_y, e_z
@@ -689,6 +690,7 @@ static cudaError_t launch_step_raw(tlbm_t h, int parity, cudaStream_t s) {
         si.wait_ns = h->wait_ns;
         return launch_staged(h->dim, h->prec, h->staged_nc, src, dst, kp, si, h->staged_grid, h->staged_smem, s);
     }
+    if (h->flat) return launch_flat_f64(h->dim, h->aa ? (parity ? AA_ODD : AA_EVEN) : PULL, src, h->aa ? h->buf[0] : dst, kp, s);
     const int vec = h->vec;
     const int bx = h->bx, by = h->by, rows = h->rows;
     const int threads_x = (h->nx + vec - 1) / vec;
@@ -1158,6 +1160,7 @@ extern "C" int tlbm_set_variant(tlbm_t h, int vec, int form, int block_x, int bl
     h->by = by;
     h->rows = nr;
     h->staged = 0;
+    h->flat = 0;
     h->variant_chosen = 1;
     h->kp.xmax_load = h->kp.L.P - v;
     drop_graph(h);

@@ -21,6 +21,10 @@ bool step_variant_available(int dim, int prec, int vec, bool trt, int rows);
 // device function of a compiled variant (for cudaFuncGetAttributes), or nullptr
 const void* step_function(int dim, int prec, int vec, bool trt, int rows);
 
+// FP64 step with one thread per node in memory order, TRT form (mode: PULL, or
+// a half of an in-place pair, which reads and writes dst)
+cudaError_t launch_flat_f64(int dim, int mode, const void* src, void* dst, const KParams& p, cudaStream_t s);
+
 // shared-memory staged (TMA bulk copy) step, TRT form, FP32/FP16/BF16 storage,
 // nc = 4 or 8 consumer warps
 const void* staged_function(int dim, int prec, int nc);

@@ -21,6 +21,7 @@ struct tlbm_s {
     int graph_steps;           // steps per CUDA graph replay in tlbm_step (0: plain launches)
     cudaGraphExec_t graph;     // captured block of graph_steps steps starting from buffer 0
     cudaStream_t capture_stream;
+    int flat;                  // 1: FP64 kernel with one thread per node in memory order
     int staged;                // 1: shared-memory staged (TMA bulk copy) kernel
     int variant_chosen;        // set by tlbm_set_variant / tlbm_set_staged: keep the caller's choice
     int staged_tw, staged_nc, staged_stages, staged_grid;

@@ -938,6 +938,7 @@ __device__ __forceinline__ void pull_row(const S* __restrict__ q, int lane, C (&
 // In both in-place halves every node reads and writes one and the same set of
 // slots, so the update is race-free in a single buffer.
 constexpr int PULL = 0, AA_EVEN = 1, AA_ODD = 2;
+constexpr int FLAT_THREADS = 128;
 
 // Write the post-collision value `val` of population i (set LS, flow or
 // thermal) of node (x, y, z) where the next step will read it, if it leaves
@@ -1151,10 +1152,22 @@ __device__ __forceinline__ void wall_writes(S* __restrict__ dst, const KParams& 
     }
 }
 
+// FLAT kernels (one node per thread): thread n of the grid (x only) takes the
+// cell's node n, x fastest, so that the lanes of a warp run over row ends and
+// only the last warp is not full.
+__device__ __forceinline__ bool flat_node(const Layout& L, int& x, int& y, int& z) {
+    const unsigned n = blockIdx.x * blockDim.x + threadIdx.x, r = n / (unsigned)L.nx;
+    const unsigned zz = L.nz > 1 ? r / (unsigned)L.ny : 0u;
+    x = (int)(n - r * (unsigned)L.nx);
+    y = (int)(r - zz * (unsigned)L.ny);
+    z = (int)zz;
+    return r < (unsigned)L.ny * (unsigned)L.nz;
+}
+
 // One thread updates VEC consecutive nodes of one row.  blockDim.x must be a
 // multiple of 32 so that a warp covers 32*VEC consecutive nodes of one row.
 // Body of the step for the block at grid position (bx, by, bz) of one cell.
-template <int DIM, class S, int VEC, bool TRT, bool CG = false>
+template <int DIM, class S, int VEC, bool TRT, bool CG = false, bool FLAT = false>
 __device__ __forceinline__ void step_block(const S* __restrict__ src, S* __restrict__ dst, const KParams& p, int bx,
                                            int by, int bz) {
     using LF = typename Lat<DIM>::F;
@@ -1163,12 +1176,18 @@ __device__ __forceinline__ void step_block(const S* __restrict__ src, S* __restr
     constexpr int QF = LF::Q, QG = LG::Q;
     const Layout& L = p.L;
     const int lane = threadIdx.x & 31;
-    const int y = by * blockDim.y + threadIdx.y;
-    const int z = DIM == 3 ? bz : 0;
-    if (y >= L.ny) return;  // uniform across the warp
-    const int x0 = (bx * blockDim.x + threadIdx.x) * VEC;
-    if (x0 - lane * VEC >= L.nx) return;  // the whole warp lies past the row end
-    const int x0ld = min(x0, p.xmax_load);
+    int x0, y, z;
+    if constexpr (FLAT) {
+        static_assert(VEC == 1, "one node per thread");
+        if (!flat_node(L, x0, y, z)) return;
+    } else {
+        y = by * blockDim.y + threadIdx.y;
+        z = DIM == 3 ? bz : 0;
+        if (y >= L.ny) return;  // uniform across the warp
+        x0 = (bx * blockDim.x + threadIdx.x) * VEC;
+        if (x0 - lane * VEC >= L.nx) return;  // the whole warp lies past the row end
+    }
+    const int x0ld = FLAT ? x0 : min(x0, p.xmax_load);
     const C scale = ScaleOf<C>::s(p);
     const long long row = L.row(y, z);
     constexpr bool KS = TRT;  // TRT works on the stored values
@@ -1274,7 +1293,7 @@ __device__ __forceinline__ void push_row(S* q, int lane, int x0, int nx, const C
 // (x - e_i) of plane ibar and pushes f+_i to (x + e_i) of plane i.  The
 // collision is the one of step_block; the wall rules go where the next half
 // reads them (ghost_write).  One buffer: `buf` is read and written.
-template <int DIM, class S, int VEC, bool TRT, int MODE>
+template <int DIM, class S, int VEC, bool TRT, int MODE, bool FLAT = false>
 __device__ __forceinline__ void step_block_aa(S* buf, const KParams& p, int bx, int by, int bz) {
     using LF = typename Lat<DIM>::F;
     using LG = typename Lat<DIM>::G;
@@ -1282,12 +1301,18 @@ __device__ __forceinline__ void step_block_aa(S* buf, const KParams& p, int bx, 
     constexpr int QF = LF::Q, QG = LG::Q;
     const Layout& L = p.L;
     const int lane = threadIdx.x & 31;
-    const int y = by * blockDim.y + threadIdx.y;
-    const int z = DIM == 3 ? bz : 0;
-    if (y >= L.ny) return;  // uniform across the warp
-    const int x0 = (bx * blockDim.x + threadIdx.x) * VEC;
-    if (x0 - lane * VEC >= L.nx) return;  // the whole warp lies past the row end
-    const int x0ld = min(x0, p.xmax_load);
+    int x0, y, z;
+    if constexpr (FLAT) {
+        static_assert(VEC == 1, "one node per thread");
+        if (!flat_node(L, x0, y, z)) return;
+    } else {
+        y = by * blockDim.y + threadIdx.y;
+        z = DIM == 3 ? bz : 0;
+        if (y >= L.ny) return;  // uniform across the warp
+        x0 = (bx * blockDim.x + threadIdx.x) * VEC;
+        if (x0 - lane * VEC >= L.nx) return;  // the whole warp lies past the row end
+    }
+    const int x0ld = FLAT ? x0 : min(x0, p.xmax_load);
     const C scale = ScaleOf<C>::s(p);
     const C inv_scale = ScaleOf<C>::inv(p);
     const long long row = L.row(y, z);
@@ -1377,6 +1402,12 @@ __device__ __forceinline__ void step_block_aa(S* buf, const KParams& p, int bx, 
         if (x0 >= L.nx) return;
     }
     wall_writes<DIM, S, VEC, C, KS, MODE>(buf, p, x0, y, z, f, g, salt);
+}
+
+template <int DIM, class S, int MODE>
+__global__ void __launch_bounds__(FLAT_THREADS) step_flat_kernel(const S* src, S* dst, const KParams p) {
+    if constexpr (MODE == PULL) step_block<DIM, S, 1, true, false, true>(src, dst, p, blockIdx.x, 0, 0);
+    else step_block_aa<DIM, S, 1, true, MODE, true>(dst, p, blockIdx.x, 0, 0);
 }
 
 template <int DIM, class S, int VEC, bool TRT, int MODE>

@@ -138,3 +138,23 @@ def test_reductions_of_a_batch_equal_those_of_its_cells(T, lattice, prec, n):  #
         b.nusselt()
     assert ei.value.code == T.TLBM_ERR_DIVERGED and f"instance {n - 1} " in str(ei.value)
     b.close()
+
+
+@pytest.mark.parametrize("lattice,shape,walls,pm", [
+    (D2, (3, 3, 1), 0, 0), (D2, (31, 5, 1), 1, 0), (D2, (33, 4, 1), 0, 1), (D2, (129, 9, 1), 0, 2),
+    (D3, (3, 3, 3), 0, 0), (D3, (33, 4, 5), 0, 0), (D3, (65, 3, 4), 1, 5), (D3, (7, 5, 6), 0, 6)])
+@pytest.mark.parametrize("inplace", [False, True])
+def test_fp64_threads_in_memory_order_equal_rows(T, lattice, shape, walls, pm, inplace):  # noqa: F811
+    """The FP64 default (one thread per node in memory order, warps over row and
+    plane ends) steps bitwise as the kernels with warps inside a row."""
+    out = []
+    for rows in (False, True):
+        s = T.Sim(*shape, lattice=lattice, Ra=1e5, Pr=0.71, Ma=0.1, precision=FP64, walls=walls, periodic_mask=pm,
+                  streaming=T.TLBM_STREAM_INPLACE if inplace else T.TLBM_STREAM_PULL)
+        if rows:
+            s.set_variant(2 if lattice == D2 else 1, 2, 32, 1, 1)
+        s.init(3, 1e-2)
+        s.step(7)
+        out.append(s.get_populations())
+        s.close()
+    assert np.array_equal(out[0][0], out[1][0]) and np.array_equal(out[0][1], out[1][1])
