@@ -162,11 +162,14 @@ TLBM_API int tlbm_init_fields(tlbm_t h, const float* T, const float* ux, const f
 
 /* Advance n >= 0 time steps (Eqs. (10)-(11), fused).  Asynchronous.  Whole
  * blocks of graph_steps steps (tlbm_set_graph, default 16) are replayed from a
- * CUDA graph captured at the first such block; the rest are plain launches. */
+ * CUDA graph captured at the first such block; the rest are plain launches.
+ * Unless tlbm_set_variant, tlbm_set_staged or tlbm_set_graph was called, calls
+ * of 16 steps or more may advance several steps per launch (2D cells whose size
+ * and storage gain by it): the same bits, fewer kernels (tlbm_launch_count). */
 TLBM_API int tlbm_step(tlbm_t h, int64_t n);
 
 /* Steps per CUDA graph replay in tlbm_step (even, <= 4096; 0 = plain launches
- * only).  The graph is captured on a private stream the first time it is needed
+ * only), one launch per step from then on.  The graph is captured on a private stream the first time it is needed
  * and dropped when the variant, the staged setting or the bound memory change. */
 TLBM_API int tlbm_set_graph(tlbm_t h, int steps);
 

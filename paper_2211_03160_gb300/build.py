@@ -32,6 +32,7 @@ UNITS = {
     "step_3d_f32.cu": [],
     "step_3d_f16.cu": [],
     "step_fp64.cu": ["--fmad=false"],
+    "step_multi.cu": [],
     "noalloc.cu": [],
     "step_staged.cu": [],
     "batch.cu": [],

@@ -49,6 +49,7 @@ static int cuda_fail(tlbm_t h, cudaError_t e, const char* what) {
 
 static void drop_graph(tlbm_t h);
 static int set_staged(tlbm_t h, int tile_width, int stages);
+static void pick_multi(tlbm_t h);
 
 // The buffer (two-buffer pull) or the order (in place: 0 natural, 1 swapped)
 // of the current state, and the matching state order for the diagnostic and
@@ -632,6 +633,7 @@ extern "C" int tlbm_bind_memory(tlbm_t h, void* dev_ptr, size_t bytes) {
         h->staged = 0;
         h->err[0] = 0;
     }
+    pick_multi(h);
     return TLBM_OK;
 }
 
@@ -709,8 +711,21 @@ static void drop_graph(tlbm_t h) {
     }
 }
 
-// Capture graph_steps steps starting from buffer 0 into a CUDA graph (on a
-// private stream; the graph is replayed on the handle's stream).
+// Calls of at least this many steps advance several steps per launch where the
+// handle does that at all (shorter calls keep one launch per step).
+constexpr int MULTI_CALL = 16;
+constexpr int MULTI_GRAPH = 8;  // launches of a graph block (even: it ends in the buffer it began in)
+
+// Launch `steps` <= h->multi steps reading buffer `parity` and writing the other.
+static cudaError_t launch_multi_raw(tlbm_t h, int parity, int steps, cudaStream_t s) {
+    MultiGeo g = h->mg;
+    g.steps = steps;
+    return launch_multi(h->prec, h->buf[parity], h->buf[parity ^ 1], h->kp, g, s);
+}
+
+// Capture a block of launches starting from buffer 0 into a CUDA graph (on a
+// private stream; the graph is replayed on the handle's stream): graph_steps
+// single steps, or MULTI_GRAPH launches of several steps.
 static int build_graph(tlbm_t h) {
     drop_graph(h);
     cudaError_t e = cudaSuccess;
@@ -719,7 +734,9 @@ static int build_graph(tlbm_t h) {
     e = cudaStreamBeginCapture(h->capture_stream, cudaStreamCaptureModeThreadLocal);
     if (e != cudaSuccess) return cuda_fail(h, e, "cudaStreamBeginCapture");
     cudaError_t le = cudaSuccess;
-    for (int k = 0; k < h->graph_steps && le == cudaSuccess; ++k) le = launch_step_raw(h, k & 1, h->capture_stream);
+    const int count = h->multi ? MULTI_GRAPH : h->graph_steps;
+    for (int k = 0; k < count && le == cudaSuccess; ++k)
+        le = h->multi ? launch_multi_raw(h, k & 1, h->multi, h->capture_stream) : launch_step_raw(h, k & 1, h->capture_stream);
     cudaGraph_t g = nullptr;
     e = cudaStreamEndCapture(h->capture_stream, &g);
     if (le != cudaSuccess || e != cudaSuccess) {
@@ -745,12 +762,41 @@ static cudaError_t launch_one_step(tlbm_t h) {
     return e;
 }
 
+// n steps, several per launch: graph blocks, then single launches, the last one
+// of fewer steps.
+static int step_multi(tlbm_t h, int64_t n) {
+    const int k = h->multi;
+    while (n > 0) {
+        if (h->cur == 0 && n >= (int64_t)k * MULTI_GRAPH) {
+            if (!h->graph) {
+                int rc = build_graph(h);
+                if (rc != TLBM_OK) return rc;
+            }
+            cudaError_t e = cudaGraphLaunch(h->graph, h->stream);
+            if (e != cudaSuccess) return cuda_fail(h, e, "cudaGraphLaunch");
+            h->t += (int64_t)k * MULTI_GRAPH;
+            h->launches += MULTI_GRAPH;
+            n -= (int64_t)k * MULTI_GRAPH;
+        } else {
+            const int now = (int)std::min<int64_t>(n, k);
+            cudaError_t e = launch_multi_raw(h, h->cur, now, h->stream);
+            if (e != cudaSuccess) return cuda_fail(h, e, "step kernel");
+            set_cur(h, h->cur ^ 1);
+            h->t += now;
+            h->launches += 1;
+            n -= now;
+        }
+    }
+    return TLBM_OK;
+}
+
 extern "C" int tlbm_step(tlbm_t h, int64_t n) {
     TLBM_CHECK_HANDLE(h);
     TLBM_CHECK_BOUND(h);
     if (n < 0) return fail(h, TLBM_ERR_ARG, "n must be >= 0");
+    if (h->multi && n >= MULTI_CALL) return step_multi(h, n);
     while (n > 0) {
-        if (h->graph_steps >= 2 && h->cur == 0 && n >= h->graph_steps) {
+        if (!h->multi && h->graph_steps >= 2 && h->cur == 0 && n >= h->graph_steps) {
             if (!h->graph) {
                 int rc = build_graph(h);
                 if (rc != TLBM_OK) return rc;
@@ -774,6 +820,8 @@ extern "C" int tlbm_set_graph(tlbm_t h, int steps) {
     if (steps < 0 || steps % 2 || steps > 4096) return fail(h, TLBM_ERR_ARG, "steps must be even, in [0, 4096]");
     drop_graph(h);
     h->graph_steps = steps;
+    h->graph_chosen = 1;  // the caller chose how single steps are launched
+    h->multi = 0;
     return TLBM_OK;
 }
 
@@ -1161,6 +1209,7 @@ extern "C" int tlbm_set_variant(tlbm_t h, int vec, int form, int block_x, int bl
     h->rows = nr;
     h->staged = 0;
     h->flat = 0;
+    h->multi = 0;
     h->variant_chosen = 1;
     h->kp.xmax_load = h->kp.L.P - v;
     drop_graph(h);
@@ -1240,10 +1289,30 @@ static int set_staged(tlbm_t h, int tile_width, int stages) {
     return TLBM_OK;
 }
 
+// Several steps per launch: 2D two-buffer cells with two-relaxation-time rates
+// whose launches the caller has not chosen, up to the size where one step fills
+// the GPU.  FP32, FP16 and BF16: 300,000 nodes (a 513^2 cell gains 1.5x, a 1025^2
+// one 1.1x in FP32 and loses a quarter in FP16), the 16-bit ones not with rows of
+// over 2048 nodes, which suit the staged kernel's tiles (4000 x 70: 8.5 us per
+// step staged, 8.8 here); FP64, bound by its pipe, 30,000 (129^2 8.1 -> 7.8 us
+// against one thread per node, 193^2 12.2 both ways).
+static void pick_multi(tlbm_t h) {
+    h->multi = 0;
+    if (h->dim != 2 || h->aa || !h->kp.trt || h->variant_chosen || h->graph_chosen) return;
+    if ((long long)h->nx * h->ny > (h->prec == TLBM_FP64 ? 30000 : 300000)) return;
+    if (h->elem == 2 && h->nx > 2048) return;
+    // a region wraps around a periodic axis at most once
+    if (((h->kp.periodic & 1) && h->nx < 16) || ((h->kp.periodic & 2) && h->ny < 16)) return;
+    if (multi_setup(h->prec, h->kp, h->mg)) h->multi = h->mg.m + 1;
+}
+
 extern "C" int tlbm_set_staged(tlbm_t h, int tile_width, int stages) {
     TLBM_CHECK_HANDLE(h);
     const int rc = set_staged(h, tile_width, stages);
-    if (rc == TLBM_OK) h->variant_chosen = 1;
+    if (rc == TLBM_OK) {
+        h->variant_chosen = 1;
+        h->multi = 0;
+    }
     return rc;
 }
 

@@ -31,6 +31,18 @@ const void* staged_function(int dim, int prec, int nc);
 cudaError_t launch_staged(int dim, int prec, int nc, const void* src, void* dst, const KParams& p,
                           const StagedInfo& si, int grid, size_t smem, cudaStream_t s);
 
+// several steps of a 2D cell per launch (step_multi.cu), TRT form
+struct MultiGeo {
+    int tw, th;  // nodes of a block's tile
+    int m;       // nodes its region has around the tile: most steps per launch - 1
+    int W, H;    // region: W >= tw + 2 m columns, H = th + 2 m rows
+    int RS;      // elements of a region row in shared memory
+    int steps;   // steps of this launch, 1 <= steps <= m + 1
+};
+// choose the tile and the steps per launch for a cell; false if the kernel cannot be used
+bool multi_setup(int prec, const KParams& p, MultiGeo& g);
+cudaError_t launch_multi(int prec, const void* src, void* dst, const KParams& p, const MultiGeo& g, cudaStream_t s);
+
 // per-unit entry points
 cudaError_t launch_step_2d_f32(int vec, bool trt, int rows, const void*, void*, const KParams&, dim3, dim3,
                                cudaStream_t);

@@ -4,7 +4,7 @@
 #include <stdint.h>
 
 #include "../../include/tlbm.h"
-#include "kernels.cuh"
+#include "dispatch.h"
 
 struct tlbm_s {
     int nx, ny, nz, dim, lattice, prec;
@@ -18,9 +18,12 @@ struct tlbm_s {
     int rows;                  // consecutive rows per thread (software-pipelined when > 1)
     int aa;                    // 1: in-place (AA) streaming in one population buffer
     int nbuf;                  // population buffers: 2, or 1 in place
+    int graph_chosen;          // set by tlbm_set_graph: launch single steps as the caller asked
     int graph_steps;           // steps per CUDA graph replay in tlbm_step (0: plain launches)
     cudaGraphExec_t graph;     // captured block of graph_steps steps starting from buffer 0
     cudaStream_t capture_stream;
+    int multi;                 // > 1: most steps per launch of calls of MULTI_CALL steps or more (step_multi.cu)
+    tlbm::MultiGeo mg;         // tile of that kernel
     int flat;                  // 1: FP64 kernel with one thread per node in memory order
     int staged;                // 1: shared-memory staged (TMA bulk copy) kernel
     int variant_chosen;        // set by tlbm_set_variant / tlbm_set_staged: keep the caller's choice

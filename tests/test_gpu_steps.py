@@ -158,3 +158,95 @@ def test_fp64_threads_in_memory_order_equal_rows(T, lattice, shape, walls, pm, i
         out.append(s.get_populations())
         s.close()
     assert np.array_equal(out[0][0], out[1][0]) and np.array_equal(out[0][1], out[1][1])
+
+
+@pytest.mark.parametrize("prec", [0, 1, 2, 3])
+@pytest.mark.parametrize("shape,walls,pm", [((16, 16), 0, 0), ((17, 33), 0, 0), ((65, 31), 1, 0), ((3, 9), 0, 0),
+                                            ((130, 67), 0, 1), ((53, 18), 0, 2), ((29, 29), 0, 3), ((129, 129), 0, 0),
+                                            ((270, 40), 1, 2)])
+def test_several_steps_per_launch_equal_single_steps(T, prec, shape, walls, pm):  # noqa: F811
+    """Small 2D cells advance several steps per launch in calls of 16 steps or
+    more: bitwise the states, counters and diagnostics of one-step launches, for
+    step counts that are no multiple of a launch's or a graph block's, on walls
+    and periodic faces, and from either buffer."""
+    kw = dict(Ra=1e5, Pr=0.71, Ma=0.1, precision=prec, walls=walls, periodic_mask=pm)
+    a, b = T.Sim(*shape, **kw), T.Sim(*shape, **kw)
+    T.tlbm_set_graph(b.h, 0)  # one launch per step
+    for s in (a, b):
+        s.init(3, 1e-2)
+    for n in (17, 1, 16, 139):
+        la = a.launches
+        a.step(n)
+        b.step(n)
+        assert n < 16 or a.launches - la <= (n + 1) // 2
+        (fa, ga), (fb, gb) = a.get_populations(), b.get_populations()
+        assert np.array_equal(fa, fb) and np.array_equal(ga, gb), n
+        assert a.status() == b.status() and a.nusselt() == b.nusselt()
+    a.close()
+    b.close()
+
+
+@pytest.mark.parametrize("choice,n", [("variant", 40), ("staged", 40), ("graph", 40), ("none", 15)])
+def test_launch_choices_of_the_caller_stay(T, choice, n):  # noqa: F811
+    """A handle whose step variant, staged kernel or graph the caller chose keeps
+    one launch per step; so do short calls."""
+    s = T.Sim(65, 40, Ra=1e5, Pr=0.71, Ma=0.1, precision=1)
+    if choice == "variant":
+        s.set_variant(2, 2, 0, 0, 1)
+    elif choice == "staged":
+        s.set_staged()
+    elif choice == "graph":
+        T.tlbm_set_graph(s.h, 16)
+    s.init(1, 1e-3)
+    c0 = s.launches
+    s.step(n)
+    assert s.launches - c0 == n
+    s.close()
+
+
+BOUNDS_SCRIPT = """
+import hashlib, json, sys
+sys.path.insert(0, {root!r})
+from paper_2211_03160_gb300 import tlbm as T
+out = {{}}
+for lattice, shape, walls, pm, prec, inplace, steps in {cases!r}:
+    s = T.Sim(*shape, lattice=lattice, Ra=1e5, Pr=0.71, Ma=0.1, precision=prec, walls=walls, periodic_mask=pm,
+              streaming=1 if inplace else 0)
+    s.init(5, 1e-2)
+    s.step(steps)
+    m = s.macros()
+    f, g = s.get_populations()
+    h = hashlib.sha256(f.tobytes() + g.tobytes() + m["T"].cpu().numpy().tobytes()).hexdigest()
+    try:
+        bad = T.tlbm_bounds_violations(s.h)
+    except T.TlbmError:
+        bad = None
+    out[repr((lattice, shape, walls, pm, prec, inplace))] = [h, s.nusselt(), bad]
+    s.close()
+print("RESULT " + json.dumps(out))
+"""
+
+
+def test_default_kernels_stay_inside_their_buffers(T):  # noqa: F811
+    """The kernels a default handle runs in calls of 16 steps and more, on the
+    bounds-checked build: no access leaves the population buffers, and states,
+    fields and reductions are those of the release build."""
+    import json
+    import os
+    import subprocess
+    import sys
+
+    root = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+    cases = [(D2, (nx, ny, 1), walls, pm, prec, False, 37) for nx, ny, walls, pm in
+             ((3, 9, 0, 0), (37, 16, 1, 0), (130, 21, 0, 1), (33, 70, 0, 3), (700, 500, 0, 0)) for prec in (0, 1, 2)]
+    cases += [(D3, (35, 6, 5), 0, 4, 0, inplace, 17) for inplace in (False, True)]
+    script = BOUNDS_SCRIPT.format(root=root, cases=cases)
+    res = []
+    for debug in ("0", "1"):
+        r = subprocess.run([sys.executable, "-c", script], env=dict(os.environ, TLBM_DEBUG_BOUNDS=debug),
+                           capture_output=True, text=True, timeout=900)
+        assert r.returncode == 0, r.stderr[-2000:]
+        res.append(json.loads(r.stdout.split("RESULT ")[1]))
+    for k in res[0]:
+        assert res[1][k][2] == 0, k
+        assert res[0][k][:2] == res[1][k][:2], k
