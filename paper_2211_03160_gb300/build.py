@@ -33,6 +33,7 @@ UNITS = {
     "step_3d_f16.cu": [],
     "step_fp64.cu": ["--fmad=false"],
     "step_multi.cu": [],
+    "step_march.cu": [],
     "noalloc.cu": [],
     "step_staged.cu": [],
     "batch.cu": [],

@@ -716,8 +716,11 @@ static void drop_graph(tlbm_t h) {
 constexpr int MULTI_CALL = 16;
 constexpr int MULTI_GRAPH = 8;  // launches of a graph block (even: it ends in the buffer it began in)
 
-// Launch `steps` <= h->multi steps reading buffer `parity` and writing the other.
+// Launch `steps` <= h->multi steps (with march: h->multi or 1) reading buffer
+// `parity` and writing the other.
 static cudaError_t launch_multi_raw(tlbm_t h, int parity, int steps, cudaStream_t s) {
+    if (h->march && steps == 1) return launch_step_raw(h, parity, s);
+    if (h->march) return launch_march(h->buf[parity], h->buf[parity ^ 1], h->kp, h->march, s);
     MultiGeo g = h->mg;
     g.steps = steps;
     return launch_multi(h->prec, h->buf[parity], h->buf[parity ^ 1], h->kp, g, s);
@@ -762,7 +765,7 @@ static cudaError_t launch_one_step(tlbm_t h) {
     return e;
 }
 
-// n steps, several per launch: graph blocks, then single launches, the last one
+// n steps, several per launch: graph blocks, then single launches, the last ones
 // of fewer steps.
 static int step_multi(tlbm_t h, int64_t n) {
     const int k = h->multi;
@@ -778,7 +781,7 @@ static int step_multi(tlbm_t h, int64_t n) {
             h->launches += MULTI_GRAPH;
             n -= (int64_t)k * MULTI_GRAPH;
         } else {
-            const int now = (int)std::min<int64_t>(n, k);
+            const int now = n >= k ? k : (h->march ? 1 : (int)n);
             cudaError_t e = launch_multi_raw(h, h->cur, now, h->stream);
             if (e != cudaSuccess) return cuda_fail(h, e, "step kernel");
             set_cur(h, h->cur ^ 1);
@@ -1290,16 +1293,26 @@ static int set_staged(tlbm_t h, int tile_width, int stages) {
 }
 
 // Several steps per launch: 2D two-buffer cells with two-relaxation-time rates
-// whose launches the caller has not chosen, up to the size where one step fills
-// the GPU.  FP32, FP16 and BF16: 300,000 nodes (a 513^2 cell gains 1.5x, a 1025^2
+// whose launches the caller has not chosen.  FP32 cells with walls all around go
+// through step_march.cu from 250,000 nodes (513^2: 6.7 us per step against 7.1
+// in tiles and 10.5 singly) unless their width would leave more than a quarter
+// of its strips' columns idle.  Else tiles (step_multi.cu) up to the size where
+// one step fills the GPU.  FP32, FP16 and BF16: 300,000 nodes (a 513^2 cell gains 1.5x, a 1025^2
 // one 1.1x in FP32 and loses a quarter in FP16), the 16-bit ones not with rows of
 // over 2048 nodes, which suit the staged kernel's tiles (4000 x 70: 8.5 us per
 // step staged, 8.8 here); FP64, bound by its pipe, 30,000 (129^2 8.1 -> 7.8 us
 // against one thread per node, 193^2 12.2 both ways).
 static void pick_multi(tlbm_t h) {
-    h->multi = 0;
+    h->multi = h->march = 0;
     if (h->dim != 2 || h->aa || !h->kp.trt || h->variant_chosen || h->graph_chosen) return;
-    if ((long long)h->nx * h->ny > (h->prec == TLBM_FP64 ? 30000 : 300000)) return;
+    const long long nodes = (long long)h->nx * h->ny;
+    const int strips = (h->nx + MARCH_COLUMNS - 1) / MARCH_COLUMNS;
+    if (h->prec == TLBM_FP32 && !h->kp.periodic && nodes >= 250000 && 4 * h->nx >= 3 * strips * MARCH_COLUMNS) {
+        h->march = march_rows(h->kp);
+        if (h->march) h->multi = MARCH_STEPS;
+        return;
+    }
+    if (nodes > (h->prec == TLBM_FP64 ? 30000 : 300000)) return;
     if (h->elem == 2 && h->nx > 2048) return;
     // a region wraps around a periodic axis at most once
     if (((h->kp.periodic & 1) && h->nx < 16) || ((h->kp.periodic & 2) && h->ny < 16)) return;

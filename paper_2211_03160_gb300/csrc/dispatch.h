@@ -43,6 +43,13 @@ struct MultiGeo {
 bool multi_setup(int prec, const KParams& p, MultiGeo& g);
 cudaError_t launch_multi(int prec, const void* src, void* dst, const KParams& p, const MultiGeo& g, cudaStream_t s);
 
+// MARCH_STEPS steps of a 2D FP32 cell with walls on every side in one pass over
+// memory, in segments of `rows` rows (step_march.cu), TRT form
+constexpr int MARCH_STEPS = 3;
+constexpr int MARCH_COLUMNS = 56;  // columns a warp stores
+int march_rows(const KParams& p);  // rows of a segment, 0: the device cannot be asked
+cudaError_t launch_march(const void* src, void* dst, const KParams& p, int rows, cudaStream_t s);
+
 // per-unit entry points
 cudaError_t launch_step_2d_f32(int vec, bool trt, int rows, const void*, void*, const KParams&, dim3, dim3,
                                cudaStream_t);

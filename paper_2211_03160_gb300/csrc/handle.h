@@ -22,8 +22,9 @@ struct tlbm_s {
     int graph_steps;           // steps per CUDA graph replay in tlbm_step (0: plain launches)
     cudaGraphExec_t graph;     // captured block of graph_steps steps starting from buffer 0
     cudaStream_t capture_stream;
-    int multi;                 // > 1: most steps per launch of calls of MULTI_CALL steps or more (step_multi.cu)
-    tlbm::MultiGeo mg;         // tile of that kernel
+    int multi;                 // > 1: steps per launch of calls of MULTI_CALL steps or more
+    int march;                 // > 0: by step_march.cu in segments of this many rows, else by step_multi.cu
+    tlbm::MultiGeo mg;         // tile of the latter
     int flat;                  // 1: FP64 kernel with one thread per node in memory order
     int staged;                // 1: shared-memory staged (TMA bulk copy) kernel
     int variant_chosen;        // set by tlbm_set_variant / tlbm_set_staged: keep the caller's choice

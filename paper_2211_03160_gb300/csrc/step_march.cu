@@ -1,0 +1,291 @@
+// Three time steps of a 2D cell in one pass over memory, FP32 storage
+// (two-relaxation-time collision, two-buffer streaming, walls on every side).
+//
+// A one-step kernel of a large cell reads and writes the state once per step and
+// is bound by HBM (62 GLUPS at 8193^2, 102 % of the copy rate).  Here a warp owns
+// a strip of MARCH_OUT = 56 columns and marches up a segment of rows: it pulls
+// row r from memory (two nodes per lane, 64 columns) and collides it (step 1);
+// from the post-collision values of rows r - 2, r - 1 and r, which it holds in
+// registers, it pulls and collides row r - 1 again (step 2), in the same way row
+// r - 2 a third time (step 3), and stores that.  The state is read and written
+// once per three steps.  The values a node needs from the columns next to it
+// come by shuffles.  A strip's outer columns are stepped by its neighbours as
+// well (64 / 56 redundant updates), and a segment steps two extra rows at either
+// end.  No barrier: every warp is on its own.  The rows on their way from memory
+// go through shared memory (asynchronous copies of each lane's own pairs): held
+// in registers instead they spilled, and a spilled load waits for its data.
+//
+// Of a row's post-collision values only those are kept that a later row pulls:
+// the populations with e_y = 0 for one row, those with e_y = +1 for two; those
+// with e_y = -1 are pulled at once (28 registers a lane and step).  Wall rules of
+// the inner steps: a node's half-way bounce-back value is its own post-collision
+// value of the opposite population, so it is put in place of the shuffled one
+// at the side walls, and in place of the missing row's values at the bottom and
+// top.
+//
+// What bounds it now: instruction issue and latency at twelve warps an SM (158
+// registers a thread); HBM moves 37 of the 112 bytes per update.  GLUPS on GB300
+// by steps per pass (blocks of four warps per SM) at 8193^2: 2 (3) 111, 3 (3)
+// 132, 3 (4, spilling) 80, 4 (2) 124; 2 (5, at 96 registers) 75.  us per step,
+// one-step kernel -> this: 513^2 10.4 -> 6.7, 1025^2 24.7 -> 13.4, 2049^2 77.1 ->
+// 41.1, 4097^2 280 -> 140, 8193^2 1081 -> 500 (134 GLUPS).
+//
+// Every node gets bitwise the values of the one-step kernels.
+#include <algorithm>
+
+#include "dispatch.h"
+
+namespace tlbm {
+
+namespace {
+
+constexpr int MARCH_W = 64;       // columns a warp steps
+constexpr int MARCH_SIDE = 4;     // columns a side that it does not store: >= MARCH_STEPS, even (aligned pairs)
+constexpr int MARCH_OUT = MARCH_W - 2 * MARCH_SIDE;
+static_assert(MARCH_OUT == MARCH_COLUMNS, "columns a warp stores");
+constexpr int MARCH_WARPS = 4;    // warps of a block
+constexpr int MARCH_BLOCKS = 3;   // blocks per SM
+constexpr int MARCH_AHEAD = 1;    // rows whose copies are in flight
+
+// value of column x - EX for the lane's two columns
+template <int EX>
+__device__ __forceinline__ float2 march_shift(float2 v) {
+    if constexpr (EX == 1) return make_float2(__shfl_up_sync(0xffffffffu, v.y, 1), v.x);
+    else if constexpr (EX == -1) return make_float2(v.y, __shfl_down_sync(0xffffffffu, v.x, 1));
+    else return v;
+}
+
+// the thermal wall rule: anti-bounce-back at a wall of temperature Tw, bounce-back at an adiabatic one
+__device__ __forceinline__ float march_rule(float v, bool iso, const KParams& p, float Tw) {
+    return iso ? -v + p.omegaf * Tw : v;
+}
+
+// copy the stored pairs a lane pulls for one row (before the shift along x) to
+// the lane's places in shared memory, as one group of its asynchronous copies
+__device__ __forceinline__ void march_fetch(const float* __restrict__ own, const KParams& p, uint32_t to) {
+#pragma unroll
+    for (int j = 0; j < 14; ++j)
+        asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"(to + j * MARCH_W * 4),
+                     "l"(TLBM_DBG(p, (own + p.loff[j]), 0, 2))
+                     : "memory");
+}
+
+// What a strip keeps of one step's post-collision values: e_y = 0 of the last
+// row (flow 0, 1, 3, thermal 0, 1, 3), e_y = +1 (flow 2, 5, 6, thermal 2) of the
+// last row and of the one before; wd: at a side wall, the last row's diagonal
+// with e_y = -1 that meets it.
+struct MarchKept {
+    float2 z[6], u1[4], u0[4];
+    float wd;
+};
+
+// f, g: the post-collision values of row r, or anything if r = ny.  Keeps what
+// later rows pull of them and turns f, g into what row r - 1 pulls.
+template <int DIM>
+__device__ __forceinline__ void march_pull(MarchKept& k, float2 (&f)[9], float2 (&g)[5], const KParams& p, int r, int x,
+                                           bool wall_strip, bool heat_y) {
+    const Layout& L = p.L;
+    float2 f4, f7, f8, g4;
+    if (r < L.ny) {
+        f4 = f[4];
+        f7 = march_shift<-1>(f[7]);
+        f8 = march_shift<1>(f[8]);
+        g4 = g[4];
+    } else {
+        // past the top wall: what row ny - 1 pulls from there is its own
+        f4 = k.u1[0];
+        f7 = k.u1[1];
+        f8 = k.u1[2];
+        g4 = make_float2(march_rule(k.u1[3].x, heat_y, p, p.Tcf), march_rule(k.u1[3].y, heat_y, p, p.Tcf));
+    }
+    const float2 f5 = march_shift<1>(k.u0[1]), f6 = march_shift<-1>(k.u0[2]);
+    const float2 f1 = march_shift<1>(k.z[1]), f3 = march_shift<-1>(k.z[2]);
+    const float2 g1 = march_shift<1>(k.z[4]), g3 = march_shift<-1>(k.z[5]);
+    const float2 f0 = k.z[0], f2 = k.u0[0], g0 = k.z[3], g2 = k.u0[3];
+    const float2 w1 = k.z[1], w3 = k.z[2], w5 = k.u1[1], w6 = k.u1[2], v1 = k.z[4], v3 = k.z[5];
+    const float wd = k.wd;
+    // keep row r
+#pragma unroll
+    for (int q = 0; q < 4; ++q) k.u0[q] = k.u1[q];
+    k.u1[0] = f[2];
+    k.u1[1] = f[5];
+    k.u1[2] = f[6];
+    k.u1[3] = g[2];
+    k.z[0] = f[0];
+    k.z[1] = f[1];
+    k.z[2] = f[3];
+    k.z[3] = g[0];
+    k.z[4] = g[1];
+    k.z[5] = g[3];
+    if (r == 0) {
+        // below the bottom wall: what row 0 pulls from there is its own
+        // (shifted back, as the next pull shifts it)
+        k.u0[0] = f[4];
+        k.u0[1] = march_shift<-1>(f[7]);
+        k.u0[2] = march_shift<1>(f[8]);
+        k.u0[3] = make_float2(march_rule(g[4].x, heat_y, p, p.Thf), march_rule(g[4].y, heat_y, p, p.Thf));
+    }
+    if (wall_strip) k.wd = x == 0 ? f[7].x : (x == L.nx - 1 ? f[8].x : f[8].y);
+    f[0] = f0;
+    f[1] = f1;
+    f[2] = f2;
+    f[3] = f3;
+    f[4] = f4;
+    f[5] = f5;
+    f[6] = f6;
+    f[7] = f7;
+    f[8] = f8;
+    g[0] = g0;
+    g[1] = g1;
+    g[2] = g2;
+    g[3] = g3;
+    g[4] = g4;
+    if (wall_strip) {
+        if (x == 0) {
+            f[1].x = w3.x;
+            f[5].x = wd;
+            f[8].x = w6.x;
+            g[1].x = march_rule(v3.x, !heat_y, p, p.Thf);
+        }
+        if (x == L.nx - 1) {
+            f[3].x = w1.x;
+            f[6].x = wd;
+            f[7].x = w5.x;
+            g[3].x = march_rule(v1.x, !heat_y, p, p.Tcf);
+        }
+        if (x + 1 == L.nx - 1) {
+            f[3].y = w1.y;
+            f[6].y = wd;
+            f[7].y = w5.y;
+            g[3].y = march_rule(v1.y, !heat_y, p, p.Tcf);
+        }
+    }
+}
+
+template <int DIM>
+__global__ void __launch_bounds__(32 * MARCH_WARPS, MARCH_BLOCKS)
+    step_march_kernel(const float* __restrict__ src, float* __restrict__ dst, const KParams p, int strips, int seg) {
+    static_assert(MARCH_SIDE >= MARCH_STEPS && MARCH_SIDE % 2 == 0, "valid columns");
+    using LF = typename Lat<DIM>::F;
+    using LG = typename Lat<DIM>::G;
+    constexpr int QF = LF::Q, QG = LG::Q, Q = QF + QG;
+    constexpr int LV = MARCH_STEPS, SIDE = MARCH_SIDE, OUT = MARCH_OUT;
+    const Layout& L = p.L;
+    const int lane = threadIdx.x & 31;
+    const int item = blockIdx.x * MARCH_WARPS + (threadIdx.x >> 5);
+    const int sg = item / strips, strip = item - sg * strips;
+    if (sg * seg >= p.L.ny) return;
+    const int x = strip * OUT - SIDE + 2 * lane;  // the lane's first column
+    const int y0 = sg * seg, y1 = min(y0 + seg, L.ny);
+    const bool wall_strip = strip == 0 || strip * OUT + OUT + SIDE >= L.nx;
+    const bool store = lane >= SIDE / 2 && lane < 32 - SIDE / 2 && x < L.nx;
+    const bool heat_y = p.heat_axis == 1;
+    const int xld = min(x, L.P - 2);
+
+    // rows on their way from memory: a ring of MARCH_AHEAD + 1 rows per warp,
+    // every lane's pairs in places of its own
+    __shared__ __align__(16) float ring[MARCH_WARPS][MARCH_AHEAD + 1][Q][MARCH_W];
+    constexpr int ROWB = Q * MARCH_W * 4;
+    float* mine = &ring[threadIdx.x >> 5][0][0][2 * lane];
+    const uint32_t mine_at = smem_addr(mine);
+    MarchKept kept[LV - 1];
+#pragma unroll
+    for (int l = 0; l < LV - 1; ++l) {
+        const float2 zero = make_float2(0.0f, 0.0f);
+        for (int k = 0; k < 6; ++k) kept[l].z[k] = zero;
+        for (int k = 0; k < 4; ++k) kept[l].u1[k] = kept[l].u0[k] = zero;
+        kept[l].wd = 0.0f;
+    }
+
+    const int r0 = max(y0 - (LV - 1), 0);
+    const int rl = min(y1 + LV - 2, L.ny - 1);  // last row to pull
+    const float* from = src + L.row(r0, 0) + xld;
+#pragma unroll
+    for (int k = 0; k < MARCH_AHEAD; ++k) {
+        if (r0 + k <= rl) march_fetch(from + (long long)k * L.P, p, mine_at + k * ROWB);
+        asm volatile("cp.async.commit_group;" ::: "memory");
+    }
+    from += (long long)MARCH_AHEAD * L.P;
+    int slot = 0, ahead = MARCH_AHEAD;
+    for (int r = r0; r <= y1 + LV - 2; ++r) {
+        float2 f[QF], g[QG];
+        if (r < L.ny) {
+            if (r + MARCH_AHEAD <= rl) march_fetch(from, p, mine_at + ahead * ROWB);
+            asm volatile("cp.async.commit_group;" ::: "memory");
+            asm volatile("cp.async.wait_group %0;" ::"n"(MARCH_AHEAD) : "memory");
+            from += L.P;
+            const float* row = mine + slot * (Q * MARCH_W);
+            slot = slot == MARCH_AHEAD ? 0 : slot + 1;
+            ahead = ahead == MARCH_AHEAD ? 0 : ahead + 1;
+            static_for<QF>([&](auto ii) {
+                constexpr int i = decltype(ii)::value;
+                f[i] = march_shift<LF::e(i, 0)>(*reinterpret_cast<const float2*>(row + i * MARCH_W));
+            });
+            static_for<QG>([&](auto ii) {
+                constexpr int i = decltype(ii)::value;
+                g[i] = march_shift<LG::e(i, 0)>(*reinterpret_cast<const float2*>(row + (QF + i) * MARCH_W));
+            });
+            collide_trt_v<DIM, float2, false, true>(f, g, p);
+        }
+        // step l + 2 of row r - 1 - l; rows past the top wall hold anything, and
+        // so do rows too close to the segment's first one
+#pragma unroll
+        for (int l = 0; l < LV - 1; ++l) {
+            march_pull<DIM>(kept[l], f, g, p, r - l, x, wall_strip, heat_y);
+            if (r - l > r0) collide_trt_v<DIM, float2, false, true>(f, g, p);
+        }
+        const int y = r - (LV - 1);
+        if (y < y0 || !store) continue;
+        float* own = dst + L.row(y, 0) + x;
+        if (x + 1 < L.nx) {
+            static_for<Q>([&](auto jj) {
+                constexpr int j = decltype(jj)::value;
+                __stwb(reinterpret_cast<float2*>(TLBM_DBG(p, (own + p.soff[j]), 0, 2)),
+                       j < QF ? f[j < QF ? j : 0] : g[j < QF ? 0 : j - QF]);
+            });
+        } else {
+            static_for<Q>([&](auto jj) {
+                constexpr int j = decltype(jj)::value;
+                *TLBM_DBG(p, (own + p.soff[j]), 0, 1) = j < QF ? f[j < QF ? j : 0].x : g[j < QF ? 0 : j - QF].x;
+            });
+        }
+        if (y == 0 || y == L.ny - 1 || x == 0 || x + 2 >= L.nx) {
+            float fw[QF][2], gw[QG][2];
+#pragma unroll
+            for (int i = 0; i < QF; ++i) { fw[i][0] = f[i].x; fw[i][1] = f[i].y; }
+#pragma unroll
+            for (int i = 0; i < QG; ++i) { gw[i][0] = g[i].x; gw[i][1] = g[i].y; }
+            wall_writes<2, float, 2, float, true>(dst, p, x, y, 0, fw, gw, 0u);
+        }
+    }
+}
+
+}  // namespace
+
+// Rows of a segment.  Every segment costs 2 (MARCH_STEPS - 1) rows more than it
+// stores, so as few segments as fill the GPU: one round of resident warps where
+// that gives segments of up to 64 rows, else the fewest whole rounds that do
+// (longer segments end too unevenly).  us per step at 2049^2 with 42 rows (one
+// round) 42.0, 21 (two) 42.7, 48 47.2; at 8193^2 with 61 500, 84 509, 168 520,
+// 683 621.
+int march_rows(const KParams& p) {
+    int dev = 0, sms = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess ||
+        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
+        return 0;
+    const int strips = (p.L.nx + MARCH_OUT - 1) / MARCH_OUT, resident = sms * MARCH_BLOCKS * MARCH_WARPS;
+    for (int rounds = 1;; ++rounds) {
+        const long long segs = std::max<long long>(1, (long long)rounds * resident / strips);
+        const int rows = (int)((p.L.ny + segs - 1) / segs);
+        if (rows <= 64) return rows;
+    }
+}
+
+cudaError_t launch_march(const void* src, void* dst, const KParams& p, int rows, cudaStream_t s) {
+    const int strips = (p.L.nx + MARCH_OUT - 1) / MARCH_OUT;
+    const int items = strips * ((p.L.ny + rows - 1) / rows), grid = (items + MARCH_WARPS - 1) / MARCH_WARPS;
+    step_march_kernel<2><<<grid, 32 * MARCH_WARPS, 0, s>>>((const float*)src, (float*)dst, p, strips, rows);
+    return cudaGetLastError();
+}
+
+}  // namespace tlbm

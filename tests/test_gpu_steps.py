@@ -186,6 +186,31 @@ def test_several_steps_per_launch_equal_single_steps(T, prec, shape, walls, pm):
     b.close()
 
 
+@pytest.mark.parametrize("shape,walls", [((560, 450), 0), ((561, 447), 1), ((562, 449), 0), ((614, 410), 0),
+                                         ((615, 409), 1), ((101, 2500), 0), ((8193, 31), 0), ((30000, 9), 1),
+                                         ((100000, 3), 0), ((513, 513), 0)])
+def test_three_steps_per_pass_equal_single_steps(T, shape, walls):  # noqa: F811
+    """Larger FP32 cells march three steps per pass over memory in strips of 56
+    columns: bitwise one-step launches at every remainder of the width by the
+    strip and of the step count by three, on both wall configurations, short
+    and long segments, and from either buffer."""
+    kw = dict(Ra=1e6, Pr=0.71, Ma=0.1, precision=1, walls=walls)
+    a, b = T.Sim(*shape, **kw), T.Sim(*shape, **kw)
+    T.tlbm_set_graph(b.h, 0)
+    for s in (a, b):
+        s.init(3, 1e-2)
+    for n in (16, 20, 1, 33):
+        la = a.launches
+        a.step(n)
+        b.step(n)
+        assert a.launches - la == n // 3 + n % 3 or n < 16
+        (fa, ga), (fb, gb) = a.get_populations(), b.get_populations()
+        assert np.array_equal(fa, fb) and np.array_equal(ga, gb), n
+        assert a.status() == b.status() and a.nusselt() == b.nusselt()
+    a.close()
+    b.close()
+
+
 @pytest.mark.parametrize("choice,n", [("variant", 40), ("staged", 40), ("graph", 40), ("none", 15)])
 def test_launch_choices_of_the_caller_stay(T, choice, n):  # noqa: F811
     """A handle whose step variant, staged kernel or graph the caller chose keeps
