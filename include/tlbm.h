@@ -303,7 +303,9 @@ TLBM_API int tlbm_batch_bind_memory(tlbm_batch_t b, void* dev_ptr, size_t bytes)
 TLBM_API int tlbm_batch_set_stream(tlbm_batch_t b, void* cuda_stream);
 /* tlbm_init of every instance with its own tlbm_instance.seed. */
 TLBM_API int tlbm_batch_init(tlbm_batch_t b, double noise_amp);
-/* Advance every instance by n steps.  Asynchronous. */
+/* Advance every instance by n steps.  Asynchronous.  Unless tlbm_batch_set_variant,
+ * _set_rows, _set_staged or _set_persistent was called, calls of 16 steps or more
+ * may advance several steps per launch, as in tlbm_step. */
 TLBM_API int tlbm_batch_step(tlbm_batch_t b, int64_t n);
 /* Launch shape of the batched kernel (0 keeps the current value; form as in
  * tlbm_set_variant) and the steps per graph launch (even; 0 = no graph). */

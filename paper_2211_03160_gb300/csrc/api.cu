@@ -711,9 +711,6 @@ static void drop_graph(tlbm_t h) {
     }
 }
 
-// Calls of at least this many steps advance several steps per launch where the
-// handle does that at all (shorter calls keep one launch per step).
-constexpr int MULTI_CALL = 16;
 constexpr int MULTI_GRAPH = 8;  // launches of a graph block (even: it ends in the buffer it began in)
 
 // Launch `steps` <= h->multi steps (with march: h->multi or 1) reading buffer
@@ -767,10 +764,16 @@ static cudaError_t launch_one_step(tlbm_t h) {
 
 // n steps, several per launch: graph blocks, then single launches, the last ones
 // of fewer steps.
+// The state ends in the buffer that n single steps would leave it in (readers of
+// the bound block and batches go by that): up to two single-step launches first
+// make the number of launches as odd as n (three steps a launch always are).
 static int step_multi(tlbm_t h, int64_t n) {
     const int k = h->multi;
+    int ones = 0;
+    if (!h->march)
+        while ((ones + (n - ones + k - 1) / k - n) % 2) ++ones;
     while (n > 0) {
-        if (h->cur == 0 && n >= (int64_t)k * MULTI_GRAPH) {
+        if (ones == 0 && h->cur == 0 && n >= (int64_t)k * MULTI_GRAPH) {
             if (!h->graph) {
                 int rc = build_graph(h);
                 if (rc != TLBM_OK) return rc;
@@ -781,7 +784,8 @@ static int step_multi(tlbm_t h, int64_t n) {
             h->launches += MULTI_GRAPH;
             n -= (int64_t)k * MULTI_GRAPH;
         } else {
-            const int now = n >= k ? k : (h->march ? 1 : (int)n);
+            const int now = ones > 0 ? 1 : (n >= k ? k : (h->march ? 1 : (int)n));
+            ones -= ones > 0;
             cudaError_t e = launch_multi_raw(h, h->cur, now, h->stream);
             if (e != cudaSuccess) return cuda_fail(h, e, "step kernel");
             set_cur(h, h->cur ^ 1);

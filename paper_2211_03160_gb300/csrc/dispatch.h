@@ -50,6 +50,28 @@ constexpr int MARCH_COLUMNS = 56;  // columns a warp stores
 int march_rows(const KParams& p);  // rows of a segment, 0: the device cannot be asked
 cudaError_t launch_march(const void* src, void* dst, const KParams& p, int rows, cudaStream_t s);
 
+// the same for the cells of a batch: what the kernel reads of a cell in its hot
+// path (members as in KParams), all of a launch's cells by value
+struct MarchCell {
+    Layout L;
+    int heat_axis, strips, block0;  // block0: its first block of the launch
+    float gbetaf, omegaf, Thf, Tcf, bodyf[3], spf, smf, shpf, shmf, qpf, qmf;
+    decltype(KParams::tf) tf;
+    int loff[14], soff[14];
+    float* buf[2];
+    const KParams* full;  // all parameters, in device memory
+};
+constexpr int MARCH_MANY = 64;  // most cells of a launch (kernel parameters hold 32 KB)
+struct MarchBatch {
+    MarchCell cell[MARCH_MANY];
+    int n, rows;
+};
+static_assert(sizeof(MarchBatch) <= 32000, "kernel parameters");
+MarchCell march_cell(const KParams& p, const void* buf0, const void* buf1, const KParams* full);
+int march_cell_blocks(const MarchCell& c, int rows);
+int march_batch_rows(const long long* strips_ny, int n);  // (strips, ny) of each cell; 0: the device cannot be asked
+cudaError_t launch_march_batch(const MarchBatch& b, int grid, int parity, cudaStream_t s);
+
 // per-unit entry points
 cudaError_t launch_step_2d_f32(int vec, bool trt, int rows, const void*, void*, const KParams&, dim3, dim3,
                                cudaStream_t);

@@ -46,6 +46,10 @@ struct tlbm_s {
 };
 
 namespace tlbm {
+// Calls of at least this many steps advance several steps per launch where the
+// handle or batch does that at all (shorter calls keep one launch per step).
+constexpr int MULTI_CALL = 16;
+
 // The reductions of many handles at once (api.cu); the first handle that
 // failed in *failed.
 int reduce_many(tlbm_t* hs, int n, const KParams* d_kp, cudaStream_t stream, double* nu, int* diverged,

@@ -295,21 +295,21 @@ template <> struct PV<double> {
     __device__ static double body(const KParams& p, int a) { return p.body[a]; }
 };
 template <> struct PV<float> {
-    __device__ static float sp(const KParams& p) { return p.spf; }
-    __device__ static float sm(const KParams& p) { return p.smf; }
-    __device__ static float shp(const KParams& p) { return p.shpf; }
-    __device__ static float shm(const KParams& p) { return p.shmf; }
-    __device__ static float qp(const KParams& p) { return p.qpf; }
-    __device__ static float qm(const KParams& p) { return p.qmf; }
-    __device__ static float S(const KParams& p, int k) { return p.Sf[k]; }
-    __device__ static float Sh(const KParams& p, int k) { return p.Shf[k]; }
-    __device__ static float Q(const KParams& p, int k) { return p.Qf[k]; }
-    __device__ static float gbeta(const KParams& p) { return p.gbetaf; }
-    __device__ static float omega(const KParams& p) { return p.omegaf; }
-    __device__ static float Th(const KParams& p) { return p.Thf; }
-    __device__ static float Tc(const KParams& p) { return p.Tcf; }
-    __device__ static float aT(const KParams& p) { return p.a_Tf; }
-    __device__ static float body(const KParams& p, int a) { return p.bodyf[a]; }
+    template <class T> __device__ static float sp(const T& p) { return p.spf; }
+    template <class T> __device__ static float sm(const T& p) { return p.smf; }
+    template <class T> __device__ static float shp(const T& p) { return p.shpf; }
+    template <class T> __device__ static float shm(const T& p) { return p.shmf; }
+    template <class T> __device__ static float qp(const T& p) { return p.qpf; }
+    template <class T> __device__ static float qm(const T& p) { return p.qmf; }
+    template <class T> __device__ static float S(const T& p, int k) { return p.Sf[k]; }
+    template <class T> __device__ static float Sh(const T& p, int k) { return p.Shf[k]; }
+    template <class T> __device__ static float Q(const T& p, int k) { return p.Qf[k]; }
+    template <class T> __device__ static float gbeta(const T& p) { return p.gbetaf; }
+    template <class T> __device__ static float omega(const T& p) { return p.omegaf; }
+    template <class T> __device__ static float Th(const T& p) { return p.Thf; }
+    template <class T> __device__ static float Tc(const T& p) { return p.Tcf; }
+    template <class T> __device__ static float aT(const T& p) { return p.a_Tf; }
+    template <class T> __device__ static float body(const T& p, int a) { return p.bodyf[a]; }
 };
 
 // flow weight w_i in precision C
@@ -680,8 +680,9 @@ __device__ __forceinline__ V vdot_unit(V x, V y, V z) {
 // +4 % for the staged 2D FP16 kernel, +1.6 % for the in-place 2D FP32 kernel;
 // -1 % to -7 % for the 3D FP16 kernels held to 96 registers and the batched
 // FP32 kernel, within 0.3 % elsewhere.
-template <int DIM, class V, bool SCALED, bool HC = false>
-__device__ __forceinline__ void collide_trt_v(V (&d)[Lat<DIM>::F::Q], V (&g)[Lat<DIM>::G::Q], const KParams& p) {
+// PT: KParams, or a structure with those of its members that the FP32 form reads.
+template <int DIM, class V, bool SCALED, bool HC = false, class PT = KParams>
+__device__ __forceinline__ void collide_trt_v(V (&d)[Lat<DIM>::F::Q], V (&g)[Lat<DIM>::G::Q], const PT& p) {
     using LF = typename Lat<DIM>::F;
     using LG = typename Lat<DIM>::G;
     using P = PV<float>;
@@ -702,8 +703,12 @@ __device__ __forceinline__ void collide_trt_v(V (&d)[Lat<DIM>::F::Q], V (&g)[Lat
         constexpr int i = decltype(ii)::value;
         if constexpr (i > 0) Ts = vadd(Ts, g[i]);
     });
-    const float sc = SCALED ? ScaleOf<float>::s(p) : 1.0f;
-    const V inv = vbc<V>(SCALED ? ScaleOf<float>::inv(p) : 1.0f);
+    float sc = 1.0f, inv1 = 1.0f;
+    if constexpr (SCALED) {
+        sc = ScaleOf<float>::s(p);
+        inv1 = ScaleOf<float>::inv(p);
+    }
+    const V inv = vbc<V>(inv1);
     const V drho = SCALED ? vmul(drs, inv) : drs;
     const V T = SCALED ? vmul(Ts, inv) : Ts;
     const V rho = vadd(vbc<V>(1.0f), drho);

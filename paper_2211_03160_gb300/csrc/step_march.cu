@@ -56,17 +56,19 @@ __device__ __forceinline__ float2 march_shift(float2 v) {
 }
 
 // the thermal wall rule: anti-bounce-back at a wall of temperature Tw, bounce-back at an adiabatic one
-__device__ __forceinline__ float march_rule(float v, bool iso, const KParams& p, float Tw) {
+template <class PT>
+__device__ __forceinline__ float march_rule(float v, bool iso, const PT& p, float Tw) {
     return iso ? -v + p.omegaf * Tw : v;
 }
 
 // copy the stored pairs a lane pulls for one row (before the shift along x) to
 // the lane's places in shared memory, as one group of its asynchronous copies
-__device__ __forceinline__ void march_fetch(const float* __restrict__ own, const KParams& p, uint32_t to) {
+template <class PT>
+__device__ __forceinline__ void march_fetch(const float* __restrict__ own, const PT& p, const KParams& full, uint32_t to) {
 #pragma unroll
     for (int j = 0; j < 14; ++j)
         asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"(to + j * MARCH_W * 4),
-                     "l"(TLBM_DBG(p, (own + p.loff[j]), 0, 2))
+                     "l"(TLBM_DBG(full, (own + p.loff[j]), 0, 2))
                      : "memory");
 }
 
@@ -81,8 +83,8 @@ struct MarchKept {
 
 // f, g: the post-collision values of row r, or anything if r = ny.  Keeps what
 // later rows pull of them and turns f, g into what row r - 1 pulls.
-template <int DIM>
-__device__ __forceinline__ void march_pull(MarchKept& k, float2 (&f)[9], float2 (&g)[5], const KParams& p, int r, int x,
+template <int DIM, class PT>
+__device__ __forceinline__ void march_pull(MarchKept& k, float2 (&f)[9], float2 (&g)[5], const PT& p, int r, int x,
                                            bool wall_strip, bool heat_y) {
     const Layout& L = p.L;
     float2 f4, f7, f8, g4;
@@ -162,9 +164,11 @@ __device__ __forceinline__ void march_pull(MarchKept& k, float2 (&f)[9], float2 
     }
 }
 
-template <int DIM>
-__global__ void __launch_bounds__(32 * MARCH_WARPS, MARCH_BLOCKS)
-    step_march_kernel(const float* __restrict__ src, float* __restrict__ dst, const KParams p, int strips, int seg) {
+// One warp's strip and segment.  p: the parameters of the hot path; full: all of
+// them, for the wall rules of the last step (the same object for a single cell).
+template <int DIM, class PT>
+__device__ __forceinline__ void march_strip(const float* __restrict__ src, float* __restrict__ dst, const PT& p,
+                                            const KParams& full, int strip, int sg, int seg) {
     static_assert(MARCH_SIDE >= MARCH_STEPS && MARCH_SIDE % 2 == 0, "valid columns");
     using LF = typename Lat<DIM>::F;
     using LG = typename Lat<DIM>::G;
@@ -172,9 +176,6 @@ __global__ void __launch_bounds__(32 * MARCH_WARPS, MARCH_BLOCKS)
     constexpr int LV = MARCH_STEPS, SIDE = MARCH_SIDE, OUT = MARCH_OUT;
     const Layout& L = p.L;
     const int lane = threadIdx.x & 31;
-    const int item = blockIdx.x * MARCH_WARPS + (threadIdx.x >> 5);
-    const int sg = item / strips, strip = item - sg * strips;
-    if (sg * seg >= p.L.ny) return;
     const int x = strip * OUT - SIDE + 2 * lane;  // the lane's first column
     const int y0 = sg * seg, y1 = min(y0 + seg, L.ny);
     const bool wall_strip = strip == 0 || strip * OUT + OUT + SIDE >= L.nx;
@@ -202,7 +203,7 @@ __global__ void __launch_bounds__(32 * MARCH_WARPS, MARCH_BLOCKS)
     const float* from = src + L.row(r0, 0) + xld;
 #pragma unroll
     for (int k = 0; k < MARCH_AHEAD; ++k) {
-        if (r0 + k <= rl) march_fetch(from + (long long)k * L.P, p, mine_at + k * ROWB);
+        if (r0 + k <= rl) march_fetch(from + (long long)k * L.P, p, full, mine_at + k * ROWB);
         asm volatile("cp.async.commit_group;" ::: "memory");
     }
     from += (long long)MARCH_AHEAD * L.P;
@@ -210,7 +211,7 @@ __global__ void __launch_bounds__(32 * MARCH_WARPS, MARCH_BLOCKS)
     for (int r = r0; r <= y1 + LV - 2; ++r) {
         float2 f[QF], g[QG];
         if (r < L.ny) {
-            if (r + MARCH_AHEAD <= rl) march_fetch(from, p, mine_at + ahead * ROWB);
+            if (r + MARCH_AHEAD <= rl) march_fetch(from, p, full, mine_at + ahead * ROWB);
             asm volatile("cp.async.commit_group;" ::: "memory");
             asm volatile("cp.async.wait_group %0;" ::"n"(MARCH_AHEAD) : "memory");
             from += L.P;
@@ -240,13 +241,13 @@ __global__ void __launch_bounds__(32 * MARCH_WARPS, MARCH_BLOCKS)
         if (x + 1 < L.nx) {
             static_for<Q>([&](auto jj) {
                 constexpr int j = decltype(jj)::value;
-                __stwb(reinterpret_cast<float2*>(TLBM_DBG(p, (own + p.soff[j]), 0, 2)),
+                __stwb(reinterpret_cast<float2*>(TLBM_DBG(full, (own + p.soff[j]), 0, 2)),
                        j < QF ? f[j < QF ? j : 0] : g[j < QF ? 0 : j - QF]);
             });
         } else {
             static_for<Q>([&](auto jj) {
                 constexpr int j = decltype(jj)::value;
-                *TLBM_DBG(p, (own + p.soff[j]), 0, 1) = j < QF ? f[j < QF ? j : 0].x : g[j < QF ? 0 : j - QF].x;
+                *TLBM_DBG(full, (own + p.soff[j]), 0, 1) = j < QF ? f[j < QF ? j : 0].x : g[j < QF ? 0 : j - QF].x;
             });
         }
         if (y == 0 || y == L.ny - 1 || x == 0 || x + 2 >= L.nx) {
@@ -255,9 +256,34 @@ __global__ void __launch_bounds__(32 * MARCH_WARPS, MARCH_BLOCKS)
             for (int i = 0; i < QF; ++i) { fw[i][0] = f[i].x; fw[i][1] = f[i].y; }
 #pragma unroll
             for (int i = 0; i < QG; ++i) { gw[i][0] = g[i].x; gw[i][1] = g[i].y; }
-            wall_writes<2, float, 2, float, true>(dst, p, x, y, 0, fw, gw, 0u);
+            wall_writes<2, float, 2, float, true>(dst, full, x, y, 0, fw, gw, 0u);
         }
     }
+}
+
+template <int DIM>
+__global__ void __launch_bounds__(32 * MARCH_WARPS, MARCH_BLOCKS)
+    step_march_kernel(const float* __restrict__ src, float* __restrict__ dst, const KParams p, int strips, int seg) {
+    const int item = blockIdx.x * MARCH_WARPS + (threadIdx.x >> 5), sg = item / strips;
+    if (sg * seg < p.L.ny) march_strip<DIM>(src, dst, p, p, item - sg * strips, sg, seg);
+}
+
+// The cells of a batch: a block's warps all march in one cell, whose parameters
+// it reads from the launch's parameters (constant memory) at an index that is
+// the same for the block.
+template <int DIM>
+__global__ void __launch_bounds__(32 * MARCH_WARPS, MARCH_BLOCKS)
+    step_march_batch_kernel(const __grid_constant__ MarchBatch b, int parity) {
+    int lo = 0, hi = b.n - 1;
+    while (lo < hi) {
+        const int mid = (lo + hi + 1) / 2;
+        if (b.cell[mid].block0 <= (int)blockIdx.x) lo = mid;
+        else hi = mid - 1;
+    }
+    const MarchCell& c = b.cell[lo];
+    const int item = ((int)blockIdx.x - c.block0) * MARCH_WARPS + (threadIdx.x >> 5), sg = item / c.strips;
+    if (sg * b.rows < c.L.ny)
+        march_strip<DIM>(c.buf[parity], c.buf[parity ^ 1], c, *c.full, item - sg * c.strips, sg, b.rows);
 }
 
 }  // namespace
@@ -285,6 +311,56 @@ cudaError_t launch_march(const void* src, void* dst, const KParams& p, int rows,
     const int strips = (p.L.nx + MARCH_OUT - 1) / MARCH_OUT;
     const int items = strips * ((p.L.ny + rows - 1) / rows), grid = (items + MARCH_WARPS - 1) / MARCH_WARPS;
     step_march_kernel<2><<<grid, 32 * MARCH_WARPS, 0, s>>>((const float*)src, (float*)dst, p, strips, rows);
+    return cudaGetLastError();
+}
+
+int march_batch_rows(const long long* strips_ny, int n) {
+    int dev = 0, sms = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess ||
+        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
+        return 0;
+    // march_rows for all cells together
+    const long long resident = (long long)sms * MARCH_BLOCKS * MARCH_WARPS;
+    for (int rows = 4;; rows += rows < 16 ? 1 : 4) {
+        long long items = 0;
+        for (int i = 0; i < n; ++i) items += strips_ny[2 * i] * ((strips_ny[2 * i + 1] + rows - 1) / rows);
+        if (items <= resident || rows >= 64) return rows;
+    }
+}
+
+MarchCell march_cell(const KParams& p, const void* buf0, const void* buf1, const KParams* full) {
+    MarchCell c{};
+    c.L = p.L;
+    c.heat_axis = p.heat_axis;
+    c.gbetaf = p.gbetaf;
+    c.omegaf = p.omegaf;
+    c.Thf = p.Thf;
+    c.Tcf = p.Tcf;
+    for (int a = 0; a < 3; ++a) c.bodyf[a] = p.bodyf[a];
+    c.spf = p.spf;
+    c.smf = p.smf;
+    c.shpf = p.shpf;
+    c.shmf = p.shmf;
+    c.qpf = p.qpf;
+    c.qmf = p.qmf;
+    c.tf = p.tf;
+    for (int j = 0; j < 14; ++j) {
+        c.loff[j] = p.loff[j];
+        c.soff[j] = p.soff[j];
+    }
+    c.buf[0] = (float*)buf0;
+    c.buf[1] = (float*)buf1;
+    c.full = full;
+    c.strips = (p.L.nx + MARCH_OUT - 1) / MARCH_OUT;
+    return c;
+}
+
+int march_cell_blocks(const MarchCell& c, int rows) {
+    return (c.strips * ((c.L.ny + rows - 1) / rows) + MARCH_WARPS - 1) / MARCH_WARPS;
+}
+
+cudaError_t launch_march_batch(const MarchBatch& b, int grid, int parity, cudaStream_t s) {
+    step_march_batch_kernel<2><<<grid, 32 * MARCH_WARPS, 0, s>>>(b, parity);
     return cudaGetLastError();
 }
 
