@@ -717,7 +717,7 @@ constexpr int MULTI_GRAPH = 8;  // launches of a graph block (even: it ends in t
 // `parity` and writing the other.
 static cudaError_t launch_multi_raw(tlbm_t h, int parity, int steps, cudaStream_t s) {
     if (h->march && steps == 1) return launch_step_raw(h, parity, s);
-    if (h->march) return launch_march(h->buf[parity], h->buf[parity ^ 1], h->kp, h->march, s);
+    if (h->march) return launch_march(h->prec, h->buf[parity], h->buf[parity ^ 1], h->kp, h->march, s);
     MultiGeo g = h->mg;
     g.steps = steps;
     return launch_multi(h->prec, h->buf[parity], h->buf[parity ^ 1], h->kp, g, s);
@@ -1297,10 +1297,10 @@ static int set_staged(tlbm_t h, int tile_width, int stages) {
 }
 
 // Several steps per launch: 2D two-buffer cells with two-relaxation-time rates
-// whose launches the caller has not chosen.  FP32 cells with walls all around go
-// through step_march.cu from 250,000 nodes (513^2: 6.7 us per step against 7.1
-// in tiles and 10.5 singly) unless their width would leave more than a quarter
-// of its strips' columns idle.  Else tiles (step_multi.cu) up to the size where
+// whose launches the caller has not chosen.  FP32 and 16-bit cells with walls all
+// around go through step_march.cu from 250,000 / 270,000 nodes (513^2 FP32: 6.7 us
+// per step against 7.1 in tiles and 10.5 singly; FP16: 7.6, 7.4 and 12.3) unless
+// their width would leave more than a quarter of its strips' columns idle.  Else tiles (step_multi.cu) up to the size where
 // one step fills the GPU.  FP32, FP16 and BF16: 300,000 nodes (a 513^2 cell gains 1.5x, a 1025^2
 // one 1.1x in FP32 and loses a quarter in FP16), the 16-bit ones not with rows of
 // over 2048 nodes, which suit the staged kernel's tiles (4000 x 70: 8.5 us per
@@ -1311,8 +1311,8 @@ static void pick_multi(tlbm_t h) {
     if (h->dim != 2 || h->aa || !h->kp.trt || h->variant_chosen || h->graph_chosen) return;
     const long long nodes = (long long)h->nx * h->ny;
     const int strips = (h->nx + MARCH_COLUMNS - 1) / MARCH_COLUMNS;
-    if (h->prec == TLBM_FP32 && !h->kp.periodic && nodes >= 250000 && 4 * h->nx >= 3 * strips * MARCH_COLUMNS) {
-        h->march = march_rows(h->kp);
+    if (h->prec != TLBM_FP64 && !h->kp.periodic && nodes >= (h->prec == TLBM_FP32 ? 250000 : 270000) && 4 * h->nx >= 3 * strips * MARCH_COLUMNS) {
+        h->march = march_rows(h->prec, h->kp);
         if (h->march) h->multi = MARCH_STEPS;
         return;
     }

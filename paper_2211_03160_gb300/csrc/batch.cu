@@ -390,23 +390,24 @@ static void build_tables(tlbm_batch_t b, std::vector<KParams>& kps, std::vector<
     b->staged_tiles = stile0;
 }
 
-// The marching form: 2D FP32 cells with walls all around and two-relaxation-time
+// The marching form: 2D FP32 and 16-bit cells with walls all around and two-relaxation-time
 // rates, in a batch whose launches the caller has not chosen.  us per step of
 // 64 FP32 cells of 129^2 to 1025^2: flattened launch untuned 606, staged (the tuned
-// form) 473, marching 289; of 64 cells of 1025^2 1445, 1156 and 652, 16 of 513^2
-// 134, 85 and 61, 48 of 65^2 37, 16 and 9.6.
+// form) 473, marching 274; of 64 cells of 1025^2 1445, 1152 and 618, 16 of 513^2
+// 135, 85 and 58, 48 of 65^2 37, 16 and 9.2; FP16 461, 336 and 296, 1065, 798 and 669,
+// 114, 62 and 59, 42, 16 and 10.3.
 static void build_marches(tlbm_batch_t b) {
     b->marches.clear();
     b->march_grids.clear();
     b->march = 0;
-    if (b->dim != 2 || b->prec != TLBM_FP32 || b->form_chosen || b->march_off || b->persist_steps > 0) return;
+    if (b->dim != 2 || b->prec == TLBM_FP64 || b->form_chosen || b->march_off || b->persist_steps > 0) return;
     std::vector<long long> sizes;
     for (tlbm_t h : b->inst) {
         if (!h->kp.trt || h->kp.periodic) return;
         sizes.push_back((h->nx + MARCH_COLUMNS - 1) / MARCH_COLUMNS);
         sizes.push_back(h->ny);
     }
-    const int rows = march_batch_rows(sizes.data(), b->n);
+    const int rows = march_batch_rows(b->prec, sizes.data(), b->n);
     if (rows == 0) return;
     for (int i0 = 0; i0 < b->n; i0 += MARCH_MANY) {
         MarchBatch m{};
@@ -428,7 +429,7 @@ static void build_marches(tlbm_batch_t b) {
 static cudaError_t launch_marches(tlbm_batch_t b, int parity, cudaStream_t s) {
     cudaError_t e = cudaSuccess;
     for (size_t i = 0; i < b->marches.size() && e == cudaSuccess; ++i)
-        e = launch_march_batch(b->marches[i], b->march_grids[i], parity, s);
+        e = launch_march_batch(b->prec, b->marches[i], b->march_grids[i], parity, s);
     return e;
 }
 

@@ -43,22 +43,22 @@ struct MultiGeo {
 bool multi_setup(int prec, const KParams& p, MultiGeo& g);
 cudaError_t launch_multi(int prec, const void* src, void* dst, const KParams& p, const MultiGeo& g, cudaStream_t s);
 
-// MARCH_STEPS steps of a 2D FP32 cell with walls on every side in one pass over
+// MARCH_STEPS steps of a 2D FP32, FP16 or BF16 cell with walls on every side in one pass over
 // memory, in segments of `rows` rows (step_march.cu), TRT form
 constexpr int MARCH_STEPS = 3;
 constexpr int MARCH_COLUMNS = 56;  // columns a warp stores
-int march_rows(const KParams& p);  // rows of a segment, 0: the device cannot be asked
-cudaError_t launch_march(const void* src, void* dst, const KParams& p, int rows, cudaStream_t s);
+int march_rows(int prec, const KParams& p);  // rows of a segment, 0: the device cannot be asked
+cudaError_t launch_march(int prec, const void* src, void* dst, const KParams& p, int rows, cudaStream_t s);
 
 // the same for the cells of a batch: what the kernel reads of a cell in its hot
 // path (members as in KParams), all of a launch's cells by value
 struct MarchCell {
     Layout L;
     int heat_axis, strips, block0;  // block0: its first block of the launch
-    float gbetaf, omegaf, Thf, Tcf, bodyf[3], spf, smf, shpf, shmf, qpf, qmf;
+    float gbetaf, omegaf, Thf, Tcf, bodyf[3], spf, smf, shpf, shmf, qpf, qmf, scale, inv_scale;
     decltype(KParams::tf) tf;
     int loff[14], soff[14];
-    float* buf[2];
+    void* buf[2];
     const KParams* full;  // all parameters, in device memory
 };
 constexpr int MARCH_MANY = 64;  // most cells of a launch (kernel parameters hold 32 KB)
@@ -69,8 +69,8 @@ struct MarchBatch {
 static_assert(sizeof(MarchBatch) <= 32000, "kernel parameters");
 MarchCell march_cell(const KParams& p, const void* buf0, const void* buf1, const KParams* full);
 int march_cell_blocks(const MarchCell& c, int rows);
-int march_batch_rows(const long long* strips_ny, int n);  // (strips, ny) of each cell; 0: the device cannot be asked
-cudaError_t launch_march_batch(const MarchBatch& b, int grid, int parity, cudaStream_t s);
+int march_batch_rows(int prec, const long long* strips_ny, int n);  // (strips, ny) of each cell; 0: the device cannot be asked
+cudaError_t launch_march_batch(int prec, const MarchBatch& b, int grid, int parity, cudaStream_t s);
 
 // per-unit entry points
 cudaError_t launch_step_2d_f32(int vec, bool trt, int rows, const void*, void*, const KParams&, dim3, dim3,

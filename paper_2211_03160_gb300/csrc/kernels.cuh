@@ -354,8 +354,8 @@ __device__ __forceinline__ S enc_g_step(C g, C scale, uint32_t salt) {
 
 template <class C> struct ScaleOf;
 template <> struct ScaleOf<float> {
-    __device__ static float s(const KParams& p) { return p.scale; }
-    __device__ static float inv(const KParams& p) { return p.inv_scale; }
+    template <class T> __device__ static float s(const T& p) { return p.scale; }
+    template <class T> __device__ static float inv(const T& p) { return p.inv_scale; }
 };
 template <> struct ScaleOf<double> {
     __device__ static double s(const KParams& p) { return (double)p.scale; }
