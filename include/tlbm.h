@@ -431,6 +431,46 @@ TLBM_API int tlbm_to_bf16(const float* a, long long n, void* b, void* stream);
  * FP64 block sums (deterministic order). */
 TLBM_API int tlbm_mse_loss(const float* y, const float* target, long long n, float* g, void* g_bf16,
                            double* loss_dev, double* partial_dev, void* stream);
+/* The same layers between channels-last tensors ("cl": BF16 [B][H][W][Cp], Cp =
+ * 16 ceil(C / 16), zero past channel C; 16-byte aligned), the layout the tensor
+ * cores take without rearrangement; what a network keeps between its layers.
+ * Channels-last copy of x (BF16 [B][C][H][W]): */
+TLBM_API int tlbm_conv_channels_last(const void* x, int B, int C, int H, int W, void* out, void* stream);
+/* tlbm_conv3x3_forward of a cl input: y (FP32 [B][cout][H][W], or NULL) and act
+ * (cl, relu'd if relu != 0, or NULL). */
+TLBM_API int tlbm_conv3x3_forward_cl(const void* x, const void* a, const float* bias, float* y, void* act, int B,
+                                     int cin, int cout, int H, int W, int relu, void* stream);
+/* Bytes of workspace of the two gradients below for this shape on this device. */
+TLBM_API int tlbm_conv3x3_cl_workspace_bytes(int B, int cin, int cout, int H, int W, size_t* bytes);
+/* Gradient with respect to the layer's input and back through the relu that
+ * made it: g (cl, cin channels) = dx where act > 0 else 0, from dy (cl, cout
+ * channels), the FP32 weights w[cout][cin][3][3] (rounded to BF16) and act (cl),
+ * the layer's input; db[cin] = sum over pixels of the same in FP32 (the bias
+ * gradient of the layer before).  Fixed summation order on a given device. */
+TLBM_API int tlbm_conv3x3_backward_data_cl(const void* dy, const float* w, const void* act, void* g, float* db, int B,
+                                           int cin, int cout, int H, int W, void* workspace, size_t workspace_bytes,
+                                           void* stream);
+/* tlbm_conv3x3_backward_weight's dw for cl x and dy. */
+TLBM_API int tlbm_conv3x3_backward_weight_cl(const void* x, const void* dy, float* dw, int B, int cin, int cout, int H,
+                                             int W, void* workspace, size_t workspace_bytes, void* stream);
+/* db[cout] = sum over pixels of dy (FP32 [B][cout][H][W]); workspace of at
+ * least 8192 bytes. */
+TLBM_API int tlbm_conv3x3_bias_grad(const float* dy, float* db, int B, int cout, int H, int W, void* workspace,
+                                    size_t workspace_bytes, void* stream);
+/* One layer of tlbm_conv_adam_layers: weights [cout][cin][3][3] and biases with
+ * their gradients and moments (FP32), and the packed operand a of
+ * tlbm_conv3x3_pack_weights (written before with the same shape). */
+typedef struct {
+    float* w; const float* gw; float* mw; float* vw;
+    float* b; const float* gb; float* mb; float* vb;
+    void* a;
+    int cout, cin;
+} tlbm_conv_layer;
+enum { TLBM_CONV_MAX_LAYERS = 16 };
+/* tlbm_adam_step on every weight and bias of n <= 16 layers and
+ * tlbm_conv3x3_pack_weights of the new weights, in one launch. */
+TLBM_API int tlbm_conv_adam_layers(const tlbm_conv_layer* layers, int n, float lr, float b1, float b2, float eps,
+                                   int t, void* stream);
 /* One Adam step (Kingma & Ba 2015) on FP32 weights w with moments m, v; t >= 1. */
 TLBM_API int tlbm_adam_step(float* w, const float* g, float* m, float* v, long long n, float lr, float b1,
                             float b2, float eps, int t, void* stream);

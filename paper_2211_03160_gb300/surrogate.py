@@ -147,62 +147,57 @@ class ConvNet:
         for (cout, cin), w, a in zip(self.shapes, self.w, self.a):
             tlbm.tlbm_conv3x3_pack_weights(w, cout, cin, a, self.torch.cuda.current_stream())
 
+    @staticmethod
+    def _cl(torch, B, ch, H, W, device):
+        """A channels-last BF16 tensor of ch channels (16 to a group)."""
+        return torch.empty((B, H, W, 16 * ((ch + 15) // 16)), dtype=torch.bfloat16, device=device)
+
     def forward(self, x16, B: int, H: int, W: int):
         """x16: BF16 [B][CIN][H][W].  Returns the FP32 output and keeps what the
-        backward pass needs."""
+        backward pass needs: the layers' inputs, channels last."""
         torch = self.torch
         s = torch.cuda.current_stream()
+        a_in = self._cl(torch, B, CIN, H, W, x16.device)
+        tlbm.tlbm_conv_channels_last(x16, B, CIN, H, W, a_in, s)
         self.cache = []
-        a_in = x16
         for k, (cout, cin) in enumerate(self.shapes):
-            y = torch.empty((B, cout, H, W), dtype=torch.float32, device=x16.device)
-            last = k == len(self.shapes) - 1
-            act = None if last else torch.empty((B, cout, H, W), dtype=torch.bfloat16, device=x16.device)
-            tlbm.tlbm_conv3x3_forward(a_in, self.a[k], self.b[k], y, act, B, cin, cout, H, W, 0 if last else 1, s)
-            self.cache.append((a_in, y))
-            a_in = act
+            self.cache.append(a_in)
+            if k == len(self.shapes) - 1:
+                y = torch.empty((B, cout, H, W), dtype=torch.float32, device=x16.device)
+                tlbm.tlbm_conv3x3_forward_cl(a_in, self.a[k], self.b[k], y, None, B, cin, cout, H, W, 0, s)
+            else:
+                act = self._cl(torch, B, cout, H, W, x16.device)
+                tlbm.tlbm_conv3x3_forward_cl(a_in, self.a[k], self.b[k], None, act, B, cin, cout, H, W, 1, s)
+                a_in = act
         return y
 
     def backward(self, g32, g16, B: int, H: int, W: int):
+        """Gradients of every layer from those of the output (FP32 and BF16 [B][COUT][H][W])."""
         torch = self.torch
         s = torch.cuda.current_stream()
-        at = torch.empty(32 * 288, dtype=torch.bfloat16, device=g32.device)
-        self.gw = [None] * len(self.shapes)
-        self.gb = [None] * len(self.shapes)
+        dev = g32.device
+        self.gw = [torch.empty_like(w) for w in self.w]
+        self.gb = [torch.empty_like(b) for b in self.b]
+        ws = torch.empty(max(8192, *[tlbm.tlbm_conv3x3_cl_workspace_bytes(B, cin, cout, H, W)
+                                     for cout, cin in self.shapes]), dtype=torch.uint8, device=dev)
+        g = self._cl(torch, B, COUT, H, W, dev)
+        tlbm.tlbm_conv_channels_last(g16, B, COUT, H, W, g, s)
+        tlbm.tlbm_conv3x3_bias_grad(g32, self.gb[-1], B, COUT, H, W, ws, s)
         for k in range(len(self.shapes) - 1, -1, -1):
             cout, cin = self.shapes[k]
-            x_in, _ = self.cache[k]
-            ws = torch.empty(tlbm.tlbm_conv3x3_workspace_bytes(B, cin, cout, H, W), dtype=torch.uint8,
-                             device=g32.device)
-            dw = torch.empty((cout, cin, 3, 3), dtype=torch.float32, device=g32.device)
-            db = torch.empty(cout, dtype=torch.float32, device=g32.device)
-            tlbm.tlbm_conv3x3_backward_weight(x_in, g16, g32, dw, db, B, cin, cout, H, W, ws, s)
-            self.gw[k], self.gb[k] = dw, db
+            x_in = self.cache[k]
+            tlbm.tlbm_conv3x3_backward_weight_cl(x_in, g, self.gw[k], B, cin, cout, H, W, ws, s)
             if k > 0:
-                wb = self.a_plain_bf16(k)
-                dx = torch.empty((B, cin, H, W), dtype=torch.float32, device=g32.device)
-                tlbm.tlbm_conv3x3_backward_data(g16, wb, dx, B, cin, cout, H, W, at, s)
-                _, y_prev = self.cache[k - 1]
-                g32 = torch.empty_like(dx)
-                g16 = torch.empty(dx.shape, dtype=torch.bfloat16, device=g32.device)
-                tlbm.tlbm_relu_backward(dx, y_prev, dx.numel(), g32, g16, s)
-
-    def a_plain_bf16(self, k):
-        """BF16 copy of layer k's weights in [cout][cin][3][3] order."""
-        torch = self.torch
-        w16 = torch.empty(self.w[k].shape, dtype=torch.bfloat16, device=self.w[k].device)
-        tlbm.tlbm_to_bf16(self.w[k], self.w[k].numel(), w16, torch.cuda.current_stream())
-        return w16
+                g_prev = self._cl(torch, B, cin, H, W, dev)
+                tlbm.tlbm_conv3x3_backward_data_cl(g, self.w[k], x_in, g_prev, self.gb[k - 1], B, cin, cout, H, W, ws, s)
+                g = g_prev
 
     def adam(self, lr: float):
-        s = self.torch.cuda.current_stream()
         self.t += 1
-        for k in range(len(self.shapes)):
-            tlbm.tlbm_adam_step(self.w[k], self.gw[k], self.mw[k], self.vw[k], self.w[k].numel(), lr, 0.9, 0.999,
-                                1e-8, self.t, s)
-            tlbm.tlbm_adam_step(self.b[k], self.gb[k], self.mb[k], self.vb[k], self.b[k].numel(), lr, 0.9, 0.999,
-                                1e-8, self.t, s)
-        self.pack()
+        tlbm.tlbm_conv_adam_layers(
+            [(self.w[k], self.gw[k], self.mw[k], self.vw[k], self.b[k], self.gb[k], self.mb[k], self.vb[k], self.a[k],
+              cout, cin) for k, (cout, cin) in enumerate(self.shapes)], lr, 0.9, 0.999, 1e-8, self.t,
+            self.torch.cuda.current_stream())
 
     def state(self):
         return {"w": [w.cpu().numpy() for w in self.w], "b": [b.cpu().numpy() for b in self.b]}

@@ -50,6 +50,11 @@ class tlbm_instance(C.Structure):
                 ("Pr", C.c_double), ("Ma", C.c_double), ("seed", C.c_uint64)]
 
 
+class tlbm_conv_layer(C.Structure):
+    _fields_ = [(k, C.c_void_p) for k in ("w", "gw", "mw", "vw", "b", "gb", "mb", "vb", "a")] + \
+               [("cout", C.c_int), ("cin", C.c_int)]
+
+
 class TlbmError(RuntimeError):
     def __init__(self, code, msg):
         super().__init__(f"tlbm error {code}: {msg}")
@@ -103,6 +108,17 @@ _SIGS = {
     "tlbm_conv3x3_backward_weight": (C.c_int, [C.c_void_p, C.c_void_p, C.c_void_p, C.c_void_p, C.c_void_p, C.c_int,
                                                C.c_int, C.c_int, C.c_int, C.c_int, C.c_void_p, C.c_size_t,
                                                C.c_void_p]),
+    "tlbm_conv_channels_last": (C.c_int, [C.c_void_p, C.c_int, C.c_int, C.c_int, C.c_int, C.c_void_p, C.c_void_p]),
+    "tlbm_conv3x3_forward_cl": (C.c_int, [C.c_void_p, C.c_void_p, C.c_void_p, C.c_void_p, C.c_void_p, C.c_int, C.c_int,
+                                          C.c_int, C.c_int, C.c_int, C.c_int, C.c_void_p]),
+    "tlbm_conv3x3_cl_workspace_bytes": (C.c_int, [C.c_int, C.c_int, C.c_int, C.c_int, C.c_int,
+                                                  C.POINTER(C.c_size_t)]),
+    "tlbm_conv3x3_backward_data_cl": (C.c_int, [C.c_void_p] * 5 + [C.c_int] * 5 + [C.c_void_p, C.c_size_t, C.c_void_p]),
+    "tlbm_conv3x3_backward_weight_cl": (C.c_int, [C.c_void_p] * 3 + [C.c_int] * 5 + [C.c_void_p, C.c_size_t,
+                                                                                    C.c_void_p]),
+    "tlbm_conv3x3_bias_grad": (C.c_int, [C.c_void_p] * 2 + [C.c_int] * 4 + [C.c_void_p, C.c_size_t, C.c_void_p]),
+    "tlbm_conv_adam_layers": (C.c_int, [C.c_void_p, C.c_int, C.c_float, C.c_float, C.c_float, C.c_float, C.c_int,
+                                        C.c_void_p]),
     "tlbm_relu_backward": (C.c_int, [C.c_void_p, C.c_void_p, C.c_longlong, C.c_void_p, C.c_void_p, C.c_void_p]),
     "tlbm_to_bf16": (C.c_int, [C.c_void_p, C.c_longlong, C.c_void_p, C.c_void_p]),
     "tlbm_mse_loss": (C.c_int, [C.c_void_p, C.c_void_p, C.c_longlong, C.c_void_p, C.c_void_p, C.c_void_p, C.c_void_p,
@@ -328,6 +344,46 @@ def tlbm_conv3x3_backward_weight(x, dy_bf16, dy, dw, db, B, cin, cout, H, W, wor
     _c(lib().tlbm_conv3x3_backward_weight(_ptr(x), _ptr(dy_bf16), _ptr(dy), _ptr(dw), _ptr(db), B, cin, cout, H, W,
                                           _ptr(workspace), workspace.numel() * workspace.element_size(),
                                           _cs(stream)))
+
+
+def tlbm_conv_channels_last(x, B, ch, H, W, out, stream=None):
+    _c(lib().tlbm_conv_channels_last(_ptr(x), B, ch, H, W, _ptr(out), _cs(stream)))
+
+
+def tlbm_conv3x3_forward_cl(x, a, bias, y, act, B, cin, cout, H, W, relu, stream=None):
+    _c(lib().tlbm_conv3x3_forward_cl(_ptr(x), _ptr(a), _ptr(bias), _ptr(y), _ptr(act), B, cin, cout, H, W, int(relu),
+                                     _cs(stream)))
+
+
+def tlbm_conv3x3_cl_workspace_bytes(B, cin, cout, H, W) -> int:
+    n = C.c_size_t()
+    _c(lib().tlbm_conv3x3_cl_workspace_bytes(B, cin, cout, H, W, C.byref(n)))
+    return n.value
+
+
+def tlbm_conv3x3_backward_data_cl(dy, w, act, g, db, B, cin, cout, H, W, workspace, stream=None):
+    _c(lib().tlbm_conv3x3_backward_data_cl(_ptr(dy), _ptr(w), _ptr(act), _ptr(g), _ptr(db), B, cin, cout, H, W,
+                                           _ptr(workspace), workspace.numel() * workspace.element_size(),
+                                           _cs(stream)))
+
+
+def tlbm_conv3x3_backward_weight_cl(x, dy, dw, B, cin, cout, H, W, workspace, stream=None):
+    _c(lib().tlbm_conv3x3_backward_weight_cl(_ptr(x), _ptr(dy), _ptr(dw), B, cin, cout, H, W, _ptr(workspace),
+                                             workspace.numel() * workspace.element_size(), _cs(stream)))
+
+
+def tlbm_conv3x3_bias_grad(dy, db, B, cout, H, W, workspace, stream=None):
+    _c(lib().tlbm_conv3x3_bias_grad(_ptr(dy), _ptr(db), B, cout, H, W, _ptr(workspace),
+                                    workspace.numel() * workspace.element_size(), _cs(stream)))
+
+
+def tlbm_conv_adam_layers(layers, lr, b1, b2, eps, t, stream=None):
+    """layers: sequence of (w, gw, mw, vw, b, gb, mb, vb, a, cout, cin)."""
+    arr = (tlbm_conv_layer * len(layers))()
+    for k, q in enumerate(layers):
+        arr[k] = tlbm_conv_layer(*[p.data_ptr() for p in q[:9]], q[9], q[10])
+    _c(lib().tlbm_conv_adam_layers(C.cast(arr, C.c_void_p), len(layers), float(lr), float(b1), float(b2), float(eps),
+                                   int(t), _cs(stream)))
 
 
 def tlbm_relu_backward(dx, y, n, g, g_bf16, stream=None):
