@@ -49,6 +49,7 @@ static int cuda_fail(tlbm_t h, cudaError_t e, const char* what) {
 
 static void drop_graph(tlbm_t h);
 static int set_staged(tlbm_t h, int tile_width, int stages);
+static void pick_16bit(tlbm_t h);
 static void pick_multi(tlbm_t h);
 
 // The buffer (two-buffer pull) or the order (in place: 0 natural, 1 swapped)
@@ -443,7 +444,7 @@ extern "C" int tlbm_create(tlbm_t* out, int nx, int ny, int nz, int lattice, dou
         kp.qpf = (float)kp.qp; kp.qmf = (float)kp.qm;
     }
     h->trt = kp.trt;
-    h->flat = precision == TLBM_FP64 && kp.trt;
+    h->flat = precision == TLBM_FP64 && kp.trt && (double)nx * ny * nz <= FLAT_NODES;
     {
         // per-population pull / store offsets (elements, relative to a node's own
         // slot in plane 0): plane j, shifted back by the population's e_y, e_z
@@ -622,17 +623,7 @@ extern "C" int tlbm_bind_memory(tlbm_t h, void* dev_ptr, size_t bytes) {
     if (e != cudaSuccess) return cuda_fail(h, e, "cudaMemset");
 #endif
     set_cur(h, 0);
-    // FP16/BF16 storage with two-relaxation-time rates defaults to the
-    // shared-memory staged kernel: in 2D 512-node tiles with the stages chosen
-    // as above (2 stages and three blocks per SM on GB300, the fastest there),
-    // in 3D whole rows with 2 stages and two blocks per SM (385^3 FP16: 46.5
-    // GLUPS against 46.3 with 3 stages and 44.4 for the register kernel); the
-    // register kernel stays if the device cannot host it
-    if (!h->variant_chosen && !h->aa && (h->prec == TLBM_FP16_OFFSET || h->prec == TLBM_BF16_OFFSET) &&
-        h->kp.trt && set_staged(h, 0, h->dim == 3 ? 2 : 0) != TLBM_OK) {
-        h->staged = 0;
-        h->err[0] = 0;
-    }
+    pick_16bit(h);
     pick_multi(h);
     return TLBM_OK;
 }
@@ -692,7 +683,7 @@ static cudaError_t launch_step_raw(tlbm_t h, int parity, cudaStream_t s) {
         si.wait_ns = h->wait_ns;
         return launch_staged(h->dim, h->prec, h->staged_nc, src, dst, kp, si, h->staged_grid, h->staged_smem, s);
     }
-    if (h->flat) return launch_flat_f64(h->dim, h->aa ? (parity ? AA_ODD : AA_EVEN) : PULL, src, h->aa ? h->buf[0] : dst, kp, s);
+    if (h->flat) return launch_flat(h->dim, h->prec, h->aa ? (parity ? AA_ODD : AA_EVEN) : PULL, src, h->aa ? h->buf[0] : dst, kp, s);
     const int vec = h->vec;
     const int bx = h->bx, by = h->by, rows = h->rows;
     const int threads_x = (h->nx + vec - 1) / vec;
@@ -1294,6 +1285,42 @@ static int set_staged(tlbm_t h, int tile_width, int stages) {
     h->staged_grid = (int)std::min<long long>(tiles, (long long)per_sm * sms);
     drop_graph(h);
     return TLBM_OK;
+}
+
+// Step kernel of an FP16 or BF16 cell with two-relaxation-time rates whose
+// launches the caller has not chosen.
+// 2D, two buffers: the staged kernel, 512-node tiles with the stages chosen as
+// above (2 stages and three blocks per SM on GB300, the fastest there).
+// 3D, two buffers: the staged kernel (2 stages, two blocks per SM) takes a row per
+// tile and seven warps, so it is for rows that nearly fill those: 385^3 1250 us per
+// step against 1297, 448 x 193^2 346 and 352 (and 385 x 129^2 174 and 166); but
+// 321^3 881 and 798, 193^3 252 and 208, 65^3 45 and 17, 513 x 193^2 654 and 435.  Else warps inside rows: one node a
+// thread up to 4 M nodes, where a second one in flight per thread is worth less
+// than twice the warps, then node pairs (33^3 7.0 us against 12.0, 97^3 39 and 50,
+// 145^3 101 and 113, 161^3 135 and 134, 177^3 173 and 166).
+// 3D, in place: one thread per node in memory order for small cells and where
+// pairs leave over 1/16 of a row's last warps idle (step_3d_f16.cu; with none idle
+// pairs are faster: 192^3 196 us against 206, 320^3 821 and 919).
+static void pick_16bit(tlbm_t h) {
+    if (h->elem != 2 || !h->kp.trt || h->variant_chosen) return;
+    const double nodes = (double)h->nx * h->ny * h->nz;
+    const long long lanes = (h->nx + 63) / 64 * 64ll;
+    if (h->aa) {
+        h->flat = h->dim == 3 && nodes <= FLAT_NODES && (nodes <= 4e6 || 16ll * h->nx < 15 * lanes);
+        return;
+    }
+    if (h->dim == 2 || (h->nx >= 384 && h->nx <= 448)) {
+        // (the register kernel stays if the device cannot host the staged one)
+        if (set_staged(h, 0, h->dim == 3 ? 2 : 0) == TLBM_OK) return;
+        h->staged = 0;
+        h->err[0] = 0;
+    }
+    if (h->dim == 3 && nodes <= 4e6) {
+        h->vec = 1;
+        h->bx = 32;
+        h->by = 2;
+        h->kp.xmax_load = h->kp.L.P - 1;
+    }
 }
 
 // Several steps per launch: 2D two-buffer cells with two-relaxation-time rates

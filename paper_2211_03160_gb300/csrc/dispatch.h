@@ -21,9 +21,19 @@ bool step_variant_available(int dim, int prec, int vec, bool trt, int rows);
 // device function of a compiled variant (for cudaFuncGetAttributes), or nullptr
 const void* step_function(int dim, int prec, int vec, bool trt, int rows);
 
-// FP64 step with one thread per node in memory order, TRT form (mode: PULL, or
-// a half of an in-place pair, which reads and writes dst)
-cudaError_t launch_flat_f64(int dim, int mode, const void* src, void* dst, const KParams& p, cudaStream_t s);
+// step with one thread per node in memory order, TRT form: FP64, and the halves of
+// a 16-bit 3D in-place pair (mode: PULL, or a half of an in-place pair, which reads
+// and writes dst).  Cells of up to FLAT_NODES nodes (32-bit thread numbers).
+constexpr double FLAT_NODES = 4e9;
+cudaError_t launch_flat(int dim, int prec, int mode, const void* src, void* dst, const KParams& p, cudaStream_t s);
+template <int DIM, class S, int MODE>
+cudaError_t launch_flat_as(const void* src, void* dst, const KParams& p, cudaStream_t s) {
+    const long long n = (long long)p.L.nx * p.L.ny * p.L.nz;
+    const unsigned grid = (unsigned)((n + FLAT_THREADS - 1) / FLAT_THREADS);
+    step_flat_kernel<DIM, S, MODE><<<grid, FLAT_THREADS, 0, s>>>((const S*)src, (S*)dst, p);
+    return cudaGetLastError();
+}
+cudaError_t launch_flat_3d_f16(int prec, int mode, const void* src, void* dst, const KParams& p, cudaStream_t s);
 
 // shared-memory staged (TMA bulk copy) step, TRT form, FP32/FP16/BF16 storage,
 // nc = 4 or 8 consumer warps

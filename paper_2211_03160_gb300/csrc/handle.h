@@ -25,7 +25,7 @@ struct tlbm_s {
     int multi;                 // > 1: steps per launch of calls of MULTI_CALL steps or more
     int march;                 // > 0: by step_march.cu in segments of this many rows, else by step_multi.cu
     tlbm::MultiGeo mg;         // tile of the latter
-    int flat;                  // 1: FP64 kernel with one thread per node in memory order
+    int flat;                  // 1: the kernel with one thread per node in memory order
     int staged;                // 1: shared-memory staged (TMA bulk copy) kernel
     int variant_chosen;        // set by tlbm_set_variant / tlbm_set_staged: keep the caller's choice
     int staged_tw, staged_nc, staged_stages, staged_grid;

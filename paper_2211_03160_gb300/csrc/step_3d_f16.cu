@@ -28,6 +28,20 @@ cudaError_t launch_step_3d_f16(int prec, int vec, bool trt, int rows, const void
     return cudaErrorInvalidValue;
 }
 
+// Halves of an in-place pair with one thread per node, nodes in their order in
+// memory: 64 registers, and no lane idle at a row's end.  us per step, warps of
+// node pairs inside rows -> this kernel: 33^3 13.8 -> 8.4, 65^3 25.6 -> 16.7, 97^3
+// 52 -> 35, 129^3 96 -> 73, 193^3 245 -> 213, 257^3 525 -> 479, 385^3 1570 -> 1561.
+template <class S>
+static cudaError_t launch_flat_aa(int mode, const void* src, void* dst, const KParams& p, cudaStream_t s) {
+    if (mode == AA_EVEN) return launch_flat_as<3, S, AA_EVEN>(src, dst, p, s);
+    if (mode == AA_ODD) return launch_flat_as<3, S, AA_ODD>(src, dst, p, s);
+    return cudaErrorInvalidValue;
+}
+cudaError_t launch_flat_3d_f16(int prec, int mode, const void* src, void* dst, const KParams& p, cudaStream_t s) {
+    return prec == 2 ? launch_flat_aa<__half>(mode, src, dst, p, s) : launch_flat_aa<__nv_bfloat16>(mode, src, dst, p, s);
+}
+
 const void* func_step_3d_f16(int prec, int vec, bool trt, int rows) {
     if (prec == 2) {
         TLBM_STEP_FUNC(3, __half, 4, true)

@@ -45,21 +45,16 @@ const void* func_step_f64(int dim, int vec, bool trt, int rows) {
 // 20 % at 129.  us per step, warps inside rows -> this kernel: 193^3 3415 -> 2904,
 // 129^3 1097 -> 877, 65^3 174 -> 125; 129^2 13.3 -> 8.1, 513^2 76 -> 63, 2049^2
 // 944 -> 925, 4097^2 3682 -> 3681; in place the same.
-cudaError_t launch_flat_f64(int dim, int mode, const void* src, void* dst, const KParams& p, cudaStream_t s) {
-    const long long n = (long long)p.L.nx * p.L.ny * p.L.nz;
-    const unsigned grid = (unsigned)((n + FLAT_THREADS - 1) / FLAT_THREADS);
-    const double* a = (const double*)src;
-    double* b = (double*)dst;
-    if (dim == 2) {
-        if (mode == PULL) step_flat_kernel<2, double, PULL><<<grid, FLAT_THREADS, 0, s>>>(a, b, p);
-        else if (mode == AA_EVEN) step_flat_kernel<2, double, AA_EVEN><<<grid, FLAT_THREADS, 0, s>>>(a, b, p);
-        else step_flat_kernel<2, double, AA_ODD><<<grid, FLAT_THREADS, 0, s>>>(a, b, p);
-    } else {
-        if (mode == PULL) step_flat_kernel<3, double, PULL><<<grid, FLAT_THREADS, 0, s>>>(a, b, p);
-        else if (mode == AA_EVEN) step_flat_kernel<3, double, AA_EVEN><<<grid, FLAT_THREADS, 0, s>>>(a, b, p);
-        else step_flat_kernel<3, double, AA_ODD><<<grid, FLAT_THREADS, 0, s>>>(a, b, p);
-    }
-    return cudaGetLastError();
+template <int DIM>
+static cudaError_t launch_flat_f64(int mode, const void* src, void* dst, const KParams& p, cudaStream_t s) {
+    if (mode == PULL) return launch_flat_as<DIM, double, PULL>(src, dst, p, s);
+    if (mode == AA_EVEN) return launch_flat_as<DIM, double, AA_EVEN>(src, dst, p, s);
+    return launch_flat_as<DIM, double, AA_ODD>(src, dst, p, s);
+}
+
+cudaError_t launch_flat(int dim, int prec, int mode, const void* src, void* dst, const KParams& p, cudaStream_t s) {
+    if (prec == 0) return dim == 2 ? launch_flat_f64<2>(mode, src, dst, p, s) : launch_flat_f64<3>(mode, src, dst, p, s);
+    return launch_flat_3d_f16(prec, mode, src, dst, p, s);
 }
 
 const void* step_function(int dim, int prec, int vec, bool trt, int rows) {

@@ -266,6 +266,36 @@ def test_launch_choices_of_the_caller_stay(T, choice, n):  # noqa: F811
     s.close()
 
 
+@pytest.mark.parametrize("prec", [2, 3])
+@pytest.mark.parametrize("shape,walls,pm,inplace", [
+    ((3, 3, 3), 0, 0, False), ((33, 5, 7), 1, 0, False), ((65, 4, 3), 0, 5, False), ((31, 6, 4), 0, 1, False),
+    ((383, 5, 6), 0, 0, False), ((384, 5, 6), 0, 0, False), ((448, 6, 3), 1, 0, False), ((449, 6, 3), 0, 4, False),
+    ((160, 158, 158), 0, 0, False),
+    ((3, 3, 3), 0, 0, True), ((33, 5, 7), 1, 0, True), ((65, 4, 3), 0, 5, True), ((31, 6, 4), 0, 1, True),
+    ((161, 160, 162), 0, 0, True), ((192, 160, 140), 0, 0, True)])
+def test_16bit_3d_kernels_by_size_equal_node_pairs(T, shape, walls, pm, inplace, prec):  # noqa: F811
+    """The kernel a 3D FP16 or BF16 cell gets by its size (either side of each
+    border) steps bitwise as warps of node pairs inside a row."""
+    import torch
+
+    out = []
+    for pairs in (False, True):
+        s = T.Sim(*shape, lattice=D3, Ra=1e5, Pr=0.71, Ma=0.1, precision=prec, walls=walls, periodic_mask=pm,
+                  streaming=T.TLBM_STREAM_INPLACE if inplace else T.TLBM_STREAM_PULL)
+        if pairs:
+            s.set_variant(2, 2, 32, 1, 1)
+        s.init(3, 1e-2)
+        s.step(5)
+        n = shape[0] * shape[1] * shape[2]
+        if n < 10000:
+            out.append([torch.from_numpy(np.ascontiguousarray(q)) for q in s.get_populations()])
+        else:
+            m = s.macros()
+            out.append([m[k].cpu() for k in sorted(m)])
+        s.close()
+    assert all(torch.equal(a, b) for a, b in zip(*out))
+
+
 BOUNDS_SCRIPT = """
 import hashlib, json, sys
 sys.path.insert(0, {root!r})
