@@ -1297,7 +1297,8 @@ static int set_staged(tlbm_t h, int tile_width, int stages) {
 // 321^3 881 and 798, 193^3 252 and 208, 65^3 45 and 17, 513 x 193^2 654 and 435.  Else warps inside rows: one node a
 // thread up to 4 M nodes, where a second one in flight per thread is worth less
 // than twice the warps, then node pairs (33^3 7.0 us against 12.0, 97^3 39 and 50,
-// 145^3 101 and 113, 161^3 135 and 134, 177^3 173 and 166).
+// 145^3 101 and 113, 161^3 135 and 134, 177^3 173 and 166).  (Figures of this
+// comment: before the wall rules went face by face, which took 1 to 10 % off all.)
 // 3D, in place: one thread per node in memory order for small cells and where
 // pairs leave over 1/16 of a row's last warps idle (step_3d_f16.cu; with none idle
 // pairs are faster: 192^3 196 us against 206, 320^3 821 and 919).

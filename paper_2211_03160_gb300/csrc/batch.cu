@@ -100,8 +100,8 @@ __device__ __forceinline__ void batch_tile(const KParams* __restrict__ kps, cons
 // parameters only when its run of tiles enters that instance (one tile per
 // block staged them for every tile, a lookup and a 1.2 KB copy in front of
 // every 1024 nodes).
-template <int DIM, class S, int VEC, bool TRT, int ROWS = 1>
-__global__ void batch_step_kernel(const KParams* __restrict__ kps, const BatchInst* __restrict__ inst, int n,
+template <int DIM, class S, int VEC, bool TRT, int ROWS>
+__device__ __forceinline__ void batch_step_body(const KParams* __restrict__ kps, const BatchInst* __restrict__ inst, int n,
                                   int parity, long long tiles, int tpb) {
     __shared__ KParams sp;
     __shared__ int si;
@@ -116,6 +116,27 @@ __global__ void batch_step_kernel(const KParams* __restrict__ kps, const BatchIn
         }
         batch_run<DIM, S, VEC, TRT, false, ROWS>(inst, parity, b, sp, si);
     }
+}
+template <int DIM, class S, int VEC, bool TRT, int ROWS>
+__global__ void batch_step_kernel(const KParams* __restrict__ kps, const BatchInst* __restrict__ inst, int n,
+                                  int parity, long long tiles, int tpb) {
+    batch_step_body<DIM, S, VEC, TRT, ROWS>(kps, inst, n, parity, tiles, tpb);
+}
+// held to REGS registers
+template <int DIM, class S, int VEC, bool TRT, int ROWS, int REGS>
+__global__ void __maxnreg__(REGS) batch_step_kernel_cap(const KParams* __restrict__ kps, const BatchInst* __restrict__ inst,
+                                                        int n, int parity, long long tiles, int tpb) {
+    batch_step_body<DIM, S, VEC, TRT, ROWS>(kps, inst, n, parity, tiles, tpb);
+}
+// the caps keep blocks of up to 800, 288 and 352 threads launchable
+template <int DIM, class S, int VEC, bool TRT, int ROWS = 1>
+constexpr auto batch_step_fn() {
+    constexpr int cap = DIM != 2 || !TRT ? 0
+                        : sizeof(S) == 4 ? (VEC == 2 && ROWS == 1 ? 80 : 0)
+                        : sizeof(S) == 2 ? (VEC == 8 && ROWS == 1 ? 224 : VEC == 4 && ROWS == 2 ? 184 : 0)
+                                         : 0;
+    if constexpr (cap > 0) return &batch_step_kernel_cap<DIM, S, VEC, TRT, ROWS, cap>;
+    else return &batch_step_kernel<DIM, S, VEC, TRT, ROWS>;
 }
 
 // ------------------------------------------------------------------ persistent form
@@ -173,9 +194,9 @@ __device__ __forceinline__ bool grid_sync(GridSync* gs, int& ok, unsigned long l
 // instances in a fixed order (block k takes tiles k, k + G, k + 2G, ...) and meet
 // at a grid barrier between steps.
 template <int DIM, class S, int VEC, bool TRT>
-__global__ void batch_persistent_kernel(const KParams* __restrict__ kps, const BatchInst* __restrict__ inst, int n,
-                                        long long tiles, int parity0, int steps, GridSync* gs,
-                                        unsigned long long wait_ns) {
+__device__ __forceinline__ void batch_persistent_body(const KParams* __restrict__ kps, const BatchInst* __restrict__ inst,
+                                                      int n, long long tiles, int parity0, int steps, GridSync* gs,
+                                                      unsigned long long wait_ns) {
     __shared__ KParams sp;
     __shared__ int si;
     __shared__ int ok;
@@ -187,6 +208,25 @@ __global__ void batch_persistent_kernel(const KParams* __restrict__ kps, const B
         }
         if (st + 1 < steps && !grid_sync(gs, ok, wait_ns)) return;
     }
+}
+template <int DIM, class S, int VEC, bool TRT>
+__global__ void batch_persistent_kernel(const KParams* __restrict__ kps, const BatchInst* __restrict__ inst, int n,
+                                        long long tiles, int parity0, int steps, GridSync* gs,
+                                        unsigned long long wait_ns) {
+    batch_persistent_body<DIM, S, VEC, TRT>(kps, inst, n, tiles, parity0, steps, gs, wait_ns);
+}
+template <int DIM, class S, int VEC, bool TRT, int REGS>
+__global__ void __maxnreg__(REGS) batch_persistent_kernel_cap(const KParams* __restrict__ kps,
+                                                              const BatchInst* __restrict__ inst, int n, long long tiles,
+                                                              int parity0, int steps, GridSync* gs,
+                                                              unsigned long long wait_ns) {
+    batch_persistent_body<DIM, S, VEC, TRT>(kps, inst, n, tiles, parity0, steps, gs, wait_ns);
+}
+// (the cap keeps blocks of up to 800 threads launchable)
+template <int DIM, class S, int VEC, bool TRT>
+constexpr auto batch_persistent_fn() {
+    if constexpr (DIM == 2 && TRT && sizeof(S) == 4 && VEC == 2) return &batch_persistent_kernel_cap<DIM, S, VEC, TRT, 80>;
+    else return &batch_persistent_kernel<DIM, S, VEC, TRT>;
 }
 
 // Persistent launch parameters (steps > 0 selects the persistent kernel: grid
@@ -203,7 +243,7 @@ struct Persist {
     if (dim == DIM && prec == PREC && vec == VEC && trt == TRT && rows == 1) {                      \
         if (pp && pp->per_sm_out)                                                                   \
             return cudaOccupancyMaxActiveBlocksPerMultiprocessor(                                   \
-                pp->per_sm_out, batch_persistent_kernel<DIM, S, VEC, TRT>, block.x * block.y, 0);    \
+                pp->per_sm_out, batch_persistent_fn<DIM, S, VEC, TRT>(), block.x * block.y, 0);    \
         if (launch && pp && pp->steps > 0) {                                                        \
             const KParams* a0 = kps;                                                                \
             const BatchInst* a1 = inst;                                                             \
@@ -213,11 +253,11 @@ struct Persist {
             GridSync* a6 = pp->gs;                                                                  \
             unsigned long long a7 = pp->wait_ns;                                                    \
             void* args[] = {&a0, &a1, &a2, &a3, &a4, &a5, &a6, &a7};                                \
-            return cudaLaunchCooperativeKernel((const void*)batch_persistent_kernel<DIM, S, VEC, TRT>, \
+            return cudaLaunchCooperativeKernel((const void*)batch_persistent_fn<DIM, S, VEC, TRT>(), \
                                                dim3((unsigned)grid), block, args, 0, s);            \
         }                                                                                           \
         if (launch)                                                                                 \
-            batch_step_kernel<DIM, S, VEC, TRT>                                                     \
+            batch_step_fn<DIM, S, VEC, TRT>()                                                       \
                 <<<(grid + tpb - 1) / tpb, block, 0, s>>>(kps, inst, n, parity, grid, tpb);         \
         return launch ? cudaGetLastError() : cudaSuccess;                                           \
     }
@@ -227,7 +267,7 @@ struct Persist {
     if (dim == DIM && prec == PREC && vec == VEC && trt && rows == ROWS) {                           \
         if (pp) return cudaErrorInvalidValue;                                                         \
         if (launch)                                                                                   \
-            batch_step_kernel<DIM, S, VEC, true, ROWS>                                                \
+            batch_step_fn<DIM, S, VEC, true, ROWS>()                                                  \
                 <<<(grid + tpb - 1) / tpb, block, 0, s>>>(kps, inst, n, parity, grid, tpb);           \
         return launch ? cudaGetLastError() : cudaSuccess;                                             \
     }

@@ -953,8 +953,9 @@ constexpr int FLAT_THREADS = 128;
 // the next AA_EVEN half reads (the node's own slot of the opposite direction
 // for a wall, the image's own slot for a periodic face).
 // RAW: flow values are f_i as stored (FP64 with the two-relaxation-time
-// collision) rather than deviations.
-template <class LS, bool THERMAL, int i, class S, class C, int MODE, bool RAW>
+// collision) rather than deviations.  WALLED: the caller knows that the value, if
+// it leaves the cell, meets a wall.
+template <class LS, bool THERMAL, int i, class S, class C, int MODE, bool RAW, bool WALLED = false>
 __device__ __forceinline__ void ghost_write(S* __restrict__ base, const KParams& p, int x, int y, int z, C val,
                                             C scale, uint32_t salt) {
     constexpr int ex = LS::e(i, 0), ey = LS::e(i, 1), ez = LS::e(i, 2);
@@ -965,7 +966,7 @@ __device__ __forceinline__ void ghost_write(S* __restrict__ base, const KParams&
     const bool oy = dy < 0 || dy >= L.ny;
     const bool oz = (ez != 0) && (dz < 0 || dz >= L.nz);
     if (!(ox || oy || oz)) return;
-    const bool wall = (ox && !(p.periodic & 1)) || (oy && !(p.periodic & 2)) || (oz && !(p.periodic & 4));
+    const bool wall = WALLED || (ox && !(p.periodic & 1)) || (oy && !(p.periodic & 2)) || (oz && !(p.periodic & 4));
     constexpr int o = LS::opp(i);
     if (wall) {
         // bounce-back: the value returns to the node as f_ibar of the next step
@@ -1073,34 +1074,125 @@ __device__ __forceinline__ void pull_node_vec(const S* __restrict__ own, const K
     });
 }
 
-// Wall and periodic rules for the nodes of a thread at the edge of the cell.
-// Kept out of line: only edge threads call it, and its fully unrolled body
-// would otherwise crowd the instruction cache of the hot path.
-template <int DIM, class S, int VEC, class C, int MODE, bool RAW>
-__device__ __noinline__ void edge_writes(S* __restrict__ dst, const KParams& p, int x0, int y, int z,
-                                         const C* __restrict__ post, uint32_t salt) {
+// Wall or periodic rule of the populations of node (x, y, z) that leave through
+// the face (AXIS, SIDE) it lies on: those with e_AXIS = SIDE, value val(j) (all
+// numbered flow first).  WALLED: that axis is not periodic, so they meet a wall
+// whatever else they cross.
+template <int DIM, class S, class C, int MODE, bool RAW, int AXIS, int SIDE, bool WALLED, class Val>
+__device__ __forceinline__ void face_writes(S* __restrict__ dst, const KParams& p, int x, int y, int z, Val val, uint32_t salt) {
     using LF = typename Lat<DIM>::F;
     using LG = typename Lat<DIM>::G;
-    constexpr int QF = LF::Q, QG = LG::Q;
     const C scale = ScaleOf<C>::s(p);
-    S* __restrict__ gdst = dst + (long long)QF * p.L.plane;
+    S* __restrict__ gdst = dst + (long long)LF::Q * p.L.plane;
+    static_for<LF::Q>([&](auto ii) {
+        constexpr int i = decltype(ii)::value;
+        if constexpr (LF::e(i, AXIS) == SIDE)
+            ghost_write<LF, false, i, S, C, MODE, RAW, WALLED>(dst, p, x, y, z, val(ii), scale, salt);
+    });
+    static_for<LG::Q>([&](auto ii) {
+        constexpr int i = decltype(ii)::value;
+        if constexpr (LG::e(i, AXIS) == SIDE)
+            ghost_write<LG, true, i, S, C, MODE, RAW, WALLED>(gdst, p, x, y, z, val(std::integral_constant<int, LF::Q + i>{}), scale, salt);
+    });
+}
+template <int DIM, class S, class C, int MODE, bool RAW, int AXIS, int SIDE, bool CLOSED, class Val>
+__device__ __forceinline__ void any_face(S* __restrict__ dst, const KParams& p, int x, int y, int z, Val val, uint32_t salt) {
+    if (!CLOSED && (p.periodic & (1 << AXIS))) face_writes<DIM, S, C, MODE, RAW, AXIS, SIDE, false>(dst, p, x, y, z, val, salt);
+    else face_writes<DIM, S, C, MODE, RAW, AXIS, SIDE, true>(dst, p, x, y, z, val, salt);
+}
+
+// The rules of a thread's nodes at the edge of the cell, one face after the other
+// (a population that crosses two faces is written twice, with the same value).
+// Kept out of line: only edge threads call them, and their unrolled bodies would
+// crowd the instruction cache of the hot path.  A step of a small cell lasts as
+// long as its face threads, and in a large one they end the warps of a row late:
+// going through all populations of such a node instead of the 4 (2D) or 6 (3D)
+// that can leave through a face cost 3D FP32 6.8 us per step at 33^3 against 4.5
+// now, 65^3 17.5 and 12.3, 385^3 FP16 1250 and 1113; 2D in place FP32 117 x 109 10
+// and 4.9; with periodic x, 193^3 FP16 480 and 227, 385^3 4027 and 1457.
+// One face per call, its populations' values handed over (post: those of all VEC
+// nodes, in their order):
+template <class LS, int AXIS, int SIDE>
+__host__ __device__ constexpr int leaving(int n) {  // populations with e_AXIS = SIDE below n
+    int k = 0;
+    for (int i = 0; i < n; ++i) k += LS::e(i, AXIS) == SIDE;
+    return k;
+}
+template <int DIM, int AXIS, int SIDE>
+__host__ __device__ constexpr int leaving_index(int j) {  // of population j (flow first)
+    using LF = typename Lat<DIM>::F;
+    using LG = typename Lat<DIM>::G;
+    return j < LF::Q ? leaving<LF, AXIS, SIDE>(j) : leaving<LF, AXIS, SIDE>(LF::Q) + leaving<LG, AXIS, SIDE>(j - LF::Q);
+}
+template <int DIM, class S, int VEC, class C, int MODE, bool RAW, int AXIS, int SIDE, bool WALLED>
+__device__ __noinline__ void face_call(S* __restrict__ dst, const KParams& p, int x0, int y, int z,
+                                       const C* __restrict__ post, uint32_t salt) {
+#pragma unroll(WALLED && VEC <= 4 ? VEC : 1)
+    for (int k = 0; k < VEC; ++k) {
+        if (x0 + k >= p.L.nx) break;
+        face_writes<DIM, S, C, MODE, RAW, AXIS, SIDE, WALLED>(
+            dst, p, x0 + k, y, z, [&](auto jj) { return post[leaving_index<DIM, AXIS, SIDE>(decltype(jj)::value) * VEC + k]; }, salt);
+    }
+}
+template <int DIM, class S, int VEC, class C, bool KS, int MODE, int AXIS, int SIDE, bool CLOSED>
+__device__ __forceinline__ void face(S* __restrict__ dst, const KParams& p, int x0, int y, int z,
+                                     const C (&f)[Lat<DIM>::F::Q][VEC], const C (&g)[Lat<DIM>::G::Q][VEC], uint32_t salt) {
+    using LF = typename Lat<DIM>::F;
+    using LG = typename Lat<DIM>::G;
+    constexpr bool RAW = KS && !Storage<S>::offset;
+    const C un = KS && Storage<S>::offset ? ScaleOf<C>::inv(p) : C(1);  // the wall rules take unscaled values
+    C post[leaving_index<DIM, AXIS, SIDE>(LF::Q + LG::Q) * VEC];
+    static_for<LF::Q + LG::Q>([&](auto jj) {
+        constexpr int j = decltype(jj)::value;
+        constexpr bool flow = j < LF::Q;
+        if constexpr ((flow ? LF::e(flow ? j : 0, AXIS) : LG::e(flow ? 0 : j - LF::Q, AXIS)) == SIDE) {
+#pragma unroll
+            for (int k = 0; k < VEC; ++k) {
+                const C v = flow ? f[flow ? j : 0][k] : g[flow ? 0 : j - LF::Q][k];
+                post[leaving_index<DIM, AXIS, SIDE>(j) * VEC + k] = KS && Storage<S>::offset ? v * un : v;
+            }
+        }
+    });
+    if (!CLOSED && (p.periodic & (1 << AXIS))) face_call<DIM, S, VEC, C, MODE, RAW, AXIS, SIDE, false>(dst, p, x0, y, z, post, salt);
+    else face_call<DIM, S, VEC, C, MODE, RAW, AXIS, SIDE, true>(dst, p, x0, y, z, post, salt);
+}
+
+// All faces in one call, for FP64: bound by the FP64 pipe, its warps gain little
+// from shorter face threads and lose more by the branches above (193^3 2945 us per
+// step against 2901, 1025^2 235.6 and 231.8; 33^3 19.5 and 20.2).
+template <int DIM, class S, int VEC, class C, int MODE, bool RAW, bool CLOSED>
+__device__ __noinline__ void edge_writes(S* __restrict__ dst, const KParams& p, int x0, int y, int z,
+                                         const C* __restrict__ post, uint32_t salt) {
+    const Layout& L = p.L;
+    const bool ylo = y == 0, yhi = y == L.ny - 1, zlo = DIM == 3 && z == 0, zhi = DIM == 3 && z == L.nz - 1;
+#pragma unroll 1
     for (int k = 0; k < VEC; ++k) {
         const int x = x0 + k;
-        if (x >= p.L.nx) break;
-        static_for<QF>([&](auto ii) {
-            constexpr int i = decltype(ii)::value;
-            ghost_write<LF, false, i, S, C, MODE, RAW>(dst, p, x, y, z, post[i * VEC + k], scale, salt);
-        });
-        static_for<QG>([&](auto ii) {
-            constexpr int i = decltype(ii)::value;
-            ghost_write<LG, true, i, S, C, MODE, RAW>(gdst, p, x, y, z, post[(QF + i) * VEC + k], scale, salt);
-        });
+        if (x >= L.nx) break;
+        auto val = [&](auto jj) { return post[decltype(jj)::value * VEC + k]; };
+        if (x == 0) any_face<DIM, S, C, MODE, RAW, 0, -1, CLOSED>(dst, p, x, y, z, val, salt);
+        if (x == L.nx - 1) any_face<DIM, S, C, MODE, RAW, 0, 1, CLOSED>(dst, p, x, y, z, val, salt);
+        if (ylo) any_face<DIM, S, C, MODE, RAW, 1, -1, CLOSED>(dst, p, x, y, z, val, salt);
+        if (yhi) any_face<DIM, S, C, MODE, RAW, 1, 1, CLOSED>(dst, p, x, y, z, val, salt);
+        if constexpr (DIM == 3) {
+            if (zlo) any_face<DIM, S, C, MODE, RAW, 2, -1, CLOSED>(dst, p, x, y, z, val, salt);
+            if (zhi) any_face<DIM, S, C, MODE, RAW, 2, 1, CLOSED>(dst, p, x, y, z, val, salt);
+        }
     }
 }
 
+// v[k], k < VEC, from registers
+template <int VEC, class C>
+__device__ __forceinline__ C pick(const C (&v)[VEC], int k) {
+    C val = v[0];
+#pragma unroll
+    for (int kk = 1; kk < VEC; ++kk)
+        if (k == kk) val = v[kk];
+    return val;
+}
+
 // The populations with e_x = SIDE of node k of a thread's VEC nodes, for a node
-// on the x face SIDE of an inner row (y, z away from the faces) with x not
-// periodic: those, and only those, leave the cell, through that face.
+// on the x face SIDE with x not periodic: they leave the cell through that face.
 template <class LS, bool THERMAL, int SIDE, class S, int VEC, class C, bool KS, int MODE = PULL>
 __device__ __forceinline__ void x_face(S* __restrict__ base, const KParams& p, int x, int y, int z, int k,
                                        const C (&v)[LS::Q][VEC], uint32_t salt) {
@@ -1109,20 +1201,15 @@ __device__ __forceinline__ void x_face(S* __restrict__ base, const KParams& p, i
     static_for<LS::Q>([&](auto ii) {
         constexpr int i = decltype(ii)::value;
         if constexpr (LS::e(i, 0) == SIDE) {
-            C val = v[i][0];
-#pragma unroll
-            for (int kk = 1; kk < VEC; ++kk)
-                if (k == kk) val = v[i][kk];
-            ghost_write<LS, THERMAL, i, S, C, MODE, KS && !Storage<S>::offset>(base, p, x, y, z, KS && Storage<S>::offset ? val * un : val, scale, salt);
+            const C val = pick<VEC>(v[i], k);
+            ghost_write<LS, THERMAL, i, S, C, MODE, KS && !Storage<S>::offset, true>(base, p, x, y, z, KS && Storage<S>::offset ? val * un : val, scale, salt);
         }
     });
 }
 
 // Wall and periodic rules for the post-collision values of a thread's nodes.
-// Threads holding x = 0 or x = nx - 1 of an inner row only have the x-face
-// populations to place (inline); rows on a y or z face, and periodic x, take the
-// general out-of-line path.
-template <int DIM, class S, int VEC, class C, bool KS, int MODE = PULL>
+// Values that meet a wall in x are placed inline, the others out of line.  CLOSED: no axis is periodic.
+template <int DIM, class S, int VEC, class C, bool KS, int MODE = PULL, bool CLOSED = false>
 __device__ __forceinline__ void wall_writes(S* __restrict__ dst, const KParams& p, int x0, int y, int z,
                                             const C (&f)[Lat<DIM>::F::Q][VEC], const C (&g)[Lat<DIM>::G::Q][VEC],
                                             uint32_t salt) {
@@ -1132,18 +1219,47 @@ __device__ __forceinline__ void wall_writes(S* __restrict__ dst, const KParams& 
     const Layout& L = p.L;
     const bool xlo = x0 == 0, xhi = x0 + VEC >= L.nx;
     const bool face_row = (y == 0) || (y == L.ny - 1) || (DIM == 3 && (z == 0 || z == L.nz - 1));
-    if (face_row || ((xlo || xhi) && (p.periodic & 1))) {
-        C post[(QF + QG) * VEC];
-        const C un = KS && Storage<S>::offset ? ScaleOf<C>::inv(p) : C(1);  // the wall rules take unscaled values
+    const bool x_wraps = !CLOSED && (xlo || xhi) && (p.periodic & 1);
+    if constexpr (sizeof(S) == 8) {
+        if (face_row || x_wraps) {
+            C post[(QF + QG) * VEC];
 #pragma unroll
-        for (int k = 0; k < VEC; ++k) {
+            for (int k = 0; k < VEC; ++k) {
 #pragma unroll
-            for (int i = 0; i < QF; ++i) post[i * VEC + k] = KS && Storage<S>::offset ? f[i][k] * un : f[i][k];
+                for (int i = 0; i < QF; ++i) post[i * VEC + k] = f[i][k];
 #pragma unroll
-            for (int i = 0; i < QG; ++i) post[(QF + i) * VEC + k] = KS && Storage<S>::offset ? g[i][k] * un : g[i][k];
+                for (int i = 0; i < QG; ++i) post[(QF + i) * VEC + k] = g[i][k];
+            }
+            edge_writes<DIM, S, VEC, C, MODE, KS && !Storage<S>::offset, CLOSED>(dst, p, x0, y, z, post, salt);
+            return;
         }
-        edge_writes<DIM, S, VEC, C, MODE, KS && !Storage<S>::offset>(dst, p, x0, y, z, post, salt);
-        return;
+    } else {
+        if (face_row) {
+            if (y == 0) face<DIM, S, VEC, C, KS, MODE, 1, -1, CLOSED>(dst, p, x0, y, z, f, g, salt);
+            if (y == L.ny - 1) face<DIM, S, VEC, C, KS, MODE, 1, 1, CLOSED>(dst, p, x0, y, z, f, g, salt);
+            if constexpr (DIM == 3) {
+                if (z == 0) face<DIM, S, VEC, C, KS, MODE, 2, -1, CLOSED>(dst, p, x0, y, z, f, g, salt);
+                if (z == L.nz - 1) face<DIM, S, VEC, C, KS, MODE, 2, 1, CLOSED>(dst, p, x0, y, z, f, g, salt);
+            }
+        }
+        if (x_wraps) {
+            C f1[QF][1], g1[QG][1];
+            if (xlo) {
+#pragma unroll
+                for (int i = 0; i < QF; ++i) f1[i][0] = f[i][0];
+#pragma unroll
+                for (int i = 0; i < QG; ++i) g1[i][0] = g[i][0];
+                face<DIM, S, 1, C, KS, MODE, 0, -1, false>(dst, p, 0, y, z, f1, g1, salt);
+            }
+            if (xhi) {
+#pragma unroll
+                for (int i = 0; i < QF; ++i) f1[i][0] = pick<VEC>(f[i], L.nx - 1 - x0);
+#pragma unroll
+                for (int i = 0; i < QG; ++i) g1[i][0] = pick<VEC>(g[i], L.nx - 1 - x0);
+                face<DIM, S, 1, C, KS, MODE, 0, 1, false>(dst, p, L.nx - 1, y, z, f1, g1, salt);
+            }
+            return;
+        }
     }
     S* __restrict__ gdst = dst + (long long)QF * L.plane;
     if (xlo) {
@@ -1419,8 +1535,8 @@ template <int DIM, class S, int VEC, bool TRT, int MODE>
 __global__ void step_kernel_aa(S* buf, const KParams p) {
     step_block_aa<DIM, S, VEC, TRT, MODE>(buf, p, blockIdx.x, blockIdx.y, blockIdx.z);
 }
-template <int DIM, class S, int VEC, bool TRT, int MODE>
-__global__ void __maxnreg__(96) step_kernel_aa_r96(S* buf, const KParams p) {
+template <int DIM, class S, int VEC, bool TRT, int MODE, int REGS>
+__global__ void __maxnreg__(REGS) step_kernel_aa_cap(S* buf, const KParams p) {
     step_block_aa<DIM, S, VEC, TRT, MODE>(buf, p, blockIdx.x, blockIdx.y, blockIdx.z);
 }
 
@@ -1587,18 +1703,24 @@ template <int DIM, class S, int VEC, bool TRT, int ROWS>
 __global__ void step_kernel_rows(const S* __restrict__ src, S* __restrict__ dst, const KParams p) {
     step_rows_block<DIM, S, VEC, TRT, ROWS>(src, dst, p, blockIdx.x, blockIdx.y, blockIdx.z);
 }
+template <int DIM, class S, int VEC, bool TRT, int ROWS, int REGS>
+__global__ void __maxnreg__(REGS) step_kernel_rows_cap(const S* __restrict__ src, S* __restrict__ dst, const KParams p) {
+    step_rows_block<DIM, S, VEC, TRT, ROWS>(src, dst, p, blockIdx.x, blockIdx.y, blockIdx.z);
+}
 
 template <int DIM, class S, int VEC, bool TRT>
 __global__ void step_kernel(const S* __restrict__ src, S* __restrict__ dst, const KParams p) {
     step_block<DIM, S, VEC, TRT>(src, dst, p, blockIdx.x, blockIdx.y, blockIdx.z);
 }
 
-// The same kernels held to 96 registers per thread.  For the 3D two-node
+// The same kernels held to REGS registers per thread: where the compiler would
+// take more than leaves blocks of up to 1024 threads (64) or the kernel's largest
+// launchable, and 96 for the 3D two-node kernels.  For the 3D two-node
 // FP16/BF16 variants the extra resident warps (21 instead of 16 per SM with
 // one-warp blocks) outweigh the few values the cap spills: 45.1 instead of
 // 43.0 GLUPS at 385^3 on GB300, same box, same process.
-template <int DIM, class S, int VEC, bool TRT>
-__global__ void __maxnreg__(96) step_kernel_r96(const S* __restrict__ src, S* __restrict__ dst, const KParams p) {
+template <int DIM, class S, int VEC, bool TRT, int REGS>
+__global__ void __maxnreg__(REGS) step_kernel_cap(const S* __restrict__ src, S* __restrict__ dst, const KParams p) {
     step_block<DIM, S, VEC, TRT>(src, dst, p, blockIdx.x, blockIdx.y, blockIdx.z);
 }
 

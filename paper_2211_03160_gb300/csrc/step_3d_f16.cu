@@ -6,23 +6,23 @@ cudaError_t launch_step_3d_f16(int prec, int vec, bool trt, int rows, const void
                         dim3 grid, dim3 block, cudaStream_t s) {
     if (prec == 2) {
         TLBM_STEP_CASE(3, __half, 4, true)
-        TLBM_STEP96_CASE(3, __half, 2, true)
-        TLBM_STEP_CASE(3, __half, 1, true)
+        TLBM_STEPCAP_CASE(3, __half, 2, true, 96)
+        TLBM_STEPCAP_CASE(3, __half, 1, true, 64)
         TLBM_STEP_CASE(3, __half, 4, false)
         TLBM_ROWS_CASE(3, __half, 1, 2)
-        TLBM_ROWS_CASE(3, __half, 1, 4)
-        TLBM_AA96_CASE(3, __half, 2, true)
-        TLBM_AA_CASE(3, __half, 1, true)
+        TLBM_ROWSCAP_CASE(3, __half, 1, 4, 128)
+        TLBM_AACAP_CASE(3, __half, 2, true, 96)
+        TLBM_AACAP_CASE(3, __half, 1, true, 64)
         TLBM_AA_CASE(3, __half, 2, false)
     } else {
         TLBM_STEP_CASE(3, __nv_bfloat16, 4, true)
-        TLBM_STEP96_CASE(3, __nv_bfloat16, 2, true)
-        TLBM_STEP_CASE(3, __nv_bfloat16, 1, true)
+        TLBM_STEPCAP_CASE(3, __nv_bfloat16, 2, true, 96)
+        TLBM_STEPCAP_CASE(3, __nv_bfloat16, 1, true, 64)
         TLBM_STEP_CASE(3, __nv_bfloat16, 4, false)
         TLBM_ROWS_CASE(3, __nv_bfloat16, 1, 2)
-        TLBM_ROWS_CASE(3, __nv_bfloat16, 1, 4)
-        TLBM_AA96_CASE(3, __nv_bfloat16, 2, true)
-        TLBM_AA_CASE(3, __nv_bfloat16, 1, true)
+        TLBM_ROWSCAP_CASE(3, __nv_bfloat16, 1, 4, 128)
+        TLBM_AACAP_CASE(3, __nv_bfloat16, 2, true, 96)
+        TLBM_AACAP_CASE(3, __nv_bfloat16, 1, true, 64)
         TLBM_AA_CASE(3, __nv_bfloat16, 2, false)
     }
     return cudaErrorInvalidValue;
@@ -31,7 +31,8 @@ cudaError_t launch_step_3d_f16(int prec, int vec, bool trt, int rows, const void
 // Halves of an in-place pair with one thread per node, nodes in their order in
 // memory: 64 registers, and no lane idle at a row's end.  us per step, warps of
 // node pairs inside rows -> this kernel: 33^3 13.8 -> 8.4, 65^3 25.6 -> 16.7, 97^3
-// 52 -> 35, 129^3 96 -> 73, 193^3 245 -> 213, 257^3 525 -> 479, 385^3 1570 -> 1561.
+// 52 -> 35, 129^3 96 -> 73, 193^3 245 -> 213, 257^3 525 -> 479, 385^3 1570 -> 1561
+// (since then the wall rules have taken another 3.4 us off 33^3 and 11 off 193^3).
 template <class S>
 static cudaError_t launch_flat_aa(int mode, const void* src, void* dst, const KParams& p, cudaStream_t s) {
     if (mode == AA_EVEN) return launch_flat_as<3, S, AA_EVEN>(src, dst, p, s);
@@ -45,23 +46,23 @@ cudaError_t launch_flat_3d_f16(int prec, int mode, const void* src, void* dst, c
 const void* func_step_3d_f16(int prec, int vec, bool trt, int rows) {
     if (prec == 2) {
         TLBM_STEP_FUNC(3, __half, 4, true)
-        TLBM_STEP96_FUNC(3, __half, 2, true)
-        TLBM_STEP_FUNC(3, __half, 1, true)
+        TLBM_STEPCAP_FUNC(3, __half, 2, true, 96)
+        TLBM_STEPCAP_FUNC(3, __half, 1, true, 64)
         TLBM_STEP_FUNC(3, __half, 4, false)
         TLBM_ROWS_FUNC(3, __half, 1, 2)
-        TLBM_ROWS_FUNC(3, __half, 1, 4)
-        TLBM_AA96_FUNC(3, __half, 2, true)
-        TLBM_AA_FUNC(3, __half, 1, true)
+        TLBM_ROWSCAP_FUNC(3, __half, 1, 4, 128)
+        TLBM_AACAP_FUNC(3, __half, 2, true, 96)
+        TLBM_AACAP_FUNC(3, __half, 1, true, 64)
         TLBM_AA_FUNC(3, __half, 2, false)
     } else {
         TLBM_STEP_FUNC(3, __nv_bfloat16, 4, true)
-        TLBM_STEP96_FUNC(3, __nv_bfloat16, 2, true)
-        TLBM_STEP_FUNC(3, __nv_bfloat16, 1, true)
+        TLBM_STEPCAP_FUNC(3, __nv_bfloat16, 2, true, 96)
+        TLBM_STEPCAP_FUNC(3, __nv_bfloat16, 1, true, 64)
         TLBM_STEP_FUNC(3, __nv_bfloat16, 4, false)
         TLBM_ROWS_FUNC(3, __nv_bfloat16, 1, 2)
-        TLBM_ROWS_FUNC(3, __nv_bfloat16, 1, 4)
-        TLBM_AA96_FUNC(3, __nv_bfloat16, 2, true)
-        TLBM_AA_FUNC(3, __nv_bfloat16, 1, true)
+        TLBM_ROWSCAP_FUNC(3, __nv_bfloat16, 1, 4, 128)
+        TLBM_AACAP_FUNC(3, __nv_bfloat16, 2, true, 96)
+        TLBM_AACAP_FUNC(3, __nv_bfloat16, 1, true, 64)
         TLBM_AA_FUNC(3, __nv_bfloat16, 2, false)
     }
     return nullptr;

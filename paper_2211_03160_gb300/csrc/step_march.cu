@@ -322,7 +322,7 @@ __device__ __forceinline__ void march_strip(const S* __restrict__ src, S* __rest
             for (int i = 0; i < QF; ++i) { fw[i][0] = f[i].x; fw[i][1] = f[i].y; }
 #pragma unroll
             for (int i = 0; i < QG; ++i) { gw[i][0] = g[i].x; gw[i][1] = g[i].y; }
-            wall_writes<2, S, 2, float, true>(dst, full, x, y, 0, fw, gw, salt);
+            wall_writes<2, S, 2, float, true, PULL, true>(dst, full, x, y, 0, fw, gw, salt);
         }
     }
 }
