@@ -527,7 +527,7 @@ __host__ __device__ constexpr int axis_pop(int a) {
 // value takes one rounding at its own ulp.  (Folding the weights into S as well
 // saves another 15 % of the instructions, but then the error of u against an
 // exact evaluation grows from 1.2e-15 to 4e-15 after 16 steps at 4097^2.)
-// 114 FP64 instructions per node in 2D and 216 in 3D, against 217 and 488 of the
+// 113 FP64 instructions per node in 2D and 213 in 3D, against 217 and 488 of the
 // uncontracted pairwise form (K0, Ks and Ka above evaluated term by term).  The
 // FP64 pipe bounds both (530 G instructions/s): 4097^2 6.63 -> 3.69 ms per step,
 // 193^3 6.29 -> 3.43 ms.
