@@ -945,6 +945,12 @@ __device__ __forceinline__ void pull_row(const S* __restrict__ q, int lane, C (&
 constexpr int PULL = 0, AA_EVEN = 1, AA_ODD = 2;
 constexpr int FLAT_THREADS = 128;
 
+// Anti-bounce-back at a wall of temperature Tw: omega Tw - val, in operations that
+// the compiler neither contracts nor splits, so that every kernel returns the same
+// bits whatever its translation unit's flags (FP64: two roundings, FP32: one).
+__device__ __forceinline__ double anti_bounce_back(double val, double omega, double Tw) { return dsub(dmul(omega, Tw), val); }
+__device__ __forceinline__ float anti_bounce_back(float val, float omega, float Tw) { return __fmaf_rn(omega, Tw, -val); }
+
 // Write the post-collision value `val` of population i (set LS, flow or
 // thermal) of node (x, y, z) where the next step will read it, if it leaves
 // the cell.  THERMAL selects the temperature rules of §2.2.  PULL: into the
@@ -977,7 +983,7 @@ __device__ __forceinline__ void ghost_write(S* __restrict__ base, const KParams&
             if (ax == p.heat_axis) {
                 const bool hi = ox ? (dx >= L.nx) : (oy ? (dy >= L.ny) : (dz >= L.nz));
                 const C Tw = hi ? PV<C>::Tc(p) : PV<C>::Th(p);
-                out = -val + PV<C>::omega(p) * Tw;  // anti-bounce-back
+                out = anti_bounce_back(val, PV<C>::omega(p), Tw);
             }
         }
         // written by PULL: slot (x + e_i) of plane ibar, where the node pulls

@@ -113,7 +113,7 @@ __device__ __forceinline__ uint32_t march_hi(uint32_t w, uint32_t v) { return __
 template <class PT>
 __device__ __forceinline__ float march_rule(float v, bool iso, const PT& p, float Tw) {
     const float val = v * ScaleOf<float>::inv(p);
-    return (iso ? -val + p.omegaf * Tw : val) * ScaleOf<float>::s(p);
+    return (iso ? anti_bounce_back(val, p.omegaf, Tw) : val) * ScaleOf<float>::s(p);
 }
 template <class PT>
 __device__ __forceinline__ float2 march_rule(float2 v, bool iso, const PT& p, float Tw) {

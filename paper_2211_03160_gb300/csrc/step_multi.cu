@@ -99,7 +99,7 @@ __device__ __forceinline__ void multi_ghost(S* sm, const KParams& p, const Multi
         if constexpr (THERMAL) {
             if ((ox ? 0 : 1) == p.heat_axis) {
                 const bool hi = ox ? x + ex >= p.L.nx : y + ey >= p.L.ny;
-                out = -val + PV<C>::omega(p) * (hi ? PV<C>::Tc(p) : PV<C>::Th(p));
+                out = anti_bounce_back(val, PV<C>::omega(p), hi ? PV<C>::Tc(p) : PV<C>::Th(p));
             }
         }
         S v;
