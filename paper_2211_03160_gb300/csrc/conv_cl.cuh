@@ -440,7 +440,10 @@ size_t wgrad_cl_smem(int GX, int GY, int Wv, int NS) {
     return 1024 + (reach > all ? reach : all);
 }
 // three tiles in shared memory where they fit (strips of up to 88 columns at 32 channels), else two
-int wgrad_cl_stages(int GX, int GY, int Wv) { return wgrad_cl_smem(GX, GY, Wv, 3) <= 220 * 1024 ? 3 : 2; }
+constexpr size_t WGRAD_CL_SMEM3 = 220 * 1024;
+int wgrad_cl_stages(int GX, int GY, int Wv) { return wgrad_cl_smem(GX, GY, Wv, 3) <= WGRAD_CL_SMEM3 ? 3 : 2; }
+// the most that any shape takes of a kernel with ns tiles
+size_t wgrad_cl_smem_limit(int GX, int GY, int ns) { return ns == 3 ? WGRAD_CL_SMEM3 : wgrad_cl_smem(GX, GY, TC_WT + 2, 2); }
 
 // ------------------------------------------------------------------ layout
 
@@ -500,7 +503,10 @@ int launch_conv_cl(const bf16* A, int M, const bf16* x, int B, int C, int H, int
     const size_t smem = conv_cl_smem(G, geo.Wv);
     auto* fn = mask ? (G == 2 ? conv_cl_kernel<2, true> : conv_cl_kernel<4, true>)
                     : (G == 2 ? conv_cl_kernel<2, false> : conv_cl_kernel<4, false>);
-    if (cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess) return TLBM_ERR_CUDA;
+    // (the limit belongs to the kernel, not to the launch: that of the widest strip,
+    // whatever the shape, so that threads with other shapes never lower it)
+    if (cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)conv_cl_smem(G, TC_WT + 2)) != cudaSuccess)
+        return TLBM_ERR_CUDA;
     fn<<<(unsigned)grid, CL_THREADS, smem, s>>>(A, M, x, H, W, bias, relu, y, act, mask, sums, geo);
     return status_of(cudaGetLastError());
 }
@@ -589,7 +595,7 @@ extern "C" int tlbm_conv3x3_backward_weight_cl(const void* x, const void* dy, fl
     const Fn fn = fns[GX == 4][GY == 4][ns == 3];
     long long S = 0;
     if (wgrad_cl_grid(B, cin, cout, H, W, &S) != TLBM_OK ||
-        cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess)
+        cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)wgrad_cl_smem_limit(GX, GY, ns)) != cudaSuccess)
         return TLBM_ERR_CUDA;
     cudaStream_t s = (cudaStream_t)stream;
     fn<<<(unsigned)S, WG_THREADS, smem, s>>>((const bf16*)dy, cout, (const bf16*)x, cin, H, W, geo, (float*)workspace);

@@ -156,3 +156,48 @@ def test_channels_last_calls_refuse_what_they_cannot_run(T):  # noqa: F811
                  lambda: T.tlbm_conv3x3_backward_weight_cl(x, x, y, 1, 1, 1, 2, 2, torch.zeros(16, device="cuda"), s)):
         with pytest.raises(T.TlbmError):
             call()
+
+
+def test_layers_of_other_widths_run_beside_each_other(T, tmp_path):  # noqa: F811
+    """Host threads call the channels-last layers with widths that need unlike
+    amounts of shared memory: every call is accepted, and the results are those
+    of a thread alone."""
+    import ctypes as C
+    import os
+    import subprocess
+
+    import torch
+
+    here = os.path.dirname(os.path.abspath(__file__))
+    so = str(tmp_path / "conv_threads.so")
+    subprocess.run(["gcc", "-O2", "-std=c11", "-shared", "-fPIC", "-pthread", os.path.join(here, "c", "conv_threads.c"),
+                    "-o", so], check=True)
+    helper = C.CDLL(so)
+    ch, H, widths = 32, 5, (65, 126, 20)
+    a = torch.zeros(T.tlbm_conv3x3_weight_elems(ch), dtype=torch.bfloat16, device="cuda")
+    w = torch.tensor(inputs.uniform_array(11, (ch, ch, 3, 3), -0.3, 0.3), dtype=torch.float32).cuda()
+    T.tlbm_conv3x3_pack_weights(w, ch, ch, a, torch.cuda.current_stream())
+    lib = T.lib()
+    fns = [C.cast(getattr(lib, f), C.c_void_p) for f in
+           ("tlbm_conv3x3_forward_cl", "tlbm_conv3x3_backward_data_cl", "tlbm_conv3x3_backward_weight_cl")]
+    per, results = [], {}
+    for W in widths:
+        x = _bf16(inputs.uniform_array(W, (1, H, W, ch), -1, 1)).cuda()
+        per.append([x, torch.empty_like(x), torch.empty_like(x), torch.empty_like(w), torch.empty(ch, device="cuda"),
+                    torch.empty(T.tlbm_conv3x3_cl_workspace_bytes(1, ch, ch, H, W), dtype=torch.uint8, device="cuda"),
+                    torch.cuda.Stream()])
+    torch.cuda.synchronize()
+    for calls in (1, 20000):
+        for group in ([[k] for k in range(len(widths))] if calls == 1 else [range(len(widths))]):
+            n = len(group)
+            ptrs = (C.c_void_p * (7 * n))(*[(t.cuda_stream if i == 6 else t.data_ptr())
+                                            for k in group for i, t in enumerate(per[k])])
+            ws = (C.c_size_t * n)(*[per[k][5].numel() for k in group])
+            wid = (C.c_int * n)(*[widths[k] for k in group])
+            refused = helper.conv_threads(*fns, C.c_void_p(a.data_ptr()), C.c_void_p(w.data_ptr()), ch, H, n, wid, ptrs,
+                                          ws, calls)
+            torch.cuda.synchronize()
+            assert refused == 0, (calls, refused)
+        results[calls] = [[t.clone() for t in q[1:5]] for q in per]
+    for W, p, q in zip(widths, results[1], results[20000]):
+        assert all(torch.equal(u, v) for u, v in zip(p, q)), W
