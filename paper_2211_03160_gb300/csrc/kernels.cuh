@@ -712,10 +712,12 @@ __device__ __forceinline__ void collide_trt_v(V (&d)[Lat<DIM>::F::Q], V (&g)[Lat
     const V drho = SCALED ? vmul(drs, inv) : drs;
     const V T = SCALED ? vmul(Ts, inv) : Ts;
     const V rho = vadd(vbc<V>(1.0f), drho);
-    const V buoy = vmul(vbc<V>(P::gbeta(p)), T);
+    // buoyancy and body force in one operation: as a product and a sum the pair
+    // instructions were contracted and the scalar ones were not
+    const V bz = vfma(vbc<V>(P::gbeta(p)), T, vbc<V>(P::body(p, DIM - 1)));
     const V Fx = vmul(rho, vbc<V>(P::body(p, 0)));
-    const V Fy = vmul(rho, DIM == 2 ? vadd(buoy, vbc<V>(P::body(p, 1))) : vbc<V>(P::body(p, 1)));
-    const V Fz = DIM == 3 ? vmul(rho, vadd(buoy, vbc<V>(P::body(p, 2)))) : zero;
+    const V Fy = vmul(rho, DIM == 2 ? bz : vbc<V>(P::body(p, 1)));
+    const V Fz = DIM == 3 ? vmul(rho, bz) : zero;
     const V ir = vrcp(rho);
     const V half = vbc<V>(0.5f);
     const V ux = vmul(vfma(jx, inv, vmul(half, Fx)), ir);
