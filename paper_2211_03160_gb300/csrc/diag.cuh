@@ -34,8 +34,10 @@ inline DiagOff diag_offsets(const KParams& p) {
     return o;
 }
 
-// The stored values of one node, unscaled: flow as the storage keeps it
-// (deviations in offset storage, f_i in FP64).
+// The stored values of one node: flow as the storage keeps it (deviations in offset
+// storage, f_i in FP64), in FP32 unscaled.  FP64 leaves the storage scale to the
+// sums (a power of two: the same bits), one multiplication each instead of one
+// per value.
 template <int DIM, class S, class C>
 __device__ __forceinline__ void diag_load(const S* __restrict__ own, const KParams& p, const int* off,
                                           C (&f)[Lat<DIM>::F::Q], C (&g)[Lat<DIM>::G::Q]) {
@@ -44,7 +46,7 @@ __device__ __forceinline__ void diag_load(const S* __restrict__ own, const KPara
     for (int i = 0; i < QF; ++i) f[i] = to_c<C>(ld_one<S, false>(TLBM_DBG(p, (own + off[i]), 0, 1)));
 #pragma unroll
     for (int i = 0; i < QG; ++i) g[i] = to_c<C>(ld_one<S, false>(TLBM_DBG(p, (own + off[QF + i]), 0, 1)));
-    if constexpr (Storage<S>::scaled) {
+    if constexpr (Storage<S>::scaled && std::is_same<C, float>::value) {
         const C inv = ScaleOf<C>::inv(p);
 #pragma unroll
         for (int i = 0; i < QF; ++i) f[i] *= inv;
@@ -82,6 +84,13 @@ __device__ __forceinline__ void diag_macros_d(const S* __restrict__ own, const K
     T = g[0];
 #pragma unroll
     for (int i = 1; i < LG::Q; ++i) T = dadd(T, g[i]);
+    if constexpr (Storage<S>::scaled) {
+        const double inv = ScaleOf<double>::inv(p);
+        drho = dmul(drho, inv);
+        T = dmul(T, inv);
+#pragma unroll
+        for (int ax = 0; ax < DIM; ++ax) j[ax] = dmul(j[ax], inv);
+    }
     rho = dadd(1.0, drho);
     // the fast reciprocal within FP32's range, IEEE division outside it
     const double ir = rho > 1e-30 && rho < 1e30 ? drcp(rho) : 1.0 / rho;

@@ -342,3 +342,39 @@ def test_default_kernels_stay_inside_their_buffers(T):  # noqa: F811
     for k in res[0]:
         assert res[1][k][2] == 0, k
         assert res[0][k][:2] == res[1][k][:2], k
+
+
+def _field_time(T, shape, prec, dtype, reduce=False):  # noqa: F811
+    """Seconds of one call for the fields (or the Nusselt number) of a 3D state, the least of 8."""
+    import time
+
+    import torch
+
+    s = T.Sim(*shape, lattice=D3, Ra=1e6, Pr=0.71, Ma=0.1, precision=prec)
+    s.init(1, 1e-2)
+    out = [torch.empty(s.N, dtype=dtype, device="cuda") for _ in range(5)]
+    code = T.TLBM_OUT_F32 if dtype == torch.float32 else T.TLBM_OUT_F64
+    best = 1e9
+    for _ in range(8):
+        torch.cuda.synchronize()
+        t0 = time.perf_counter()
+        for _ in range(10):
+            if reduce:
+                s.nusselt(allow_diverged=True)
+            else:
+                T.tlbm_macros(s.h, *out, code)
+        torch.cuda.synchronize()
+        best = min(best, (time.perf_counter() - t0) / 10)
+    s.close()
+    return best
+
+
+@pytest.mark.parametrize("prec", [2, 3])
+def test_fp64_fields_of_16bit_states_cost_as_those_of_fp32_ones(T, prec):  # noqa: F811
+    """FP64 fields are bound by the FP64 pipe: unscaling every 16-bit value there
+    would take 1.3 times the FP32 state's fields."""
+    import torch
+
+    shape = (161, 161, 161)
+    t16, t32 = (_field_time(T, shape, q, torch.float64) for q in (prec, 1))
+    assert t16 < 1.15 * t32, (t16, t32)
