@@ -837,7 +837,7 @@ extern "C" int tlbm_macros(tlbm_t h, void* rho, void* ux, void* uy, void* uz, vo
 
 // the reduction's view of a handle's current state (parameters by value)
 static RedState red_state(tlbm_t h) {
-    return {h->buf[h->cur], nullptr, (double*)(h->mem + h->red_off), (const int*)(h->mem + h->status_off), 0, 0};
+    return {h->buf[h->cur], nullptr, (double*)(h->mem + h->red_off), (const int*)(h->mem + h->status_off), 0, 0, false};
 }
 
 // runs the two-pass reduction and copies the six results to the host

@@ -1,9 +1,10 @@
 // Diagnostics of a state: macroscopic fields and the FP64 reductions (a6)
 // behind tlbm_nusselt, tlbm_energy and tlbm_status, one state or many at once.
 //
-// Both kernels walk segments of 32 nodes of one row: a warp takes a segment,
-// lane by lane, so that every population is one coalesced 32-element load at an
-// offset known per launch (no division or address table per node and value).
+// Both kernels walk segments of 32 nodes: a warp takes a segment, lane by lane,
+// so that every population is one coalesced 32-element load at an offset known
+// per launch (no division or address table per node and value).  A segment is a
+// stretch of one row, or of the cell's nodes in memory order (walks_flat).
 #include <algorithm>
 
 #include "diag.cuh"
@@ -25,6 +26,35 @@ __device__ __forceinline__ void segment(unsigned k, unsigned segs, const Layout&
     y = (int)(r - zz * (unsigned)L.ny);
 }
 
+// this lane's node of segment k in memory order, across row ends, so that only the
+// cell's last segment is not full; false if it has none
+__device__ __forceinline__ bool flat_segment(unsigned k, const Layout& L, int& x, int& y, int& z) {
+    const unsigned n = 32u * k + (threadIdx.x & 31u), r = n / (unsigned)L.nx;
+    const unsigned zz = L.nz > 1 ? r / (unsigned)L.ny : 0u;
+    x = (int)(n - r * (unsigned)L.nx);
+    y = (int)(r - zz * (unsigned)L.ny);
+    z = (int)zz;
+    return r < (unsigned)L.ny * (unsigned)L.nz;
+}
+
+// segments of a state
+__host__ __device__ inline unsigned segments(const Layout& L, bool flat) {
+    const unsigned rows = (unsigned)L.ny * (unsigned)L.nz;
+    return flat ? ((unsigned)L.nx * rows + 31u) / 32u : (unsigned)(L.nx + 31) / 32u * rows;
+}
+
+// Whether a state is walked in memory order.  FP64 arithmetic: always, the FP64
+// pipe spends as much on an idle lane as on a busy one.  FP32 arithmetic, bound by
+// HBM and the latency of its loads: where over a quarter of the lanes would idle,
+// else a division less per node is worth more.  us, rows -> memory order: FP64
+// fields of an FP16 state 161^3 882 -> 744, 385^3 10797 -> 9994, 3 x 300^2 517 ->
+// 55, 256^3 2945 both ways; FP32 fields of an FP32 state, 2D, 33 nodes a row 31 ->
+// 27, 65 32.2 -> 29.9, 129 49.8 and 51.1, 8193^2 869 and 1009.
+bool walks_flat(const Layout& L, bool fp64) {
+    const int lanes = (L.nx + 31) / 32 * 32;
+    return fp64 || 4 * (lanes - L.nx) > lanes;
+}
+
 template <int DIM, class S>
 __device__ __noinline__ void macros_node_d(const S* own, const KParams& p, const int* off, double* m) {
     double u[3];
@@ -35,9 +65,13 @@ __device__ __noinline__ void macros_node_d(const S* own, const KParams& p, const
 }
 
 // Bound by HBM for FP32 fields (the state read once, the fields written once)
-// and by the FP64 pipe for FP64 ones.
+// and by the FP64 pipe for FP64 ones.  40 registers for FP32 fields of 2D 16-bit
+// states, which let more of a node's loads go out together than the 32 the
+// compiler takes by itself: 8193^2 FP16 799 -> 758 us.
 template <int DIM, class S, class O>
-__global__ void __launch_bounds__(THREADS)
+constexpr int MACRO_BLOCKS = DIM == 2 && sizeof(S) == 2 && sizeof(O) == 4 ? 6 : 0;  // per SM, 0: as it comes
+template <int DIM, class S, class O, bool FLAT>
+__global__ void __launch_bounds__(THREADS, (MACRO_BLOCKS<DIM, S, O>))
     macros_kernel(const S* __restrict__ buf, const KParams p, const DiagOff k, unsigned segs, unsigned n,
                   O* __restrict__ rho, O* __restrict__ ux, O* __restrict__ uy, O* __restrict__ uz,
                   O* __restrict__ T) {
@@ -45,9 +79,13 @@ __global__ void __launch_bounds__(THREADS)
     const unsigned nw = gridDim.x * WARPS;
     for (unsigned i = blockIdx.x * WARPS + (threadIdx.x >> 5); i < n; i += nw) {
         int x, y, z;
-        segment(i, segs, L, x, y, z);
-        x += threadIdx.x & 31;
-        if (x >= L.nx) continue;
+        if constexpr (FLAT) {
+            if (!flat_segment(i, L, x, y, z)) continue;
+        } else {
+            segment(i, segs, L, x, y, z);
+            x += threadIdx.x & 31;
+            if (x >= L.nx) continue;
+        }
         const S* own = buf + L.slot(x, y, z);
         O m[5];
         if constexpr (std::is_same<O, float>::value && !std::is_same<S, double>::value) {
@@ -161,17 +199,29 @@ __global__ void __launch_bounds__(THREADS)
     const int* off = ONE ? k1.off : soff;
     const Layout L = p.L;
     const S* buf = static_cast<const S*>(q.buf);
-    const unsigned segs = (unsigned)(L.nx + 31) / 32u, n = segs * (unsigned)L.ny * (unsigned)L.nz;
+    const unsigned segs = (unsigned)(L.nx + 31) / 32u, n = segments(L, q.flat);
     const unsigned W = (unsigned)q.blocks * WARPS;
+    const unsigned k0 = ((unsigned)blockIdx.x - (unsigned)q.block0) * WARPS + (threadIdx.x >> 5);
     Sums<C> sum;
-    for (unsigned k = ((unsigned)blockIdx.x - (unsigned)q.block0) * WARPS + (threadIdx.x >> 5); k < n; k += W) {
-        int x, y, z;
-        segment(k, segs, L, x, y, z);
-        x += threadIdx.x & 31;
-        if (x < L.nx) {
-            C t[5];
-            node_terms<DIM, S>(buf + L.slot(x, y, z), p, off, t);
-            sum.add(t);
+    if (q.flat) {
+        for (unsigned k = k0; k < n; k += W) {
+            int x, y, z;
+            if (flat_segment(k, L, x, y, z)) {
+                C t[5];
+                node_terms<DIM, S>(buf + L.slot(x, y, z), p, off, t);
+                sum.add(t);
+            }
+        }
+    } else if constexpr (!std::is_same<C, double>::value) {
+        for (unsigned k = k0; k < n; k += W) {
+            int x, y, z;
+            segment(k, segs, L, x, y, z);
+            x += threadIdx.x & 31;
+            if (x < L.nx) {
+                C t[5];
+                node_terms<DIM, S>(buf + L.slot(x, y, z), p, off, t);
+                sum.add(t);
+            }
         }
     }
     sum.close();
@@ -218,24 +268,25 @@ __global__ void __launch_bounds__(32 * RED_FIELDS)
 
 // blocks of one state's reduction: a few segments per warp, at most four blocks
 // on each of 152 SMs (a constant, so that the sums do not depend on the device)
-int red_blocks(const KParams& p) {
-    const long long n = (long long)((p.L.nx + 31) / 32) * p.L.ny * p.L.nz;
+int red_blocks(const KParams& p, bool flat) {
+    const long long n = segments(p.L, flat);
     return (int)std::max<long long>(1, std::min<long long>(RED_BLOCKS, (n + 4 * WARPS - 1) / (4 * WARPS)));
 }
 
+template <int DIM, class S, class O, bool FLAT>
+cudaError_t macros_as(const void* buf, const KParams& p, void* rho, void* ux, void* uy, void* uz, void* T, cudaStream_t s) {
+    const unsigned n = segments(p.L, FLAT), grid = std::min(16384u, (n + WARPS - 1) / WARPS);
+    macros_kernel<DIM, S, O, FLAT><<<grid, THREADS, 0, s>>>((const S*)buf, p, diag_offsets<DIM>(p), (unsigned)(p.L.nx + 31) / 32u,
+                                                            n, (O*)rho, (O*)ux, (O*)uy, (O*)uz, (O*)T);
+    return cudaGetLastError();
+}
 template <int DIM, class S>
 cudaError_t macros_t(const void* buf, const KParams& p, void* rho, void* ux, void* uy, void* uz, void* T, bool f64,
                      cudaStream_t s) {
-    const DiagOff k = diag_offsets<DIM>(p);
-    const unsigned segs = (unsigned)(p.L.nx + 31) / 32u, n = segs * (unsigned)p.L.ny * (unsigned)p.L.nz;
-    const unsigned grid = std::min(16384u, (n + WARPS - 1) / WARPS);
-    if (f64)
-        macros_kernel<DIM, S, double><<<grid, THREADS, 0, s>>>((const S*)buf, p, k, segs, n, (double*)rho, (double*)ux,
-                                                               (double*)uy, (double*)uz, (double*)T);
-    else
-        macros_kernel<DIM, S, float><<<grid, THREADS, 0, s>>>((const S*)buf, p, k, segs, n, (float*)rho, (float*)ux,
-                                                              (float*)uy, (float*)uz, (float*)T);
-    return cudaGetLastError();
+    if (f64) return macros_as<DIM, S, double, true>(buf, p, rho, ux, uy, uz, T, s);
+    if constexpr (!std::is_same<S, double>::value)
+        if (!walks_flat(p.L, false)) return macros_as<DIM, S, float, false>(buf, p, rho, ux, uy, uz, T, s);
+    return macros_as<DIM, S, float, true>(buf, p, rho, ux, uy, uz, T, s);
 }
 
 template <int DIM, class S>
@@ -266,7 +317,8 @@ cudaError_t launch_reduce(int dim, int prec, RedStates& st, int count, const KPa
     int grid = 0;
     for (int i = 0; i < count; ++i) {
         st.s[i].block0 = grid;
-        st.s[i].blocks = red_blocks(*host_kp[i]);
+        st.s[i].flat = walks_flat(host_kp[i]->L, prec == 0);
+        st.s[i].blocks = red_blocks(*host_kp[i], st.s[i].flat);
         grid += st.s[i].blocks;
     }
     const KParams* p1 = count == 1 && !st.s[0].kp ? host_kp[0] : nullptr;

@@ -26,6 +26,7 @@ struct RedState {
     double* partials;
     const int* status;
     int block0, blocks;  // its blocks of the flattened grid (set by launch_reduce)
+    bool flat;           // walked in memory order (set by launch_reduce)
 };
 struct RedStates {
     RedState s[RED_MANY];

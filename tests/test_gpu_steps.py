@@ -369,6 +369,21 @@ def _field_time(T, shape, prec, dtype, reduce=False):  # noqa: F811
     return best
 
 
+@pytest.mark.parametrize("prec", [0, 1, 2, 3])
+def test_fields_of_narrow_rows_cost_as_those_of_wide_ones(T, prec):  # noqa: F811
+    """What the FP64 pipe bounds (FP64 fields, and fields and reductions of FP64
+    states) takes for a cell with three nodes a row at most three times as long
+    as for as many nodes in rows of 100: no warp is spent on a row (which costs
+    about ten times)."""
+    import torch
+
+    narrow, wide = (3, 600, 600), (100, 108, 100)
+    kinds = [(torch.float64, False)] + ([(torch.float32, False), (torch.float64, True)] if prec == 0 else [])
+    for dtype, reduce in kinds:
+        t = [_field_time(T, sh, prec, dtype, reduce) for sh in (narrow, wide)]
+        assert t[0] < 3 * t[1], (dtype, reduce, t)
+
+
 @pytest.mark.parametrize("prec", [2, 3])
 def test_fp64_fields_of_16bit_states_cost_as_those_of_fp32_ones(T, prec):  # noqa: F811
     """FP64 fields are bound by the FP64 pipe: unscaling every 16-bit value there
