@@ -954,16 +954,15 @@ __device__ __forceinline__ double anti_bounce_back(double val, double omega, dou
 __device__ __forceinline__ float anti_bounce_back(float val, float omega, float Tw) { return __fmaf_rn(omega, Tw, -val); }
 
 // Write the post-collision value `val` of population i (set LS, flow or
-// thermal) of node (x, y, z) where the next step will read it, if it leaves
-// the cell.  THERMAL selects the temperature rules of §2.2.  PULL: into the
-// ghost slot the node (wall) or its periodic image pulls from.  AA_EVEN: into
-// the ghost slot the following AA_ODD half reads it from.  AA_ODD: into the slot
-// the next AA_EVEN half reads (the node's own slot of the opposite direction
-// for a wall, the image's own slot for a periodic face).
+// thermal) of node (x, y, z), which leaves the cell through a wall, where the
+// next step will read it: half-way bounce-back, as population ibar of the same
+// node.  THERMAL selects the temperature rules of §2.2.  PULL: into the ghost slot
+// the node pulls from.  AA_EVEN: into the ghost slot the following AA_ODD half
+// reads it from.  AA_ODD: into the slot the next AA_EVEN half reads (the node's
+// own slot of the opposite direction).
 // RAW: flow values are f_i as stored (FP64 with the two-relaxation-time
-// collision) rather than deviations.  WALLED: the caller knows that the value, if
-// it leaves the cell, meets a wall.
-template <class LS, bool THERMAL, int i, class S, class C, int MODE, bool RAW, bool WALLED = false>
+// collision) rather than deviations.
+template <class LS, bool THERMAL, int i, class S, class C, int MODE, bool RAW>
 __device__ __forceinline__ void ghost_write(S* __restrict__ base, const KParams& p, int x, int y, int z, C val,
                                             C scale, uint32_t salt) {
     constexpr int ex = LS::e(i, 0), ey = LS::e(i, 1), ez = LS::e(i, 2);
@@ -974,41 +973,47 @@ __device__ __forceinline__ void ghost_write(S* __restrict__ base, const KParams&
     const bool oy = dy < 0 || dy >= L.ny;
     const bool oz = (ez != 0) && (dz < 0 || dz >= L.nz);
     if (!(ox || oy || oz)) return;
-    const bool wall = WALLED || (ox && !(p.periodic & 1)) || (oy && !(p.periodic & 2)) || (oz && !(p.periodic & 4));
-    constexpr int o = LS::opp(i);
-    if (wall) {
-        // bounce-back: the value returns to the node as f_ibar of the next step
-        C out = val;
-        if constexpr (THERMAL) {
-            // axis-aligned: exactly one axis is crossed
-            const int ax = ox ? 0 : (oy ? 1 : 2);
-            if (ax == p.heat_axis) {
-                const bool hi = ox ? (dx >= L.nx) : (oy ? (dy >= L.ny) : (dz >= L.nz));
-                const C Tw = hi ? PV<C>::Tc(p) : PV<C>::Th(p);
-                out = anti_bounce_back(val, PV<C>::omega(p), Tw);
-            }
+    C out = val;
+    if constexpr (THERMAL) {
+        // axis-aligned: exactly one axis is crossed
+        const int ax = ox ? 0 : (oy ? 1 : 2);
+        if (ax == p.heat_axis) {
+            const bool hi = ox ? (dx >= L.nx) : (oy ? (dy >= L.ny) : (dz >= L.nz));
+            const C Tw = hi ? PV<C>::Tc(p) : PV<C>::Th(p);
+            out = anti_bounce_back(val, PV<C>::omega(p), Tw);
         }
-        // written by PULL: slot (x + e_i) of plane ibar, where the node pulls
-        // ibar from; by AA_EVEN: slot (x + e_i) of plane i, where the next
-        // AA_ODD half reads it; by AA_ODD: the node's own slot of plane ibar,
-        // where the next AA_EVEN half reads it
-        constexpr int plane = MODE == AA_EVEN ? i : o;
-        const long long s = MODE == AA_ODD ? L.slot(x, y, z) : L.slot(dx, dy, dz);
-        if constexpr (THERMAL) *TLBM_DBG(p, (base + ((long long)plane * L.plane + s)), 0, 1) = enc_g_step<S, C>(out, scale, salt);
-        else *TLBM_DBG(p, (base + ((long long)plane * L.plane + s)), 0, 1) = enc_f_step<LS, S, C, RAW>(out, plane, scale, salt);
-    } else {
-        // periodic: the value reaches the image node w = wrap(x + e_i) as f_i;
-        // written by PULL: slot (w - e_i) of plane i; by AA_EVEN: slot (w - e_i)
-        // of plane ibar (the next AA_ODD half reads there); by AA_ODD: w's own
-        // slot of plane i (the next AA_EVEN half reads there)
-        const int wx = ox ? (dx < 0 ? dx + L.nx : dx - L.nx) : dx;
-        const int wy = oy ? (dy < 0 ? dy + L.ny : dy - L.ny) : dy;
-        const int wz = oz ? (dz < 0 ? dz + L.nz : dz - L.nz) : dz;
-        constexpr int plane = MODE == AA_EVEN ? o : i;
-        const long long s = MODE == AA_ODD ? L.slot(wx, wy, wz) : L.slot(wx - ex, wy - ey, wz - ez);
-        if constexpr (THERMAL) *TLBM_DBG(p, (base + ((long long)plane * L.plane + s)), 0, 1) = enc_g_step<S, C>(val, scale, salt);
-        else *TLBM_DBG(p, (base + ((long long)plane * L.plane + s)), 0, 1) = enc_f_step<LS, S, C, RAW>(val, plane, scale, salt);
     }
+    constexpr int plane = MODE == AA_EVEN ? i : LS::opp(i);
+    const long long s = MODE == AA_ODD ? L.slot(x, y, z) : L.slot(dx, dy, dz);
+    if constexpr (THERMAL) *TLBM_DBG(p, (base + ((long long)plane * L.plane + s)), 0, 1) = enc_g_step<S, C>(out, scale, salt);
+    else *TLBM_DBG(p, (base + ((long long)plane * L.plane + s)), 0, 1) = enc_f_step<LS, S, C, RAW>(out, plane, scale, salt);
+}
+
+// The same for a population that leaves through the periodic face (AXIS, SIDE) its
+// node lies on.  It reaches the image node w = wrap(x + e_i) as f_i, unless it
+// also crosses a wall along its second axis, B (flow only), where it bounces
+// back.  Written by PULL into slot w - e_i of plane i; by AA_EVEN into slot
+// w - e_i of plane ibar (the next AA_ODD half reads there); by AA_ODD into w's
+// own slot of plane i (the next AA_EVEN half reads there); a bounced one as by
+// ghost_write.  Offsets are relative to the node's own slot in plane 0 (`own`):
+// a crossing shifts a slot by the cell's extent along that axis.
+template <class LS, bool THERMAL, int i, class S, class C, int MODE, bool RAW, int AXIS, int SIDE>
+__device__ __forceinline__ void image_write(S* __restrict__ own, const KParams& p, const int (&at)[3], C val, C scale,
+                                            uint32_t salt) {
+    constexpr int B = LS::e(i, (AXIS + 1) % 3) != 0 ? (AXIS + 1) % 3 : (AXIS + 2) % 3, eb = LS::e(i, B);
+    static_assert(LS::e(i, AXIS) == SIDE && (!THERMAL || eb == 0), "a population of this face");
+    const Layout& L = p.L;
+    const int n[3] = {L.nx, L.ny, L.nz}, stride[3] = {1, L.P, p.rp};
+    const bool two = eb != 0 && at[B] == (eb > 0 ? n[B] - 1 : 0);  // crosses B as well
+    const bool back = two && !(p.periodic & (1 << B));
+    const int step = SIDE * stride[AXIS] + eb * stride[B];
+    const int wrap = SIDE * n[AXIS] * stride[AXIS] + (two ? eb * n[B] * stride[B] : 0);
+    const int off = back ? (MODE == AA_ODD ? 0 : step) : (MODE == AA_ODD ? step - wrap : -wrap);
+    constexpr int o = LS::opp(i);
+    const int plane = back == (MODE == AA_EVEN) ? i : o;
+    S* to = own + ((long long)plane * L.plane + off);
+    if constexpr (THERMAL) *TLBM_DBG(p, to, 0, 1) = enc_g_step<S, C>(val, scale, salt);
+    else *TLBM_DBG(p, to, 0, 1) = enc_f_step<LS, S, C, RAW>(val, i, scale, salt);  // w_i = w_ibar
 }
 
 // ------------------------------------------------------------------ step kernel
@@ -1092,15 +1097,22 @@ __device__ __forceinline__ void face_writes(S* __restrict__ dst, const KParams& 
     using LG = typename Lat<DIM>::G;
     const C scale = ScaleOf<C>::s(p);
     S* __restrict__ gdst = dst + (long long)LF::Q * p.L.plane;
+    const int at[3] = {x, y, z};
+    const long long own = WALLED ? 0 : p.L.slot(x, y, z);
     static_for<LF::Q>([&](auto ii) {
         constexpr int i = decltype(ii)::value;
-        if constexpr (LF::e(i, AXIS) == SIDE)
-            ghost_write<LF, false, i, S, C, MODE, RAW, WALLED>(dst, p, x, y, z, val(ii), scale, salt);
+        if constexpr (LF::e(i, AXIS) == SIDE) {
+            if constexpr (WALLED) ghost_write<LF, false, i, S, C, MODE, RAW>(dst, p, x, y, z, val(ii), scale, salt);
+            else image_write<LF, false, i, S, C, MODE, RAW, AXIS, SIDE>(dst + own, p, at, val(ii), scale, salt);
+        }
     });
     static_for<LG::Q>([&](auto ii) {
         constexpr int i = decltype(ii)::value;
-        if constexpr (LG::e(i, AXIS) == SIDE)
-            ghost_write<LG, true, i, S, C, MODE, RAW, WALLED>(gdst, p, x, y, z, val(std::integral_constant<int, LF::Q + i>{}), scale, salt);
+        if constexpr (LG::e(i, AXIS) == SIDE) {
+            constexpr std::integral_constant<int, LF::Q + i> j{};
+            if constexpr (WALLED) ghost_write<LG, true, i, S, C, MODE, RAW>(gdst, p, x, y, z, val(j), scale, salt);
+            else image_write<LG, true, i, S, C, MODE, RAW, AXIS, SIDE>(gdst + own, p, at, val(j), scale, salt);
+        }
     });
 }
 template <int DIM, class S, class C, int MODE, bool RAW, int AXIS, int SIDE, bool CLOSED, class Val>
@@ -1210,7 +1222,7 @@ __device__ __forceinline__ void x_face(S* __restrict__ base, const KParams& p, i
         constexpr int i = decltype(ii)::value;
         if constexpr (LS::e(i, 0) == SIDE) {
             const C val = pick<VEC>(v[i], k);
-            ghost_write<LS, THERMAL, i, S, C, MODE, KS && !Storage<S>::offset, true>(base, p, x, y, z, KS && Storage<S>::offset ? val * un : val, scale, salt);
+            ghost_write<LS, THERMAL, i, S, C, MODE, KS && !Storage<S>::offset>(base, p, x, y, z, KS && Storage<S>::offset ? val * un : val, scale, salt);
         }
     });
 }
