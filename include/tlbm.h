@@ -355,10 +355,13 @@ TLBM_API int tlbm_batch_get_staged(tlbm_batch_t b, int* consumer_warps, int* sta
 /* Time the compiled launch shapes (nodes per thread x rows per thread x block
  * shape, then tiles per block, then the staged form where it applies: 4 or the
  * most consumer warps x 2 to 4 stages; trials launches each) on the bound
- * state and keep the fastest.  The state is not changed. */
+ * state and keep the fastest; then, where calls of 16 steps or more take several
+ * steps per launch, those launches against it.  The state is not changed. */
 TLBM_API int tlbm_batch_autotune(tlbm_batch_t b, int trials);
 /* (trials < 0: reuse the shape this process tuned for the same lattice, storage,
- * collision form and size class floor(log2(total nodes)), if any.) */
+ * collision form and size class floor(log2(total nodes)), if any, and what it
+ * measured of several steps per launch for a batch of as many and as wide cells;
+ * else that is timed.) */
 /* Borrow instance idx as a single-cell handle (owned by the batch). */
 TLBM_API int tlbm_batch_instance(tlbm_batch_t b, int idx, tlbm_t* out);
 /* Per-instance Nusselt numbers / divergence flags into nu[n] / diverged[n].

@@ -859,7 +859,7 @@ extern "C" int tlbm_batch_get_variant(tlbm_batch_t b, int* vec, int* form, int* 
 // Tuned launch shapes of this process, per (lattice, storage, collision form,
 // size class = floor(log2(total nodes))).
 static std::mutex g_tune_mu;
-static std::map<std::tuple<int, int, int, int>, std::array<int, 8>> g_tune_cache;
+static std::map<std::tuple<int, int, int, int>, std::array<int, 7>> g_tune_cache;
 
 static std::tuple<int, int, int, int> tune_key(tlbm_batch_t b) {
     long long nodes = 0;
@@ -869,30 +869,97 @@ static std::tuple<int, int, int, int> tune_key(tlbm_batch_t b) {
     return std::make_tuple(b->lattice, b->prec, b->trt, cls);
 }
 
+// Whether marching was found slower than the tuned one-step form, per (that key,
+// floor(log2(cells)), eighths of the strips' columns that hold nodes): what a
+// marching launch does with a cell follows from its width.  No entry: not measured.
+static std::map<std::tuple<std::tuple<int, int, int, int>, int, int>, int> g_march_cache;
+
+static std::tuple<std::tuple<int, int, int, int>, int, int> march_key(tlbm_batch_t b) {
+    long long nodes = 0, columns = 0;
+    for (tlbm_t h : b->inst) {
+        nodes += (long long)h->nx * h->ny;
+        columns += (long long)((h->nx + MARCH_COLUMNS - 1) / MARCH_COLUMNS) * MARCH_COLUMNS * h->ny;
+    }
+    int cells = 0;
+    while ((2 << cells) <= b->n) ++cells;
+    return std::make_tuple(tune_key(b), cells, (int)(8 * nodes / columns));
+}
+
+// ms of `reps` runs of `launch` on the batch's stream after one to warm up; 1e30
+// if one is refused
+template <class F>
+static float time_launches(tlbm_batch_t b, int reps, F launch) {
+    cudaEvent_t e0 = nullptr, e1 = nullptr;
+    cudaError_t e = cudaEventCreate(&e0);
+    if (e == cudaSuccess) e = cudaEventCreate(&e1);
+    if (e == cudaSuccess) e = launch();
+    if (e == cudaSuccess) e = cudaEventRecord(e0, b->stream);
+    for (int r = 0; r < reps && e == cudaSuccess; ++r) e = launch();
+    if (e == cudaSuccess) e = cudaEventRecord(e1, b->stream);
+    if (e == cudaSuccess) e = cudaEventSynchronize(e1);
+    float ms = 1e30f;
+    if (e == cudaSuccess) e = cudaEventElapsedTime(&ms, e0, e1);
+    if (e != cudaSuccess) cudaGetLastError();
+    if (e0) cudaEventDestroy(e0);
+    if (e1) cudaEventDestroy(e1);
+    return e == cudaSuccess ? ms : 1e30f;
+}
+
+// Three steps per launch against the one-step form in use: march_off, from the
+// cache if `reuse` and this kind of batch was measured, else measured here.  A
+// batch that cannot march, or whose form the caller chose, leaves no entry.
+static int tune_march(tlbm_batch_t b, int reps, bool reuse) {
+    b->march_off = 0;
+    const int rc = upload_tables(b);
+    if (rc != TLBM_OK || !b->march) return rc;
+    const auto key = march_key(b);
+    if (reuse) {
+        std::lock_guard<std::mutex> lk(g_tune_mu);
+        auto it = g_march_cache.find(key);
+        if (it != g_march_cache.end()) {
+            b->march_off = it->second;
+            return b->march_off ? upload_tables(b) : TLBM_OK;
+        }
+    }
+    const float one = time_launches(b, reps, [&] { return launch_batch(b, b->parity, b->stream); });
+    const float three = time_launches(b, reps, [&] { return launch_marches(b, b->parity, b->stream); });
+    b->launches += (int64_t)(reps + 1) * (1 + (int64_t)b->marches.size());
+    b->march_off = three > MARCH_STEPS * one;
+    {
+        std::lock_guard<std::mutex> lk(g_tune_mu);
+        g_march_cache[key] = b->march_off;
+    }
+    return b->march_off ? upload_tables(b) : TLBM_OK;
+}
+
 // Time each candidate launch shape on the bound state without changing it
 // (every trial step reads the current buffers and writes the other ones, and
 // the current buffers stay current), keep the fastest.  trials < 0 reuses the
 // choice cached for the batch's (lattice, storage, form, size class) when there
-// is one.
+// is one, and what was measured of marching for batches like it.
 extern "C" int tlbm_batch_autotune(tlbm_batch_t b, int trials) {
     if (!b) return bfail(nullptr, TLBM_ERR_ARG, "NULL batch");
     if (!b->mem) return bfail(b, TLBM_ERR_UNBOUND, "device memory not bound");
+    const int reps = trials > 0 ? trials : 5;
     if (trials < 0) {
-        std::lock_guard<std::mutex> lk(g_tune_mu);
-        auto it = g_tune_cache.find(tune_key(b));
-        if (it != g_tune_cache.end()) {
-            b->vec = it->second[0];
-            b->bx = it->second[1];
-            b->by = it->second[2];
-            b->rows = it->second[3];
-            b->tpb = it->second[4];
-            b->march_off = it->second[7];
-            if (it->second[5] > 0 && staged_possible(b)) return batch_set_staged(b, it->second[5], it->second[6]);
+        bool found = false;
+        std::array<int, 7> t{};
+        {
+            std::lock_guard<std::mutex> lk(g_tune_mu);
+            auto it = g_tune_cache.find(tune_key(b));
+            if ((found = it != g_tune_cache.end())) t = it->second;
+        }
+        if (found) {
+            b->vec = t[0];
+            b->bx = t[1];
+            b->by = t[2];
+            b->rows = t[3];
+            b->tpb = t[4];
             b->staged_nc = 0;
-            return upload_tables(b);
+            const int rc = t[5] > 0 && staged_possible(b) ? batch_set_staged(b, t[5], t[6]) : TLBM_OK;
+            return rc != TLBM_OK ? rc : tune_march(b, reps, true);
         }
     }
-    const int reps = trials > 0 ? trials : 5;
     const int vecs[] = {8, 4, 2, 1};
     const int shapes[][2] = {{32, 1}, {32, 2}, {32, 4}, {64, 1}, {64, 2}, {128, 1}};
     const int keep_vec = b->vec, keep_bx = b->bx, keep_by = b->by, keep_rows = b->rows;
@@ -1001,28 +1068,15 @@ extern "C" int tlbm_batch_autotune(tlbm_batch_t b, int trials) {
         }
         b->staged_nc = 0;
     }
-    // three steps per launch against the best of these
-    b->march_off = 0;
-    if (rc == TLBM_OK && (rc = upload_tables(b)) == TLBM_OK && b->march) {
-        cudaError_t e = launch_marches(b, b->parity, b->stream);  // warm
-        cudaEventRecord(e0, b->stream);
-        for (int r = 0; r < reps && e == cudaSuccess; ++r) e = launch_marches(b, b->parity, b->stream);
-        cudaEventRecord(e1, b->stream);
-        if (e == cudaSuccess) e = cudaEventSynchronize(e1);
-        if (e != cudaSuccess) cudaGetLastError();
-        float ms = 1e30f;
-        if (e == cudaSuccess) cudaEventElapsedTime(&ms, e0, e1);
-        b->launches += (int64_t)(reps + 1) * (int64_t)b->marches.size();
-        b->march_off = ms > MARCH_STEPS * best;
-    }
     cudaEventDestroy(e0);
     cudaEventDestroy(e1);
     if (rc == TLBM_OK) {
         std::lock_guard<std::mutex> lk(g_tune_mu);
-        g_tune_cache[tune_key(b)] = {bv, bbx, bby, brows, btpb, bnc, bns, b->march_off};
+        g_tune_cache[tune_key(b)] = {bv, bbx, bby, brows, btpb, bnc, bns};
     }
-    int rc2 = bnc > 0 ? batch_set_staged(b, bnc, bns) : upload_tables(b);
-    return rc != TLBM_OK ? rc : rc2;
+    const int rc2 = bnc > 0 ? batch_set_staged(b, bnc, bns) : upload_tables(b);
+    if (rc == TLBM_OK) rc = rc2;
+    return rc != TLBM_OK ? rc : tune_march(b, reps, false);
 }
 
 extern "C" int tlbm_batch_instance(tlbm_batch_t b, int idx, tlbm_t* out) {

@@ -255,3 +255,32 @@ def test_staged_batch_wait_times_out_and_recovers(T):
         assert np.array_equal(fa, fb) and np.array_equal(ga, gb), k
     b.close()
     ref.close()
+
+
+def test_marching_is_measured_for_each_kind_of_batch(T):
+    """autotune(-1) takes over what was measured of marching for a batch of as
+    many cells as wide, and measures where nothing was: after a periodic batch and
+    one whose form the caller chose (neither marches), and for one wide cell of
+    as many nodes as several narrow ones."""
+    def launches(cells, choose=None, trials=-1, **kw):
+        b = T.Batch([c + (1, 1e6, 0.71, 0.1, i) for i, c in enumerate(cells)], precision=3, **kw)
+        b.init(1e-3)
+        if choose:
+            choose(b)
+        l0 = b.launches
+        b.autotune(trials)
+        n = b.launches - l0
+        b.close()
+        return n
+
+    narrow, wide = [(131, 127)] * 4, [(4200, 16)]  # both 2^16 to 2^17 nodes
+    assert launches(narrow, trials=2, periodic_mask=1) > 0
+    assert launches(narrow, periodic_mask=1) == 0
+    assert launches(narrow) > 0
+    assert launches(narrow) == 0
+    assert launches(wide) > 0
+    assert launches(wide) == 0
+    small = [(67, 61)] * 4
+    assert launches(small, choose=lambda b: b.set_rows(1), trials=2) > 0
+    assert launches(small) > 0
+    assert launches(small) == 0
