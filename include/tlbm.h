@@ -304,9 +304,9 @@ TLBM_API int tlbm_batch_bind_memory(tlbm_batch_t b, void* dev_ptr, size_t bytes)
 TLBM_API int tlbm_batch_set_stream(tlbm_batch_t b, void* cuda_stream);
 /* tlbm_init of every instance with its own tlbm_instance.seed. */
 TLBM_API int tlbm_batch_init(tlbm_batch_t b, double noise_amp);
-/* Advance every instance by n steps.  Asynchronous.  Unless tlbm_batch_set_variant,
- * _set_rows, _set_staged or _set_persistent was called, calls of 16 steps or more
- * may advance several steps per launch, as in tlbm_step. */
+/* Advance every instance by n steps.  Asynchronous.  Unless tlbm_batch_set_variant
+ * or _set_rows was called or the staged or persistent form is in force, calls of
+ * 16 steps or more may advance several steps per launch, as in tlbm_step. */
 TLBM_API int tlbm_batch_step(tlbm_batch_t b, int64_t n);
 /* Launch shape of the batched kernel (0 keeps the current value; form as in
  * tlbm_set_variant) and the steps per graph launch (even; 0 = no graph). */
@@ -315,8 +315,8 @@ TLBM_API int tlbm_batch_set_variant(tlbm_batch_t b, int vec, int form, int block
 /* Persistent form: steps_per_launch > 0 makes tlbm_batch_step run up to that
  * many steps per launch of one cooperative kernel whose blocks (as many as fit
  * on the device at once) work through the tiles of every instance in a fixed
- * order and meet at a grid barrier between steps; 0 returns to one flattened
- * launch per step (graph-captured).  The barrier's waits are bounded: a block
+ * order and meet at a grid barrier between steps; 0 returns to what
+ * tlbm_batch_step runs without it.  The barrier's waits are bounded: a block
  * that waits too long gives up, and tlbm_batch_status then returns
  * TLBM_ERR_TIMEOUT.  TLBM_ERR_UNSUPPORTED without cooperative launch. */
 TLBM_API int tlbm_batch_set_persistent(tlbm_batch_t b, int steps_per_launch);

@@ -316,6 +316,7 @@ size_t align_up(size_t v, size_t a) { return (v + a - 1) / a * a; }
 
 }  // namespace
 
+enum { FORM_SHAPE = 1, FORM_STAGED = 2, FORM_PERSISTENT = 4 };
 struct tlbm_batch_s {
     int n, dim, lattice, prec;
     std::vector<tlbm_t> inst;
@@ -332,7 +333,7 @@ struct tlbm_batch_s {
     int tpb;            // tiles per block of the flattened launch
     int graph_steps;
     int persist_steps;  // > 0: persistent kernel, this many steps per launch
-    int form_chosen;    // the caller chose a form or launch shape: one step per launch
+    int form_chosen;    // FORM_* the caller has in force: one step per launch (or the persistent form)
     int march;          // 1: calls of MULTI_CALL steps or more march three steps per launch (step_march.cu)
     int march_off;      // the tuner found one step per launch faster
     std::vector<MarchBatch> marches;  // one launch each
@@ -716,7 +717,7 @@ extern "C" int tlbm_batch_set_variant(tlbm_batch_t b, int vec, int form, int blo
     b->by = by;
     b->graph_steps = graph_steps;
     b->staged_nc = 0;  // an explicit register-kernel shape
-    b->form_chosen = 1;
+    b->form_chosen |= FORM_SHAPE;
     if (batch_dispatch(false, b->dim, b->prec, v, trt != 0, nullptr, nullptr, 0, 0, 0, dim3(), nullptr, nullptr, b->rows) !=
         cudaSuccess)
         b->rows = 1;  // no pipelined-row variant for this one
@@ -734,7 +735,7 @@ extern "C" int tlbm_batch_set_persistent(tlbm_batch_t b, int steps_per_launch) {
     if (steps_per_launch > 0 && (e != cudaSuccess || !coop))
         return bfail(b, TLBM_ERR_UNSUPPORTED, "the device has no cooperative launch");
     b->persist_steps = steps_per_launch;
-    b->form_chosen = 1;
+    b->form_chosen = steps_per_launch > 0 ? b->form_chosen | FORM_PERSISTENT : b->form_chosen & ~FORM_PERSISTENT;
     if (b->mem) return upload_tables(b);  // the persistent form runs one row per thread
     return TLBM_OK;
 }
@@ -746,7 +747,7 @@ extern "C" int tlbm_batch_set_rows(tlbm_batch_t b, int rows) {
         cudaSuccess)
         return bfail(b, TLBM_ERR_UNSUPPORTED, "batch variant (vec %d, %d rows) not built", b->vec, rows);
     b->rows = rows;
-    b->form_chosen = 1;
+    b->form_chosen |= FORM_SHAPE;
     if (b->mem) return upload_tables(b);
     return TLBM_OK;
 }
@@ -833,8 +834,11 @@ extern "C" int tlbm_batch_set_staged(tlbm_batch_t b, int consumer_warps, int sta
     if (consumer_warps != 0 && b->persist_steps > 0)
         return bfail(b, TLBM_ERR_UNSUPPORTED, "the persistent form has no staged variant");
     if (consumer_warps < 0) return bfail(b, TLBM_ERR_ARG, "consumer_warps must be >= 0");
-    b->form_chosen = 1;
-    return batch_set_staged(b, consumer_warps, stages);
+    const int before = b->form_chosen;
+    b->form_chosen = consumer_warps > 0 ? before | FORM_STAGED : before & ~FORM_STAGED;
+    const int rc = batch_set_staged(b, consumer_warps, stages);
+    if (rc != TLBM_OK) b->form_chosen = before;  // a refused form is not in force
+    return rc;
 }
 
 extern "C" int tlbm_batch_get_staged(tlbm_batch_t b, int* consumer_warps, int* stages, long long* tiles) {

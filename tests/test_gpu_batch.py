@@ -284,3 +284,37 @@ def test_marching_is_measured_for_each_kind_of_batch(T):
     assert launches(small, choose=lambda b: b.set_rows(1), trials=2) > 0
     assert launches(small) > 0
     assert launches(small) == 0
+
+
+def test_forms_turned_off_give_the_choice_back(T):
+    """Turning the staged or persistent form off, or asking for one that is
+    refused, leaves the batch as it was before: three steps per launch in calls
+    of 16 steps, unless a launch shape was chosen."""
+    b = T.Batch([(65, 70, 1, 1e6, 0.71, 0.1, i) for i in range(3)], precision=1)
+    b.init(1e-3)
+
+    def launches():
+        l0 = b.launches
+        b.step(16)
+        return b.launches - l0
+
+    assert launches() == 6
+    b.set_persistent(0)
+    b.set_staged(0)
+    assert launches() == 6
+    b.set_persistent(8)
+    assert launches() == 2
+    b.set_persistent(0)
+    assert launches() == 6
+    b.set_staged(8)
+    assert launches() == 16
+    b.set_staged(0)
+    assert launches() == 6
+    with pytest.raises(T.TlbmError):
+        b.set_staged(5)  # 4 or 8 in 2D
+    assert launches() == 6
+    b.set_rows(1)
+    b.set_staged(0)
+    b.set_persistent(0)
+    assert launches() == 16
+    b.close()
