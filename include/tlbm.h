@@ -163,8 +163,8 @@ TLBM_API int tlbm_init_fields(tlbm_t h, const float* T, const float* ux, const f
 /* Advance n >= 0 time steps (Eqs. (10)-(11), fused).  Asynchronous.  Whole
  * blocks of graph_steps steps (tlbm_set_graph, default 16) are replayed from a
  * CUDA graph captured at the first such block; the rest are plain launches.
- * Unless tlbm_set_variant, tlbm_set_staged or tlbm_set_graph was called, calls
- * of 16 steps or more may advance several steps per launch (2D cells whose size
+ * Unless tlbm_set_variant (other than with every argument 0), tlbm_set_staged or
+ * tlbm_set_graph was called, calls of 16 steps or more may advance several steps per launch (2D cells whose size
  * and storage gain by it): the same bits, fewer kernels (tlbm_launch_count). */
 TLBM_API int tlbm_step(tlbm_t h, int64_t n);
 
@@ -241,7 +241,10 @@ TLBM_API int tlbm_derived(tlbm_t h, double* out, int cap, int* count);
  * form = 0 automatic (two-relaxation-time evaluation when the rates allow it,
  * else the general MRT), 1 general MRT, 2 two-relaxation-time (TLBM_ERR_ARG if
  * the rates are not of that form); block_x (multiple of 32) x block_y threads
- * per block (0 = the tuned default of the lattice and precision).  All variants compute the same collision;
+ * per block (0 = the tuned default of the lattice and precision).  With every
+ * argument 0 the library chooses among the register kernels again (one thread per
+ * node in memory order among them) and calls of 16 steps or more may take several
+ * steps per launch.  All variants compute the same collision;
  * TLBM_ERR_UNSUPPORTED if the variant is not compiled. */
 TLBM_API int tlbm_set_variant(tlbm_t h, int vec, int form, int block_x, int block_y, int rows);
 /* Use the shared-memory staged step kernel instead: a persistent grid whose
@@ -281,7 +284,9 @@ TLBM_API int tlbm_bounds_violations(tlbm_t h, int64_t* count);
  * (blocks per SM x SMs).  Outputs may be NULL. */
 TLBM_API int tlbm_get_staged(tlbm_t h, int* tile_width, int* stages, int* blocks);
 /* Current variant (form reported as 1 MRT or 2 TRT; vec 0 for the staged
- * kernel).  Outputs may be NULL. */
+ * kernel): the register kernel that these arguments of tlbm_set_variant choose.  An
+ * FP64 handle, and an in-place 16-bit 3D one by its size, steps with one thread
+ * per node in memory order until one is chosen.  Outputs may be NULL. */
 TLBM_API int tlbm_get_variant(tlbm_t h, int* vec, int* form, int* block_x, int* block_y, int* rows);
 
 /* ---------------------------------------------------------------- batched ensemble

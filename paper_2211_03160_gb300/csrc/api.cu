@@ -334,6 +334,11 @@ static VariantDefault default_variant(int dim, int prec) {
 }
 static int default_vec(int dim, int prec) { return default_variant(dim, prec).vec; }
 
+// FP64 cells with two-relaxation-time rates: one thread per node in memory order
+static int flat_fp64(tlbm_t h) {
+    return h->prec == TLBM_FP64 && h->kp.trt && (double)h->nx * h->ny * h->nz <= FLAT_NODES;
+}
+
 extern "C" int tlbm_create(tlbm_t* out, int nx, int ny, int nz, int lattice, double Ra, double Pr, double Ma,
                            int precision, const tlbm_params* pin) {
     g_create_error[0] = 0;
@@ -444,7 +449,7 @@ extern "C" int tlbm_create(tlbm_t* out, int nx, int ny, int nz, int lattice, dou
         kp.qpf = (float)kp.qp; kp.qmf = (float)kp.qm;
     }
     h->trt = kp.trt;
-    h->flat = precision == TLBM_FP64 && kp.trt && (double)nx * ny * nz <= FLAT_NODES;
+    h->flat = flat_fp64(h);
     {
         // per-population pull / store offsets (elements, relative to a node's own
         // slot in plane 0): plane j, shifted back by the population's e_y, e_z
@@ -1208,8 +1213,16 @@ extern "C" int tlbm_set_variant(tlbm_t h, int vec, int form, int block_x, int bl
     h->staged = 0;
     h->flat = 0;
     h->multi = 0;
-    h->variant_chosen = 1;
     h->kp.xmax_load = h->kp.L.P - v;
+    if (vec > 0 || form > 0 || block_x > 0 || block_y > 0 || rows > 0) {
+        h->variant_chosen = 2;
+    } else {
+        // every argument 0: the library's choice among the register kernels
+        h->variant_chosen = 1;
+        h->flat = flat_fp64(h);
+        pick_16bit(h);
+        pick_multi(h);
+    }
     drop_graph(h);
     return TLBM_OK;
 }
@@ -1303,14 +1316,14 @@ static int set_staged(tlbm_t h, int tile_width, int stages) {
 // pairs leave over 1/16 of a row's last warps idle (step_3d_f16.cu; with none idle
 // pairs are faster: 192^3 196 us against 206, 320^3 821 and 919).
 static void pick_16bit(tlbm_t h) {
-    if (h->elem != 2 || !h->kp.trt || h->variant_chosen) return;
+    if (h->elem != 2 || !h->kp.trt || h->variant_chosen > 1) return;
     const double nodes = (double)h->nx * h->ny * h->nz;
     const long long lanes = (h->nx + 63) / 64 * 64ll;
     if (h->aa) {
         h->flat = h->dim == 3 && nodes <= FLAT_NODES && (nodes <= 4e6 || 16ll * h->nx < 15 * lanes);
         return;
     }
-    if (h->dim == 2 || (h->nx >= 384 && h->nx <= 448)) {
+    if (!h->variant_chosen && (h->dim == 2 || (h->nx >= 384 && h->nx <= 448))) {
         // (the register kernel stays if the device cannot host the staged one)
         if (set_staged(h, 0, h->dim == 3 ? 2 : 0) == TLBM_OK) return;
         h->staged = 0;
@@ -1336,7 +1349,7 @@ static void pick_16bit(tlbm_t h) {
 // against one thread per node, 193^2 12.2 both ways).
 static void pick_multi(tlbm_t h) {
     h->multi = h->march = 0;
-    if (h->dim != 2 || h->aa || !h->kp.trt || h->variant_chosen || h->graph_chosen) return;
+    if (h->dim != 2 || h->aa || !h->kp.trt || h->variant_chosen > 1 || h->graph_chosen) return;
     const long long nodes = (long long)h->nx * h->ny;
     const int strips = (h->nx + MARCH_COLUMNS - 1) / MARCH_COLUMNS;
     if (h->prec != TLBM_FP64 && !h->kp.periodic && nodes >= (h->prec == TLBM_FP32 ? 250000 : 270000) && 4 * h->nx >= 3 * strips * MARCH_COLUMNS) {
@@ -1355,7 +1368,7 @@ extern "C" int tlbm_set_staged(tlbm_t h, int tile_width, int stages) {
     TLBM_CHECK_HANDLE(h);
     const int rc = set_staged(h, tile_width, stages);
     if (rc == TLBM_OK) {
-        h->variant_chosen = 1;
+        h->variant_chosen = 2;
         h->multi = 0;
     }
     return rc;

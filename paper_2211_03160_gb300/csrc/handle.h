@@ -27,7 +27,7 @@ struct tlbm_s {
     tlbm::MultiGeo mg;         // tile of the latter
     int flat;                  // 1: the kernel with one thread per node in memory order
     int staged;                // 1: shared-memory staged (TMA bulk copy) kernel
-    int variant_chosen;        // set by tlbm_set_variant / tlbm_set_staged: keep the caller's choice
+    int variant_chosen;        // 2: tlbm_set_variant / tlbm_set_staged chose the kernel; 1: the register kernels, as the library chooses
     int staged_tw, staged_nc, staged_stages, staged_grid;
     unsigned long long wait_ns;  // staged kernel: give up on a copy after this long
     size_t staged_smem;

@@ -419,3 +419,40 @@ def test_periodic_faces_cost_as_walls(T, prec, inplace):  # noqa: F811
         best.append(min(ms))
         s.close()
     assert best[1] < 1.3 * best[0], best
+
+
+@pytest.mark.parametrize("lattice,shape,prec,inplace", [
+    (D2, (129, 129, 1), FP64, False), (D2, (513, 513, 1), 1, False), (D2, (700, 500, 1), 2, False),
+    (D3, (33, 33, 33), FP64, False), (D3, (33, 33, 33), FP64, True), (D3, (33, 33, 33), 2, True),
+    (D3, (33, 33, 33), 3, False)])
+def test_default_arguments_give_the_choice_back(T, lattice, shape, prec, inplace):  # noqa: F811
+    """tlbm_set_variant with every argument 0, at once and after another variant:
+    the launches and the bits of a handle as created, and its speed (within a
+    quarter; the kernels a chosen variant leaves take 1.4 times as long or more)
+    where no staged kernel is behind it."""
+    import torch
+
+    got = []
+    for calls in ((), ((),), ((2 if lattice == D2 or prec > 1 else 1, 2, 32, 1, 1), ())):
+        s = T.Sim(*shape, lattice=lattice, Ra=1e6, Pr=0.71, Ma=0.1, precision=prec,
+                  streaming=T.TLBM_STREAM_INPLACE if inplace else T.TLBM_STREAM_PULL)
+        for c in calls:
+            s.set_variant(*c)
+        s.init(3, 1e-2)
+        l0 = s.launches
+        s.step(64)
+        n = s.launches - l0
+        state = s.get_populations()
+        best = 1e9
+        for _ in range(8):
+            a, b = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+            a.record()
+            s.step(64)
+            b.record()
+            b.synchronize()
+            best = min(best, a.elapsed_time(b))
+        got.append((n, state, best))
+        s.close()
+    for n, state, ms in got[1:]:
+        assert n == got[0][0] and ms < 1.25 * got[0][2], (n, ms, got[0][0], got[0][2])
+        assert all(np.array_equal(p, q) for p, q in zip(state, got[0][1]))
