@@ -192,6 +192,13 @@ class ConvNet:
                 tlbm.tlbm_conv3x3_backward_data_cl(g, self.w[k], x_in, g_prev, self.gb[k - 1], B, cin, cout, H, W, ws, s)
                 g = g_prev
 
+    def a_plain_bf16(self, k):
+        """BF16 copy of layer k's weights in [cout][cin][3][3] order."""
+        torch = self.torch
+        w16 = torch.empty(self.w[k].shape, dtype=torch.bfloat16, device=self.w[k].device)
+        tlbm.tlbm_to_bf16(self.w[k], self.w[k].numel(), w16, torch.cuda.current_stream())
+        return w16
+
     def adam(self, lr: float):
         self.t += 1
         tlbm.tlbm_conv_adam_layers(

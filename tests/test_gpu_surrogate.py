@@ -276,3 +276,15 @@ def test_warm_start_reaches_steady_nusselt_sooner(T):
         assert e["held_conductive"] is not None and e["held_warm"] is not None, e
         assert e["held_warm"] <= 0.5 * e["held_conductive"], e
     torch.cuda.synchronize()
+
+
+def test_plain_bf16_weights_of_a_layer(T):
+    """ConvNet.a_plain_bf16: a layer's weights rounded to BF16, in their own order
+    (what tlbm_conv3x3_backward_data takes)."""
+    import torch
+
+    from paper_2211_03160_gb300 import surrogate
+
+    net = surrogate.ConvNet(seed=3)
+    for k, w in enumerate(net.w):
+        assert torch.equal(net.a_plain_bf16(k), w.to(torch.bfloat16))
