@@ -456,3 +456,28 @@ def test_default_arguments_give_the_choice_back(T, lattice, shape, prec, inplace
     for n, state, ms in got[1:]:
         assert n == got[0][0] and ms < 1.25 * got[0][2], (n, ms, got[0][0], got[0][2])
         assert all(np.array_equal(p, q) for p, q in zip(state, got[0][1]))
+
+
+@pytest.mark.parametrize("shape,walls", [((560, 490), 0), ((561, 487), 1), ((562, 489), 0), ((614, 450), 0),
+                                         ((615, 449), 1), ((101, 2700), 0), ((8193, 37), 0), ((700, 500), 1)])
+@pytest.mark.parametrize("prec", [2, 3])
+def test_16bit_cells_march_as_single_steps(T, shape, walls, prec):  # noqa: F811
+    """FP16 and BF16 cells of 270,000 nodes and more, all of which march: bitwise
+    one-step launches, with the launches of three steps a pass, at remainders of
+    the width by the strip and of the step count by three, in tall and flat
+    cells, and from either buffer."""
+    kw = dict(Ra=1e6, Pr=0.71, Ma=0.1, precision=prec, walls=walls)
+    a, b = T.Sim(*shape, **kw), T.Sim(*shape, **kw)
+    T.tlbm_set_graph(b.h, 0)
+    for s in (a, b):
+        s.init(3, 1e-2)
+    for n in (16, 20, 1, 33):
+        la = a.launches
+        a.step(n)
+        b.step(n)
+        assert a.launches - la == (n // 3 + n % 3 if n >= 16 else n)
+        (fa, ga), (fb, gb) = a.get_populations(), b.get_populations()
+        assert np.array_equal(fa, fb) and np.array_equal(ga, gb), n
+        assert a.status() == b.status() and a.nusselt() == b.nusselt()
+    a.close()
+    b.close()
