@@ -481,3 +481,68 @@ def test_16bit_cells_march_as_single_steps(T, shape, walls, prec):  # noqa: F811
         assert a.status() == b.status() and a.nusselt() == b.nusselt()
     a.close()
     b.close()
+
+
+BATCH_BOUNDS_SCRIPT = """
+import hashlib, json, sys
+sys.path.insert(0, {root!r})
+from paper_2211_03160_gb300 import tlbm as T
+out = {{}}
+def count(h):
+    try:
+        return T.tlbm_bounds_violations(h)
+    except T.TlbmError:
+        return None
+for lattice, shape, walls, pm, prec, inplace, steps in {cells!r}:
+    s = T.Sim(*shape, lattice=lattice, Ra=1e5, Pr=0.71, Ma=0.1, precision=prec, walls=walls, periodic_mask=pm,
+              streaming=1 if inplace else 0)
+    s.init(5, 1e-2)
+    s.step(steps)
+    m = [s.macros(d) for d in (None, __import__("torch").float32)]
+    f, g = s.get_populations()
+    h = hashlib.sha256(f.tobytes() + g.tobytes() + b"".join(q[k].cpu().numpy().tobytes() for q in m for k in sorted(q)))
+    out[repr((lattice, shape, walls, pm, prec, inplace))] = [h.hexdigest(), s.nusselt(), count(s.h)]
+    s.close()
+for prec, sizes, steps in {batches!r}:
+    b = T.Batch([tuple(q) + (1, 1e5 * (1 + i), 0.71, 0.1, i) for i, q in enumerate(sizes)], precision=prec)
+    b.init(1e-2)
+    l0 = b.launches
+    b.step(steps)
+    n = b.launches - l0
+    nu = b.nusselt()
+    for k in range(len(sizes)):
+        f, g = b.get_populations(k)
+        out[repr((prec, len(sizes), k))] = [hashlib.sha256(f.tobytes() + g.tobytes()).hexdigest(), [n, nu[k]], count(b.instance(k))]
+    b.close()
+print("RESULT " + json.dumps(out))
+"""
+
+
+def test_marching_batches_and_16bit_defaults_stay_inside_their_buffers(T):  # noqa: F811
+    """The bounds-checked build on batches that march (70 cells, two launches a
+    pass), on BF16 and 16-bit 3D cells by size, on narrow cells (whose fields
+    are walked in memory order) and with every face periodic: no access leaves
+    the population buffers, and all results are those of the release build."""
+    import json
+    import os
+    import subprocess
+    import sys
+
+    root = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+    cells = [(D2, s, w, pm, 3, False, 37) for s, w, pm in
+             (((3, 9, 1), 0, 0), ((33, 70, 1), 0, 3), ((130, 21, 1), 0, 1), ((562, 489, 1), 1, 0))]
+    cells += [(D3, (nx, 6, 5), w, pm, prec, inplace, 17) for nx, w, pm in
+              ((3, 0, 0), (35, 0, 7), (384, 0, 0), (448, 1, 0), (449, 0, 4)) for prec in (2, 3) for inplace in (False, True)]
+    cells += [(D3, (5, 4, 6), 0, pm, prec, inplace, 17) for pm in (3, 5, 7) for prec in (0, 1) for inplace in (False, True)]
+    sizes = [((3, 57, 112, 113, 200, 65, 56)[i % 7], (9, 3, 70, 31, 129)[i % 5]) for i in range(70)]
+    script = BATCH_BOUNDS_SCRIPT.format(root=root, cells=cells, batches=[(prec, sizes, 20) for prec in (1, 2, 3)])
+    res = []
+    for debug in ("0", "1"):
+        r = subprocess.run([sys.executable, "-c", script], env=dict(os.environ, TLBM_DEBUG_BOUNDS=debug),
+                           capture_output=True, text=True, timeout=900)
+        assert r.returncode == 0, r.stderr[-2000:]
+        res.append(json.loads(r.stdout.split("RESULT ")[1]))
+    for k in res[0]:
+        assert res[1][k][2] == 0, k
+        assert res[0][k][:2] == res[1][k][:2], k
+    assert sum(v[1][0] == 6 * 2 + 2 for v in res[0].values() if isinstance(v[1], list)) == 3 * 70  # they marched
