@@ -96,12 +96,8 @@ __device__ __forceinline__ void multi_ghost(S* sm, const KParams& p, const Multi
         if (rr < 0 || rr >= g.H || cc < 0 || cc >= g.W) return;  // outside: pulled by no node of this block
         const C scale = ScaleOf<C>::s(p);
         C out = val;
-        if constexpr (THERMAL) {
-            if ((ox ? 0 : 1) == p.heat_axis) {
-                const bool hi = ox ? x + ex >= p.L.nx : y + ey >= p.L.ny;
-                out = anti_bounce_back(val, PV<C>::omega(p), hi ? PV<C>::Tc(p) : PV<C>::Th(p));
-            }
-        }
+        if constexpr (THERMAL)  // axis-aligned: its direction names the face
+            if (p.heat_axis == (ex != 0 ? 0 : 1)) out = anti_bounce_back(val, PV<C>::omega(p), ex + ey > 0 ? PV<C>::Tc(p) : PV<C>::Th(p));
         S v;
         if constexpr (THERMAL) v = enc_g_step<S, C>(out, scale, salt);
         else v = enc_f_step<LS, S, C, RAW>(out, o, scale, salt);
