@@ -474,9 +474,11 @@ def summarize(ev) -> dict:
 
 def time_layers(batch: int = 48, n: int = COARSE, reps: int = 20, warmup: int = 3):
     """CUDA-event timings (ms per call, median over reps) of the 32 -> 32
-    channel layer at the training batch: forward (tcgen05), data gradient
-    (tcgen05) and weight gradient (tcgen05), each with the FLOPs of its GEMM
-    (2 x pixels x 32 x 288) as TFLOP/s and its compulsory HBM bytes as GB/s."""
+    channel layer at the training batch: forward, data gradient and weight
+    gradient (all tcgen05), as ConvNet runs them between channels-last tensors
+    (the data gradient with the relu mask and the bias sums) and as single NCHW
+    calls, each with the FLOPs of its GEMM (2 x pixels x 32 x 288) as TFLOP/s and
+    its compulsory HBM bytes as GB/s."""
     import torch
 
     s = torch.cuda.current_stream()
@@ -497,7 +499,17 @@ def time_layers(batch: int = 48, n: int = COARSE, reps: int = 20, warmup: int = 
     ws = torch.empty(tlbm.tlbm_conv3x3_workspace_bytes(B, C, M, n, n), dtype=torch.uint8, device="cuda")
     dw = torch.empty((M, C, 3, 3), dtype=torch.float32, device="cuda")
     db = torch.empty(M, dtype=torch.float32, device="cuda")
+    xc, dyc, gc = (ConvNet._cl(torch, B, C, n, n, "cuda") for _ in range(3))
+    tlbm.tlbm_conv_channels_last(x, B, C, n, n, xc, s)
+    tlbm.tlbm_conv_channels_last(dy16, B, M, n, n, dyc, s)
+    wc = torch.empty(tlbm.tlbm_conv3x3_cl_workspace_bytes(B, C, M, n, n), dtype=torch.uint8, device="cuda")
     ops = {
+        "forward_cl": (lambda: tlbm.tlbm_conv3x3_forward_cl(xc, a, bias, None, gc, B, C, M, n, n, 1, s),
+                       xc.numel() * 2 + gc.numel() * 2),
+        "backward_data_cl": (lambda: tlbm.tlbm_conv3x3_backward_data_cl(dyc, w, xc, gc, db, B, C, M, n, n, wc, s),
+                             dyc.numel() * 2 + xc.numel() * 2 + gc.numel() * 2),
+        "backward_weight_cl": (lambda: tlbm.tlbm_conv3x3_backward_weight_cl(xc, dyc, dw, B, C, M, n, n, wc, s),
+                               xc.numel() * 2 + dyc.numel() * 2),
         "forward": (lambda: tlbm.tlbm_conv3x3_forward(x, a, bias, y, act, B, C, M, n, n, 1, s),
                     x.numel() * 2 + y.numel() * 6),
         "backward_data": (lambda: tlbm.tlbm_conv3x3_backward_data(dy16, w16, dx, B, C, M, n, n, at, s),
