@@ -65,11 +65,12 @@ __device__ __noinline__ void macros_node_d(const S* own, const KParams& p, const
 }
 
 // Bound by HBM for FP32 fields (the state read once, the fields written once)
-// and by the FP64 pipe for FP64 ones.  40 registers for FP32 fields of 2D 16-bit
-// states, which let more of a node's loads go out together than the 32 the
-// compiler takes by itself: 8193^2 FP16 799 -> 758 us.
+// and by the FP64 pipe for FP64 ones.  40 registers for the FP32 fields of 2D
+// 16-bit and 3D FP32 states: the compiler's own 32 send too few of a node's loads
+// out together (8193^2 FP16 799 -> 758 us), its 42 leave five blocks on an SM
+// (385^3 FP32 1339 -> 1246).
 template <int DIM, class S, class O>
-constexpr int MACRO_BLOCKS = DIM == 2 && sizeof(S) == 2 && sizeof(O) == 4 ? 6 : 0;  // per SM, 0: as it comes
+constexpr int MACRO_BLOCKS = sizeof(O) == 4 && sizeof(S) == (DIM == 2 ? 2 : 4) ? 6 : 0;  // per SM, 0: as it comes
 template <int DIM, class S, class O, bool FLAT>
 __global__ void __launch_bounds__(THREADS, (MACRO_BLOCKS<DIM, S, O>))
     macros_kernel(const S* __restrict__ buf, const KParams p, const DiagOff k, unsigned segs, unsigned n,

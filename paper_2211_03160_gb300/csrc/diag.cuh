@@ -121,10 +121,11 @@ __device__ __forceinline__ float df_val(Df a) { return __fadd_rn(a.h, a.l); }
 
 // FP32 fields of a node of FP32 / FP16 / BF16 storage, rounded from double-FP32
 // arithmetic: the sums are exact to the last bits of the low words (about
-// 2^-46), so the results are those of FP64 arithmetic rounded to FP32.  The same
-// in FP64 took 51 FP64-pipe operations (conversions included) per node in 2D:
-// the fields of an 8193^2 FP32 state 7.36 ms, now 0.87 (5.6 TB/s); of a 385^3
-// FP16 state 11.5 ms, now 1.26.
+// 2^-46), so the results are those of FP64 arithmetic rounded to FP32, except
+// where a rounding boundary falls between the two (a few nodes in a million, each
+// within 0.5001 units).  The same in FP64 took 51 FP64-pipe operations
+// (conversions included) per node in 2D: the fields of an 8193^2 FP32 state 7.36
+// ms, now 0.88 (5.5 TB/s); of a 385^3 FP16 state 11.5 ms, now 1.26.
 // false: some value is outside the range where this holds (the caller then
 // evaluates the node in FP64).
 template <int DIM>
@@ -147,6 +148,16 @@ __device__ __forceinline__ bool diag_macros_f(const float (&f)[Lat<DIM>::F::Q], 
         constexpr int i = decltype(ii)::value;
         if constexpr (i > 0) df_add(t, g[i]);
     });
+    // where terms cancel, much of a sum may stand in its low word, whose 24 bits then
+    // decide: bring it up (always doing so took 8 % longer in 3D FP32)
+    bool low = fabsf(t.l) > 0x1p-12f * fabsf(t.h);
+#pragma unroll
+    for (int ax = 0; ax < DIM; ++ax) low |= fabsf(j[ax].l) > 0x1p-12f * fabsf(j[ax].h);
+    if (low) {
+#pragma unroll
+        for (int ax = 0; ax < DIM; ++ax) j[ax] = two_sum(j[ax].h, j[ax].l);
+        t = two_sum(t.h, t.l);
+    }
     Df r = two_sum(1.0f, dr.h);
     r.l = __fadd_rn(r.l, dr.l);
     rho = df_val(r);

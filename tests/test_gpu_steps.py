@@ -546,3 +546,23 @@ def test_marching_batches_and_16bit_defaults_stay_inside_their_buffers(T):  # no
         assert res[1][k][2] == 0, k
         assert res[0][k][:2] == res[1][k][:2], k
     assert sum(v[1][0] == 6 * 2 + 2 for v in res[0].values() if isinstance(v[1], list)) == 3 * 70  # they marched
+
+
+@pytest.mark.parametrize("lattice,shape", [(D2, (513, 400, 1)), (D2, (33, 300, 1)), (D3, (65, 50, 40))])
+@pytest.mark.parametrize("prec", [1, 2, 3])
+@pytest.mark.parametrize("noise,steps", [(1e-2, 300), (1e-6, 60), (1e-9, 200)])
+def test_fp32_fields_of_weak_and_developed_flow(T, lattice, shape, prec, noise, steps):  # noqa: F811
+    """FP32 fields are the FP64 ones rounded also where the populations nearly
+    cancel (a velocity far below them, as at the onset of convection): within
+    half a unit and 2^-8 of one, what the two evaluations may differ by."""
+    import torch
+
+    s = T.Sim(*shape, lattice=lattice, Ra=1e7, Pr=0.71, Ma=0.1, precision=prec)
+    s.init(7, noise)
+    s.step(steps)
+    m, m32 = s.macros(), s.macros(torch.float32)
+    for k in m32:
+        ref = m[k].cpu().numpy()
+        ulp = np.spacing(np.abs(ref.astype(np.float32))).astype(np.float64)
+        assert (np.abs(m32[k].cpu().numpy().astype(np.float64) - ref) <= (0.5 + 2.0 ** -8) * ulp).all(), k
+    s.close()
