@@ -1305,16 +1305,19 @@ static int set_staged(tlbm_t h, int tile_width, int stages) {
 // 2D, two buffers: the staged kernel, 512-node tiles with the stages chosen as
 // above (2 stages and three blocks per SM on GB300, the fastest there).
 // 3D, two buffers: the staged kernel (2 stages, two blocks per SM) takes a row per
-// tile and seven warps, so it is for rows that nearly fill those: 385^3 1250 us per
-// step against 1297, 448 x 193^2 346 and 352 (and 385 x 129^2 174 and 166); but
-// 321^3 881 and 798, 193^3 252 and 208, 65^3 45 and 17, 513 x 193^2 654 and 435.  Else warps inside rows: one node a
-// thread up to 4 M nodes, where a second one in flight per thread is worth less
-// than twice the warps, then node pairs (33^3 7.0 us against 12.0, 97^3 39 and 50,
-// 145^3 101 and 113, 161^3 135 and 134, 177^3 173 and 166).  (Figures of this
-// comment: before the wall rules went face by face, which took 1 to 10 % off all.)
+// tile and seven warps, so it is for rows that nearly fill those.  us per step,
+// staged and node pairs in rows: 385^3 1110 and 1283, 448 x 385^2 1160 and 1305, 385 x
+// 129^2 133 and 150, 416 x 129^2 134 and 150, 448 x 129^2 137 and 153; at the border 384
+// x 129^2 136 and 132, 383 x 129^2 143 and 141, 449 x 129^2 254 and 170; 321^3 782 and
+// 791, 193^3 208 and 193, 65^3 26 and 14.  (Cells too small to fill the GPU lose: 385 x
+// 33^2 15.5 and 12.7.)  Else warps inside rows: one node a thread up to 4 M nodes,
+// where a second one in flight per thread is worth less than twice the warps, then
+// node pairs (one node and pairs: 33^3 5.0 and 6.4, 65^3 13.0 and 14.0, 145^3 95 and
+// 94, 161^3 129 and 116; between, 97^3 36 and 34, 129^3 75 and 72).
 // 3D, in place: one thread per node in memory order for small cells and where
-// pairs leave over 1/16 of a row's last warps idle (step_3d_f16.cu; with none idle
-// pairs are faster: 192^3 196 us against 206, 320^3 821 and 919).
+// pairs leave over 1/16 of a row's last warps idle (step_3d_f16.cu).  With none
+// idle it was pairs' gain before the wall rules went face by face (192^3 196 us
+// against 206, 320^3 821 and 919).
 static void pick_16bit(tlbm_t h) {
     if (h->elem != 2 || !h->kp.trt || h->variant_chosen > 1) return;
     const double nodes = (double)h->nx * h->ny * h->nz;
@@ -1339,14 +1342,16 @@ static void pick_16bit(tlbm_t h) {
 
 // Several steps per launch: 2D two-buffer cells with two-relaxation-time rates
 // whose launches the caller has not chosen.  FP32 and 16-bit cells with walls all
-// around go through step_march.cu from 250,000 / 270,000 nodes (513^2 FP32: 6.7 us
-// per step against 7.1 in tiles and 10.5 singly; FP16: 7.6, 7.4 and 12.3) unless
-// their width would leave more than a quarter of its strips' columns idle.  Else tiles (step_multi.cu) up to the size where
-// one step fills the GPU.  FP32, FP16 and BF16: 300,000 nodes (a 513^2 cell gains 1.5x, a 1025^2
-// one 1.1x in FP32 and loses a quarter in FP16), the 16-bit ones not with rows of
-// over 2048 nodes, which suit the staged kernel's tiles (4000 x 70: 8.5 us per
-// step staged, 8.8 here); FP64, bound by its pipe, 30,000 (129^2 8.1 -> 7.8 us
-// against one thread per node, 193^2 12.2 both ways).
+// around go through step_march.cu from 250,000 / 270,000 nodes unless their width
+// would leave more than a quarter of its strips' columns idle (513^2 when the line
+// was drawn, FP32: 6.7 us per step, 7.1 in tiles, 10.5 singly; FP16: 7.6, 7.4 and
+// 12.3; now 5.7 against 7.4 singly and 6.8 against 8.9).  Else tiles
+// (step_multi.cu) up to the size where one step fills the GPU.  FP32, FP16 and BF16:
+// 300,000 nodes (a 513^2 cell gains 1.5x, a 1025^2 one 1.1x in FP32 and loses a
+// quarter in FP16), the 16-bit ones not with rows of over 2048 nodes, which suit
+// the staged kernel's tiles (4000 x 70: 8.5 us per step staged, 8.8 here); FP64,
+// bound by its pipe, 30,000 (65^2 6.9 -> 5.4 us against one thread per node, 129^2
+// 7.0 and 7.2, 193^2 12.2 both ways).
 static void pick_multi(tlbm_t h) {
     h->multi = h->march = 0;
     if (h->dim != 2 || h->aa || !h->kp.trt || h->variant_chosen > 1 || h->graph_chosen) return;

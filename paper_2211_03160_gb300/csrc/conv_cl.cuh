@@ -20,8 +20,8 @@
 // forward 36.4 -> 16.5, data gradient with mask and bias sums 35.1 (no mask, no
 // sums) -> 24.6, weight gradient with its reduction 100.7 -> 30.8; the training
 // iteration of that network 787 -> 297.  What bounds them now: issue and latency of
-// the copies (a tile's 16-byte pieces, 40 to 120 cp.async a thread); the tensor
-// cores are idle most of the time and DRAM traffic stays in L2.
+// the copies (a tile's 16-byte pieces, 40 to 120 cp.async a thread) and the barriers
+// around them; the tensor pipe is 11 to 15 % active and what they write stays in L2.
 // Included by conv.cu, whose geometry and descriptor helpers it uses.
 #pragma once
 

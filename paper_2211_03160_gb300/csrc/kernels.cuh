@@ -1121,9 +1121,9 @@ __device__ __forceinline__ void any_face(S* __restrict__ dst, const KParams& p, 
 // crowd the instruction cache of the hot path.  A step of a small cell lasts as
 // long as its face threads, and in a large one they end the warps of a row late:
 // going through all populations of such a node instead of the 4 (2D) or 6 (3D)
-// that can leave through a face cost 3D FP32 6.8 us per step at 33^3 against 4.5
-// now, 65^3 17.5 and 12.3, 385^3 FP16 1250 and 1113; 2D in place FP32 117 x 109 10
-// and 4.9; with periodic x, 193^3 FP16 480 and 227, 385^3 4027 and 1457.
+// that can leave through a face cost 3D FP32 6.8 us per step at 33^3 against 4.4
+// now, 65^3 17.5 and 12.2, 385^3 FP16 1250 and 1113; 2D in place FP32 117 x 109 10
+// and 4.9; with periodic x, 193^3 FP16 480 and 197, 385^3 4027 and 1218.
 // One face per call, its populations' values handed over (post: those of all VEC
 // nodes, in their order):
 template <class LS, int AXIS, int SIDE>

@@ -30,9 +30,8 @@ cudaError_t launch_step_3d_f16(int prec, int vec, bool trt, int rows, const void
 
 // Halves of an in-place pair with one thread per node, nodes in their order in
 // memory: 64 registers, and no lane idle at a row's end.  us per step, warps of
-// node pairs inside rows -> this kernel: 33^3 13.8 -> 8.4, 65^3 25.6 -> 16.7, 97^3
-// 52 -> 35, 129^3 96 -> 73, 193^3 245 -> 213, 257^3 525 -> 479, 385^3 1570 -> 1561
-// (since then the wall rules have taken another 3.4 us off 33^3 and 11 off 193^3).
+// node pairs inside rows -> this kernel: 33^3 7.5 -> 5.0, 65^3 16.4 -> 11.3, 97^3
+// 34 -> 28, 129^3 78 -> 64, 193^3 220 -> 201, 257^3 481 -> 465, 385^3 1504 and 1515.
 template <class S>
 static cudaError_t launch_flat_aa(int mode, const void* src, void* dst, const KParams& p, cudaStream_t s) {
     if (mode == AA_EVEN) return launch_flat_as<3, S, AA_EVEN>(src, dst, p, s);

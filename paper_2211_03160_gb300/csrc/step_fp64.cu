@@ -44,7 +44,8 @@ const void* func_step_f64(int dim, int vec, bool trt, int rows) {
 // on its rest: 14 % of the lanes at 193 nodes,
 // 20 % at 129.  us per step, warps inside rows -> this kernel: 193^3 3415 -> 2904,
 // 129^3 1097 -> 877, 65^3 174 -> 125; 129^2 13.3 -> 8.1, 513^2 76 -> 63, 2049^2
-// 944 -> 925, 4097^2 3682 -> 3681; in place the same.
+// 944 -> 925, 4097^2 3682 -> 3681; in place the same.  (With the wall rules face by
+// face and nine blocks per SM in 2D: 129^2 7.0, 513^2 61.5, 2049^2 909, 4097^2 3621.)
 template <int DIM>
 static cudaError_t launch_flat_f64(int mode, const void* src, void* dst, const KParams& p, cudaStream_t s) {
     if (mode == PULL) return launch_flat_as<DIM, double, PULL>(src, dst, p, s);

@@ -23,15 +23,16 @@
 // at the side walls, and in place of the missing row's values at the bottom and
 // top.
 //
-// What bounds it now: instruction issue and latency at twelve warps an SM (158
-// registers a thread); HBM moves 37 of the 112 bytes per update.  GLUPS on GB300
+// What bounds it now: instruction issue and latency at twelve warps an SM (167
+// registers a thread; at 4097^2 issue slots 59 % used, 173 instructions per node and
+// step, 211 in FP16); HBM moves 37 of the 112 bytes per update.  GLUPS on GB300
 // by steps per pass (blocks of four warps per SM) at 8193^2: 2 (3) 111, 3 (3)
 // 132, 3 (4, spilling) 80, 4 (2) 124; 2 (5, at 96 registers) 75.  us per step,
-// one-step kernel -> this: 513^2 10.4 -> 6.7, 1025^2 24.7 -> 13.4, 2049^2 77.1 ->
-// 40.4, 4097^2 281 -> 139, 8193^2 1084 -> 499 (134 GLUPS).  16-bit storage rounds (and
+// one-step kernel -> this: 513^2 7.4 -> 5.7, 1025^2 22.2 -> 12.4, 2049^2 75.5 ->
+// 38.1, 4097^2 279 -> 135, 8193^2 1081 -> 493 (136 GLUPS).  16-bit storage rounds (and
 // hashes) every value of every step, so its steps cost more instructions and its
-// one-step kernel was further from the HBM rate: FP16 1025^2 18.9 -> 16.4, 2049^2 48.2
-// -> 46.1, 4097^2 179 -> 160, 8193^2 643 -> 563 (119 GLUPS).
+// one-step kernel was further from the HBM rate: FP16 1025^2 17.3 -> 15.7, 2049^2 47.5
+// -> 44.8, 4097^2 173 -> 157, 8193^2 620 -> 564 (119 GLUPS).
 //
 // Every node gets bitwise the values of the one-step kernels.
 #include <algorithm>

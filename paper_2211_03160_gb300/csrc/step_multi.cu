@@ -13,10 +13,10 @@
 // of it launch, instruction fetch and one pass through memory latency.  K steps a
 // launch pay that once and run the collision from a warm instruction cache, for
 // the price of (1 + 2 (K - 1) / tile)^2 redundant updates.  us per step on GB300,
-// one-step launches in a CUDA graph -> this kernel: FP32 65^2 9.0 -> 2.0, 129^2
-// 8.2 -> 2.4, 257^2 8.1 -> 2.9, 513^2 10.4 -> 7.1; FP16 129^2 6.7 -> 2.8, 257^2 7.0 ->
-// 3.2, 513^2 12.1 -> 7.4; FP64, whose pipe the redundant updates keep busy, 65^2
-// 7.7 -> 5.8, 129^2 8.1 -> 7.8.  (Launching the next block of steps early, with
+// one-step launches in a CUDA graph -> this kernel: FP32 65^2 5.1 -> 1.7, 129^2
+// 4.8 -> 1.9, 257^2 4.8 -> 2.4; FP16 129^2 4.5 -> 2.2, 257^2 4.9 -> 2.7, 500^2 8.7 ->
+// 6.5; FP64, whose pipe the redundant updates keep busy, 65^2 6.9 -> 5.4 and 129^2
+// 7.0 and 7.2.  (Launching the next block of steps early, with
 // programmatic stream serialization, gained at most 2 % and lost 20 % in FP64.)
 //
 // Every node gets bitwise the values of the one-step kernels: the same
