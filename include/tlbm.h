@@ -253,9 +253,10 @@ TLBM_API int tlbm_set_variant(tlbm_t h, int vec, int form, int block_x, int bloc
  * shared memory (completing on mbarriers), 4 or 8 warps (2D) or 4 or 7 warps
  * (3D) collide two nodes per thread and store them straight to global memory;
  * `stages` tiles are in flight per block.  Handles with FP16/BF16 storage and
- * two-relaxation-time rates start on this kernel in 2D (stages automatic) and
- * in 3D with rows of 384 to 448 nodes (2 stages), whole rows, unless
- * tlbm_set_variant was called.
+ * two-relaxation-time rates take this kernel for single steps in 2D (stages
+ * automatic) and in 3D with rows of 384 to 448 nodes (2 stages), whole rows,
+ * unless tlbm_set_variant was called; calls of 16 steps or more of 2D cells may
+ * take several steps per launch instead (tlbm_step).
  * tile_width: a multiple of 16 bytes' worth of elements, at most 512 in 2D and
  * 448 in 3D (0 = whole rows up to that width, else that width); stages: 2 .. 8 (0 = the most tiles in
  * flight per SM, blocks x stages, up to six, more blocks first).  FP32/FP16/BF16 storage with two-relaxation-time rates

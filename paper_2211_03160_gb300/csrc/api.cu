@@ -478,6 +478,8 @@ extern "C" int tlbm_create(tlbm_t* out, int nx, int ny, int nz, int lattice, dou
     h->rows = default_variant(dim, precision).rows;
     kp.xmax_load = kp.L.P - h->vec;
     kp.gbeta = h->gbeta; kp.omega = h->omega; kp.Th = h->prm.Th; kp.Tc = h->prm.Tc; kp.a_T = h->a_T;
+    kp.wTh = kp.omega * kp.Th;
+    kp.wTc = kp.omega * kp.Tc;
     for (int a = 0; a < 3; ++a) {
         kp.body[a] = prm.body_force[a];
         kp.bodyf[a] = (float)prm.body_force[a];

@@ -56,6 +56,7 @@ struct KParams {
     int grav_axis;           // 1 (2D) or 2 (3D)
     int xmax_load;           // largest safe vector start for lanes past the row end
     double gbeta, omega, Th, Tc, a_T;
+    double wTh, wTc;         // omega Th, omega Tc
     double body[3];
     double S[MAXQ], Sh[MAXQ];  // flow rates and 1 - S/2
     double Q[7];
@@ -947,11 +948,14 @@ __device__ __forceinline__ void pull_row(const S* __restrict__ q, int lane, C (&
 constexpr int PULL = 0, AA_EVEN = 1, AA_ODD = 2;
 constexpr int FLAT_THREADS = 128;
 
-// Anti-bounce-back at a wall of temperature Tw: omega Tw - val, in operations that
-// the compiler neither contracts nor splits, so that every kernel returns the same
-// bits whatever its translation unit's flags (FP64: two roundings, FP32: one).
-__device__ __forceinline__ double anti_bounce_back(double val, double omega, double Tw) { return dsub(dmul(omega, Tw), val); }
-__device__ __forceinline__ float anti_bounce_back(float val, float omega, float Tw) { return __fmaf_rn(omega, Tw, -val); }
+// Anti-bounce-back at the cold (HI) or hot wall of temperature Tw: omega Tw - val,
+// in operations that the compiler neither contracts nor splits, so that every
+// kernel returns the same bits whatever its translation unit's flags (FP64: two
+// roundings, the product's on the host; FP32: one).
+template <bool HI>
+__device__ __forceinline__ double anti_bounce_back(double val, const KParams& p) { return dsub(HI ? p.wTc : p.wTh, val); }
+template <bool HI, class PT>
+__device__ __forceinline__ float anti_bounce_back(float val, const PT& p) { return __fmaf_rn(p.omegaf, HI ? p.Tcf : p.Thf, -val); }
 
 // Write the post-collision value `val` of population i (set LS, flow or
 // thermal) of node (x, y, z), which leaves the cell through a wall, where the
@@ -976,7 +980,7 @@ __device__ __forceinline__ void ghost_write(S* __restrict__ base, const KParams&
     C out = val;
     if constexpr (THERMAL)  // axis-aligned: its direction names the face
         if (p.heat_axis == (ex != 0 ? 0 : (ey != 0 ? 1 : 2)))
-            out = anti_bounce_back(val, PV<C>::omega(p), ex + ey + ez > 0 ? PV<C>::Tc(p) : PV<C>::Th(p));
+            out = anti_bounce_back<(ex + ey + ez > 0)>(val, p);
     constexpr int plane = MODE == AA_EVEN ? i : LS::opp(i);
     const long long s = MODE == AA_ODD ? L.slot(x, y, z) : L.slot(dx, dy, dz);
     if constexpr (THERMAL) *TLBM_DBG(p, (base + ((long long)plane * L.plane + s)), 0, 1) = enc_g_step<S, C>(out, scale, salt);

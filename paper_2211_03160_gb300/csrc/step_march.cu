@@ -108,17 +108,17 @@ __device__ __forceinline__ float2 march_lo(float2 w, float2 v) { return make_flo
 __device__ __forceinline__ float2 march_hi(float2 w, float2 v) { return make_float2(w.x, v.y); }
 __device__ __forceinline__ uint32_t march_lo(uint32_t w, uint32_t v) { return __byte_perm(w, v, 0x3254); }
 __device__ __forceinline__ uint32_t march_hi(uint32_t w, uint32_t v) { return __byte_perm(w, v, 0x7610); }
-// The thermal wall rule for a post-collision value (scaled as it is stored,
+// The thermal wall rule of the lower / upper (HI) wall for a post-collision value (scaled as it is stored,
 // not yet rounded): anti-bounce-back at a wall of temperature Tw, bounce-back at
 // an adiabatic one.
-template <class PT>
-__device__ __forceinline__ float march_rule(float v, bool iso, const PT& p, float Tw) {
+template <bool HI, class PT>
+__device__ __forceinline__ float march_rule(float v, bool iso, const PT& p) {
     const float val = v * ScaleOf<float>::inv(p);
-    return (iso ? anti_bounce_back(val, p.omegaf, Tw) : val) * ScaleOf<float>::s(p);
+    return (iso ? anti_bounce_back<HI>(val, p) : val) * ScaleOf<float>::s(p);
 }
-template <class PT>
-__device__ __forceinline__ float2 march_rule(float2 v, bool iso, const PT& p, float Tw) {
-    return make_float2(march_rule(v.x, iso, p, Tw), march_rule(v.y, iso, p, Tw));
+template <bool HI, class PT>
+__device__ __forceinline__ float2 march_rule(float2 v, bool iso, const PT& p) {
+    return make_float2(march_rule<HI>(v.x, iso, p), march_rule<HI>(v.y, iso, p));
 }
 
 // copy the stored pairs a lane pulls for one row (before the shift along x) to
@@ -201,8 +201,8 @@ __device__ __forceinline__ void march_pull(MarchKept<S>& k, float2 (&f)[9], floa
         // keep what row r's node at a side wall gets back
         const bool upper = x + 1 == L.nx - 1;
         k.wd = march_one(x == 0 ? F[7] : F[8], upper);
-        const float t = x == 0 ? march_rule(g[3].x, !heat_y, p, p.Thf)
-                               : march_rule(upper ? g[1].y : g[1].x, !heat_y, p, p.Tcf);
+        const float t = x == 0 ? march_rule<false>(g[3].x, !heat_y, p)
+                               : march_rule<true>(upper ? g[1].y : g[1].x, !heat_y, p);
         k.wg = march_pack1<S>(t, salt);
     }
     // keep row r
@@ -224,9 +224,9 @@ __device__ __forceinline__ void march_pull(MarchKept<S>& k, float2 (&f)[9], floa
         k.u0[0] = F[4];
         k.u0[1] = march_shift<-1>(F[7]);
         k.u0[2] = march_shift<1>(F[8]);
-        k.u0[3] = march_pack<S>(march_rule(g[4], heat_y, p, p.Thf), salt);
+        k.u0[3] = march_pack<S>(march_rule<false>(g[4], heat_y, p), salt);
     }
-    if (r == L.ny - 1) k.u1[3] = march_pack<S>(march_rule(g[2], heat_y, p, p.Tcf), salt);
+    if (r == L.ny - 1) k.u1[3] = march_pack<S>(march_rule<true>(g[2], heat_y, p), salt);
 #pragma unroll
     for (int i = 0; i < 9; ++i) f[i] = march_unpack<S>(n[i]);
 #pragma unroll

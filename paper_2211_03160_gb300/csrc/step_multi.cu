@@ -97,7 +97,7 @@ __device__ __forceinline__ void multi_ghost(S* sm, const KParams& p, const Multi
         const C scale = ScaleOf<C>::s(p);
         C out = val;
         if constexpr (THERMAL)  // axis-aligned: its direction names the face
-            if (p.heat_axis == (ex != 0 ? 0 : 1)) out = anti_bounce_back(val, PV<C>::omega(p), ex + ey > 0 ? PV<C>::Tc(p) : PV<C>::Th(p));
+            if (p.heat_axis == (ex != 0 ? 0 : 1)) out = anti_bounce_back<(ex + ey > 0)>(val, p);
         S v;
         if constexpr (THERMAL) v = enc_g_step<S, C>(out, scale, salt);
         else v = enc_f_step<LS, S, C, RAW>(out, o, scale, salt);
