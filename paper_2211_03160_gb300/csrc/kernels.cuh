@@ -957,6 +957,11 @@ __device__ __forceinline__ double anti_bounce_back(double val, const KParams& p)
 template <bool HI, class PT>
 __device__ __forceinline__ float anti_bounce_back(float val, const PT& p) { return __fmaf_rn(p.omegaf, HI ? p.Tcf : p.Thf, -val); }
 
+// Whether a kernel names the walls: all but the 16-bit march, which at its 128
+// registers takes 1 % longer with them named (8193^2 FP16 1692 -> 1711 us a pass).
+template <class S, bool CLOSED>
+constexpr bool wall_named = !(CLOSED && sizeof(S) == 2);
+
 // Write the post-collision value `val` of population i (set LS, flow or
 // thermal) of node (x, y, z), which leaves the cell through a wall, where the
 // next step will read it: half-way bounce-back, as population ibar of the same
@@ -966,7 +971,9 @@ __device__ __forceinline__ float anti_bounce_back(float val, const PT& p) { retu
 // own slot of the opposite direction).
 // RAW: flow values are f_i as stored (FP64 with the two-relaxation-time
 // collision) rather than deviations.
-template <class LS, bool THERMAL, int i, class S, class C, int MODE, bool RAW>
+// NAMED: the wall is known from the direction when the kernel is compiled; else the
+// node's place tells it, the same values (wall_named).
+template <class LS, bool THERMAL, int i, class S, class C, int MODE, bool RAW, bool NAMED = true>
 __device__ __forceinline__ void ghost_write(S* __restrict__ base, const KParams& p, int x, int y, int z, C val,
                                             C scale, uint32_t salt) {
     constexpr int ex = LS::e(i, 0), ey = LS::e(i, 1), ez = LS::e(i, 2);
@@ -978,9 +985,14 @@ __device__ __forceinline__ void ghost_write(S* __restrict__ base, const KParams&
     const bool oz = (ez != 0) && (dz < 0 || dz >= L.nz);
     if (!(ox || oy || oz)) return;
     C out = val;
-    if constexpr (THERMAL)  // axis-aligned: its direction names the face
-        if (p.heat_axis == (ex != 0 ? 0 : (ey != 0 ? 1 : 2)))
-            out = anti_bounce_back<(ex + ey + ez > 0)>(val, p);
+    if constexpr (THERMAL && NAMED) {  // axis-aligned: exactly one axis is crossed
+        if (p.heat_axis == (ex != 0 ? 0 : (ey != 0 ? 1 : 2))) out = anti_bounce_back<(ex + ey + ez > 0)>(val, p);
+    } else if constexpr (THERMAL) {
+        if (p.heat_axis == (ox ? 0 : (oy ? 1 : 2))) {
+            const bool hi = ox ? dx >= L.nx : (oy ? dy >= L.ny : dz >= L.nz);
+            out = hi ? anti_bounce_back<true>(val, p) : anti_bounce_back<false>(val, p);
+        }
+    }
     constexpr int plane = MODE == AA_EVEN ? i : LS::opp(i);
     const long long s = MODE == AA_ODD ? L.slot(x, y, z) : L.slot(dx, dy, dz);
     if constexpr (THERMAL) *TLBM_DBG(p, (base + ((long long)plane * L.plane + s)), 0, 1) = enc_g_step<S, C>(out, scale, salt);
@@ -1089,7 +1101,7 @@ __device__ __forceinline__ void pull_node_vec(const S* __restrict__ own, const K
 // the face (AXIS, SIDE) it lies on: those with e_AXIS = SIDE, value val(j) (all
 // numbered flow first).  WALLED: that axis is not periodic, so they meet a wall
 // whatever else they cross.
-template <int DIM, class S, class C, int MODE, bool RAW, int AXIS, int SIDE, bool WALLED, class Val>
+template <int DIM, class S, class C, int MODE, bool RAW, int AXIS, int SIDE, bool WALLED, bool NAMED, class Val>
 __device__ __forceinline__ void face_writes(S* __restrict__ dst, const KParams& p, int x, int y, int z, Val val, uint32_t salt) {
     using LF = typename Lat<DIM>::F;
     using LG = typename Lat<DIM>::G;
@@ -1100,7 +1112,7 @@ __device__ __forceinline__ void face_writes(S* __restrict__ dst, const KParams& 
     static_for<LF::Q>([&](auto ii) {
         constexpr int i = decltype(ii)::value;
         if constexpr (LF::e(i, AXIS) == SIDE) {
-            if constexpr (WALLED) ghost_write<LF, false, i, S, C, MODE, RAW>(dst, p, x, y, z, val(ii), scale, salt);
+            if constexpr (WALLED) ghost_write<LF, false, i, S, C, MODE, RAW, NAMED>(dst, p, x, y, z, val(ii), scale, salt);
             else image_write<LF, false, i, S, C, MODE, RAW, AXIS, SIDE>(dst + own, p, at, val(ii), scale, salt);
         }
     });
@@ -1108,15 +1120,15 @@ __device__ __forceinline__ void face_writes(S* __restrict__ dst, const KParams& 
         constexpr int i = decltype(ii)::value;
         if constexpr (LG::e(i, AXIS) == SIDE) {
             constexpr std::integral_constant<int, LF::Q + i> j{};
-            if constexpr (WALLED) ghost_write<LG, true, i, S, C, MODE, RAW>(gdst, p, x, y, z, val(j), scale, salt);
+            if constexpr (WALLED) ghost_write<LG, true, i, S, C, MODE, RAW, NAMED>(gdst, p, x, y, z, val(j), scale, salt);
             else image_write<LG, true, i, S, C, MODE, RAW, AXIS, SIDE>(gdst + own, p, at, val(j), scale, salt);
         }
     });
 }
 template <int DIM, class S, class C, int MODE, bool RAW, int AXIS, int SIDE, bool CLOSED, class Val>
 __device__ __forceinline__ void any_face(S* __restrict__ dst, const KParams& p, int x, int y, int z, Val val, uint32_t salt) {
-    if (!CLOSED && (p.periodic & (1 << AXIS))) face_writes<DIM, S, C, MODE, RAW, AXIS, SIDE, false>(dst, p, x, y, z, val, salt);
-    else face_writes<DIM, S, C, MODE, RAW, AXIS, SIDE, true>(dst, p, x, y, z, val, salt);
+    if (!CLOSED && (p.periodic & (1 << AXIS))) face_writes<DIM, S, C, MODE, RAW, AXIS, SIDE, false, true>(dst, p, x, y, z, val, salt);
+    else face_writes<DIM, S, C, MODE, RAW, AXIS, SIDE, true, true>(dst, p, x, y, z, val, salt);
 }
 
 // The rules of a thread's nodes at the edge of the cell, one face after the other
@@ -1142,13 +1154,13 @@ __host__ __device__ constexpr int leaving_index(int j) {  // of population j (fl
     using LG = typename Lat<DIM>::G;
     return j < LF::Q ? leaving<LF, AXIS, SIDE>(j) : leaving<LF, AXIS, SIDE>(LF::Q) + leaving<LG, AXIS, SIDE>(j - LF::Q);
 }
-template <int DIM, class S, int VEC, class C, int MODE, bool RAW, int AXIS, int SIDE, bool WALLED>
+template <int DIM, class S, int VEC, class C, int MODE, bool RAW, int AXIS, int SIDE, bool WALLED, bool NAMED>
 __device__ __noinline__ void face_call(S* __restrict__ dst, const KParams& p, int x0, int y, int z,
                                        const C* __restrict__ post, uint32_t salt) {
 #pragma unroll(WALLED && VEC <= 4 ? VEC : 1)
     for (int k = 0; k < VEC; ++k) {
         if (x0 + k >= p.L.nx) break;
-        face_writes<DIM, S, C, MODE, RAW, AXIS, SIDE, WALLED>(
+        face_writes<DIM, S, C, MODE, RAW, AXIS, SIDE, WALLED, NAMED>(
             dst, p, x0 + k, y, z, [&](auto jj) { return post[leaving_index<DIM, AXIS, SIDE>(decltype(jj)::value) * VEC + k]; }, salt);
     }
 }
@@ -1171,8 +1183,8 @@ __device__ __forceinline__ void face(S* __restrict__ dst, const KParams& p, int 
             }
         }
     });
-    if (!CLOSED && (p.periodic & (1 << AXIS))) face_call<DIM, S, VEC, C, MODE, RAW, AXIS, SIDE, false>(dst, p, x0, y, z, post, salt);
-    else face_call<DIM, S, VEC, C, MODE, RAW, AXIS, SIDE, true>(dst, p, x0, y, z, post, salt);
+    if (!CLOSED && (p.periodic & (1 << AXIS))) face_call<DIM, S, VEC, C, MODE, RAW, AXIS, SIDE, false, true>(dst, p, x0, y, z, post, salt);
+    else face_call<DIM, S, VEC, C, MODE, RAW, AXIS, SIDE, true, wall_named<S, CLOSED>>(dst, p, x0, y, z, post, salt);
 }
 
 // All faces in one call, for FP64: bound by the FP64 pipe, its warps gain little
@@ -1211,7 +1223,7 @@ __device__ __forceinline__ C pick(const C (&v)[VEC], int k) {
 
 // The populations with e_x = SIDE of node k of a thread's VEC nodes, for a node
 // on the x face SIDE with x not periodic: they leave the cell through that face.
-template <class LS, bool THERMAL, int SIDE, class S, int VEC, class C, bool KS, int MODE = PULL>
+template <class LS, bool THERMAL, int SIDE, class S, int VEC, class C, bool KS, int MODE, bool NAMED>
 __device__ __forceinline__ void x_face(S* __restrict__ base, const KParams& p, int x, int y, int z, int k,
                                        const C (&v)[LS::Q][VEC], uint32_t salt) {
     const C scale = ScaleOf<C>::s(p);
@@ -1220,7 +1232,7 @@ __device__ __forceinline__ void x_face(S* __restrict__ base, const KParams& p, i
         constexpr int i = decltype(ii)::value;
         if constexpr (LS::e(i, 0) == SIDE) {
             const C val = pick<VEC>(v[i], k);
-            ghost_write<LS, THERMAL, i, S, C, MODE, KS && !Storage<S>::offset>(base, p, x, y, z, KS && Storage<S>::offset ? val * un : val, scale, salt);
+            ghost_write<LS, THERMAL, i, S, C, MODE, KS && !Storage<S>::offset, NAMED>(base, p, x, y, z, KS && Storage<S>::offset ? val * un : val, scale, salt);
         }
     });
 }
@@ -1279,15 +1291,16 @@ __device__ __forceinline__ void wall_writes(S* __restrict__ dst, const KParams& 
             return;
         }
     }
+    constexpr bool NAMED = wall_named<S, CLOSED>;
     S* __restrict__ gdst = dst + (long long)QF * L.plane;
     if (xlo) {
-        x_face<LF, false, -1, S, VEC, C, KS, MODE>(dst, p, 0, y, z, 0, f, salt);
-        x_face<LG, true, -1, S, VEC, C, KS, MODE>(gdst, p, 0, y, z, 0, g, salt);
+        x_face<LF, false, -1, S, VEC, C, KS, MODE, NAMED>(dst, p, 0, y, z, 0, f, salt);
+        x_face<LG, true, -1, S, VEC, C, KS, MODE, NAMED>(gdst, p, 0, y, z, 0, g, salt);
     }
     if (xhi) {
         const int k = L.nx - 1 - x0;
-        x_face<LF, false, 1, S, VEC, C, KS, MODE>(dst, p, L.nx - 1, y, z, k, f, salt);
-        x_face<LG, true, 1, S, VEC, C, KS, MODE>(gdst, p, L.nx - 1, y, z, k, g, salt);
+        x_face<LF, false, 1, S, VEC, C, KS, MODE, NAMED>(dst, p, L.nx - 1, y, z, k, f, salt);
+        x_face<LG, true, 1, S, VEC, C, KS, MODE, NAMED>(gdst, p, L.nx - 1, y, z, k, g, salt);
     }
 }
 
