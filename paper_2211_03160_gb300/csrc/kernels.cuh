@@ -958,7 +958,8 @@ template <bool HI, class PT>
 __device__ __forceinline__ float anti_bounce_back(float val, const PT& p) { return __fmaf_rn(p.omegaf, HI ? p.Tcf : p.Thf, -val); }
 
 // Whether a kernel names the walls: all but the 16-bit march, which at its 128
-// registers takes 1 % longer with them named (8193^2 FP16 1692 -> 1711 us a pass).
+// registers takes 1 % longer with them named (8193^2 FP16 1692 -> 1711 us a pass),
+// and FP64 in 3D (any_face).
 template <class S, bool CLOSED>
 constexpr bool wall_named = !(CLOSED && sizeof(S) == 2);
 
@@ -1125,10 +1126,12 @@ __device__ __forceinline__ void face_writes(S* __restrict__ dst, const KParams& 
         }
     });
 }
+// (FP64; in 3D the walls are told from the node's place: named, 193^3 took 2942 us a
+// step instead of 2907)
 template <int DIM, class S, class C, int MODE, bool RAW, int AXIS, int SIDE, bool CLOSED, class Val>
 __device__ __forceinline__ void any_face(S* __restrict__ dst, const KParams& p, int x, int y, int z, Val val, uint32_t salt) {
     if (!CLOSED && (p.periodic & (1 << AXIS))) face_writes<DIM, S, C, MODE, RAW, AXIS, SIDE, false, true>(dst, p, x, y, z, val, salt);
-    else face_writes<DIM, S, C, MODE, RAW, AXIS, SIDE, true, true>(dst, p, x, y, z, val, salt);
+    else face_writes<DIM, S, C, MODE, RAW, AXIS, SIDE, true, DIM == 2>(dst, p, x, y, z, val, salt);
 }
 
 // The rules of a thread's nodes at the edge of the cell, one face after the other

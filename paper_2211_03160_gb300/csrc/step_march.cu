@@ -25,7 +25,7 @@
 //
 // What bounds it now: instruction issue and latency at twelve warps an SM (167
 // registers a thread; at 4097^2 issue slots 59 % used, 173 instructions per node and
-// step, 211 in FP16); HBM moves 37 of the 112 bytes per update.  GLUPS on GB300
+// step, 210 in FP16); HBM moves 37 of the 112 bytes per update.  GLUPS on GB300
 // by steps per pass (blocks of four warps per SM) at 8193^2: 2 (3) 111, 3 (3)
 // 132, 3 (4, spilling) 80, 4 (2) 124; 2 (5, at 96 registers) 75.  us per step,
 // one-step kernel -> this: 513^2 7.4 -> 5.7, 1025^2 22.2 -> 12.4, 2049^2 75.5 ->
