@@ -434,8 +434,8 @@ static void build_tables(tlbm_batch_t b, std::vector<KParams>& kps, std::vector<
 // The marching form: 2D FP32 and 16-bit cells with walls all around and two-relaxation-time
 // rates, in a batch whose launches the caller has not chosen.  us per step of
 // 64 FP32 cells of 129^2 to 1025^2: flattened launch untuned 606, staged (the tuned
-// form) 473, marching 274; of 64 cells of 1025^2 1445, 1152 and 618, 16 of 513^2
-// 135, 85 and 58, 48 of 65^2 37, 16 and 9.2; FP16 461, 336 and 296, 1065, 798 and 669,
+// form) 473, marching 254; of 64 cells of 1025^2 1445, 1152 and 618, 16 of 513^2
+// 135, 85 and 58, 48 of 65^2 37, 16 and 9.2; FP16 461, 336 and 292, 1065, 798 and 669,
 // 114, 62 and 59, 42, 16 and 10.3.
 static void build_marches(tlbm_batch_t b) {
     b->marches.clear();
